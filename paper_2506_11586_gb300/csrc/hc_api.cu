@@ -301,6 +301,13 @@ hc_status copy_lane(CopyLane **out)
     return HC_OK;
 }
 
+// c if q = 2^50 - c with 0 < c < 2^22, else 0
+uint64_t special_c50(uint64_t q)
+{
+    const uint64_t c = (1ull << 50) - q;
+    return c < (1ull << 22) ? c : 0;
+}
+
 struct ScratchGuard {
     void *p = nullptr;
     cudaStream_t s;
@@ -629,10 +636,13 @@ hc_status hc_ctx_create_ex(uint32_t N, const uint64_t *moduli, uint32_t L, uint6
     // per limb: forward, inverse, then the rearranged tables (inverse first round,
     // forward last round) for LOGC = 3, 4, 5
     constexpr uint32_t kTablesPerLimb = 8;
-    std::vector<ulonglong2> tw((size_t)kTablesPerLimb * L * N);
+    std::vector<ulonglong2> tables((size_t)kTablesPerLimb * L * N);
     std::vector<LimbConst> lcs(L);
     std::vector<uint64_t> delta(L);
     delta_residues(moduli, L, t, delta.data());
+    c->fold = true;
+    for (uint32_t i = 0; i < L; ++i)
+        if (!special_c50(moduli[i])) c->fold = false;
     for (uint32_t i = 0; i < L; ++i) {
         const uint64_t q = moduli[i];
         const uint64_t psi = min_primitive_2n_root(q, N);
@@ -643,23 +653,26 @@ hc_status hc_ctx_create_ex(uint32_t N, const uint64_t *moduli, uint32_t L, uint6
         const uint64_t psi_inv = powmod_u64(psi, q - 2, q);
         c->q[i] = q;
         c->psi[i] = psi;
-        ulonglong2 *f = tw.data() + (size_t)(kTablesPerLimb * i) * N;
-        ulonglong2 *b = tw.data() + (size_t)(kTablesPerLimb * i + 1) * N;
+        // a twiddle as the kernels read it (TwArith): the folded form, or the constant and
+        // its Shoup companion
+        auto tw = [&](uint64_t w) {
+            return c->fold ? fold_twiddle(w, q) : make_ulonglong2(w, shoup_companion(w, q));
+        };
+        ulonglong2 *f = tables.data() + (size_t)(kTablesPerLimb * i) * N;
+        ulonglong2 *b = tables.data() + (size_t)(kTablesPerLimb * i + 1) * N;
         // powers psi^j and psi^-j in natural order, then scattered to bit-reversed slots
         uint64_t pf = 1, pb = 1;
         for (uint32_t j = 0; j < N; ++j) {
             const uint32_t k = bit_reverse(j, c->logN);
-            f[k].x = pf;
-            f[k].y = shoup_companion(pf, q);
-            b[k].x = pb;
-            b[k].y = shoup_companion(pb, q);
+            f[k] = tw(pf);
+            b[k] = tw(pb);
             pf = mulmod_u64(pf, psi, q);
             pb = mulmod_u64(pb, psi_inv, q);
         }
         // first inverse register round with 2^lc residues per thread (thread t, stage s,
         // group g uses b[(N >> (s+1)) + t*2^(lc-1-s) + g]), rearranged for coalesced reads
         for (uint32_t lcg = 3; lcg <= 5 && lcg < c->logN; ++lcg) {
-            ulonglong2 *r0 = tw.data() + (size_t)(kTablesPerLimb * i + 2 + (lcg - 3)) * N;
+            ulonglong2 *r0 = tables.data() + (size_t)(kTablesPerLimb * i + 2 + (lcg - 3)) * N;
             const uint32_t T = N >> lcg;
             for (uint32_t st = 0; st < lcg; ++st) {
                 const uint32_t ngrp = 1u << (lcg - 1 - st), off = N - (N >> st);
@@ -669,7 +682,7 @@ hc_status hc_ctx_create_ex(uint32_t N, const uint64_t *moduli, uint32_t L, uint6
             // last forward register round (stages S0 .. log2 N - 1, SUBS sub-transforms per
             // thread): thread t, sub-transform v, stage S0 + sig, group lam uses
             // f[2^(S0+sig) + (t*SUBS + v)*2^sig + lam]
-            ulonglong2 *rl = tw.data() + (size_t)(kTablesPerLimb * i + 5 + (lcg - 3)) * N;
+            ulonglong2 *rl = tables.data() + (size_t)(kTablesPerLimb * i + 5 + (lcg - 3)) * N;
             const uint32_t nr = (c->logN + lcg - 1) / lcg, S0 = (nr - 1) * lcg, K = c->logN - S0;
             const uint32_t subs = 1u << (lcg - K);
             for (uint32_t sig = 0; sig < K; ++sig) {
@@ -686,17 +699,18 @@ hc_status hc_ctx_create_ex(uint32_t N, const uint64_t *moduli, uint32_t L, uint6
         lc.r64 = (uint64_t)(((unsigned __int128)1 << 64) % q);
         lc.r64_s = shoup_companion(lc.r64, q);
         lc.one_s = shoup_companion(1, q);
-        lc.ninv = powmod_u64(N, q - 2, q);
-        lc.ninv_s = shoup_companion(lc.ninv, q);
-        lc.ninvw = mulmod_u64(lc.ninv, b[1].x, q);
-        lc.ninvw_s = shoup_companion(lc.ninvw, q);
+        const uint64_t ninv = powmod_u64(N, q - 2, q);
+        const ulonglong2 tn = tw(ninv), tnw = tw(mulmod_u64(ninv, powmod_u64(psi_inv, N / 2, q), q));
+        lc.ninv = tn.x;
+        lc.ninv_s = tn.y;
+        lc.ninvw = tnw.x;
+        lc.ninvw_s = tnw.y;
         lc.delta = delta[i];
         lc.delta_s = shoup_companion(delta[i], q);
-        const uint64_t c50 = (1ull << 50) - q;
-        lc.special_c = c50 > 0 && c50 < (1ull << 22) ? c50 : 0;
+        lc.special_c = special_c50(q);
     }
 
-    c->table_bytes = tw.size() * sizeof(ulonglong2);
+    c->table_bytes = tables.size() * sizeof(ulonglong2);
     c->d_tables = dev_alloc_persistent(c->table_bytes);
     c->d_limbs = (LimbConst *)dev_alloc_persistent(sizeof(LimbConst) * L);
     c->d_flag = (int *)dev_alloc_persistent(sizeof(int) * 4);
@@ -712,7 +726,7 @@ hc_status hc_ctx_create_ex(uint32_t N, const uint64_t *moduli, uint32_t L, uint6
         lcs[i].tw_i = (const ulonglong2 *)c->d_tables + (size_t)(kTablesPerLimb * i + 1) * N;
         lcs[i].tw_r = (const ulonglong2 *)c->d_tables + (size_t)(kTablesPerLimb * i + 2) * N;
     }
-    cudaError_t e = cudaMemcpy(c->d_tables, tw.data(), c->table_bytes, cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMemcpy(c->d_tables, tables.data(), c->table_bytes, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(c->d_limbs, lcs.data(), sizeof(LimbConst) * L, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(c->d_flag, 0, sizeof(int) * 4);
     if (e != cudaSuccess) {

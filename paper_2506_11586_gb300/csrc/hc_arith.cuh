@@ -101,6 +101,114 @@ __device__ __forceinline__ uint64_t canon4(uint64_t x, uint64_t q)
     return csub(csub(x, 2 * q), q);
 }
 
+// ---- twiddle products ---------------------------------------------------------------
+// TwArith<false>: any q, unsigned lazy values, Shoup products (twiddle = {w, w'}).
+//
+// TwArith<true>: q = 2^50 - c with 0 < c < 2^22 (LimbConst::special_c), signed lazy
+// values, folded products.  The constant w < q is kept as two residues, w and
+// v = w * 2^32 mod q, each cut at 2^20 (fold_twiddle).  With y = yl + 2^32 yh (yl
+// unsigned, yh signed),
+//     y*w = yl*w + yh*v = lo + 2^20 mid    (mod q),
+//     lo = yl*wl + yh*vl,  mid = yl*wh + yh*vh,
+// and, because 2^52 = 4c (mod q), mid's high word folds down as it stands:
+//     t = lo + 2^20 lo32(mid) + 4c hi32(mid).
+// For every signed 64-bit y: -2^51 <= lo < 2^52 + 2^51 and -2^61 <= mid < 2^62 + 2^61,
+// so -10 * 2^50 <= t < 34 * 2^50, i.e. |t| <= kFoldMax q.  Six wide multiply-adds and
+// no other instruction: the cut at 2^20 puts the fold at 2^52 on a word boundary of
+// mid, so nothing is shifted, masked or carried, and signed values need no multiple of
+// q added to a difference (two more instructions on the same pipes per butterfly).
+// Bound by the multiply pipe (24 of its cycles per warp).  Measured on GB300, a
+// radix-32 round in registers at 16 warps per SM: 28.6 cycles per warp butterfly and SM
+// sub-partition, 33.5 with unsigned values, 41.6 with Shoup products (5 wide and 4
+// narrow multiply-adds, 5 additions and moves).
+constexpr uint64_t kFoldMax = 35;
+
+template <bool SP>
+struct TwArith;
+
+template <>
+struct TwArith<false> {
+    static constexpr bool kFolded = false;
+    uint64_t q, nq;
+    uint32_t ones;  // floor(2^64 / q)
+    __device__ __forceinline__ TwArith(uint64_t q_, uint64_t, uint64_t one_s)
+        : q(q_), nq(0ull - q_), ones((uint32_t)one_s)
+    {
+    }
+    // y*w mod q, < 4q
+    __device__ __forceinline__ uint64_t mul(uint64_t y, ulonglong2 w) const { return shoup_lazy(y, w.x, w.y, nq); }
+    __device__ __forceinline__ uint64_t mul_canon(uint64_t y, ulonglong2 w) const { return canon4(mul(y, w), q); }
+    // x - y for y <= b (b = 0: y is a product)
+    __device__ __forceinline__ uint64_t sub(uint64_t x, uint64_t y, uint64_t b = 0) const
+    {
+        return x - y + (b ? b : 4 * q);
+    }
+    // canonical residue of any x < 2^64
+    __device__ __forceinline__ uint64_t canon(uint64_t x) const { return canon3(reduce_lazy(x, ones, nq), q); }
+};
+
+template <>
+struct TwArith<true> {
+    static constexpr bool kFolded = true;
+    uint64_t q;
+    uint32_t c, c4, p20;
+    __device__ __forceinline__ TwArith(uint64_t q_, uint64_t c_, uint64_t)
+        : q(q_), c((uint32_t)c_), c4(4 * (uint32_t)c_)
+    {
+        // 2^20 as a register the compiler does not see through: a visible power of two
+        // becomes shifts and carries, five instructions for one
+        asm("mov.u32 %0, 0x100000;" : "=r"(p20));
+    }
+    // y*w + add mod q for any signed y, |result - add| <= kFoldMax q.  Each lo / hi pair
+    // is one wide multiply-add, written by halves because the compiler gives
+    // mad.wide.u32's result a fresh register pair and moves it back (2 moves a product).
+    __device__ __forceinline__ uint64_t mul(uint64_t y, ulonglong2 w, uint64_t add = 0) const
+    {
+        uint64_t t;
+        asm("{\n\t"
+            ".reg .u32 yl, yh, wl, wh, vl, vh, ml, mh, ll, lh;\n\t"
+            "mov.b64 {yl, yh}, %1;\n\t"
+            "mov.b64 {wl, wh}, %2;\n\t"
+            "mov.b64 {vl, vh}, %3;\n\t"
+            "mov.b64 {ll, lh}, %6;\n\t"
+            "mul.lo.u32 ml, yl, wh;\n\t"        // mid
+            "mul.hi.u32 mh, yl, wh;\n\t"
+            "mad.lo.cc.s32 ml, yh, vh, ml;\n\t"
+            "madc.hi.s32 mh, yh, vh, mh;\n\t"
+            "mad.lo.cc.u32 ll, yl, wl, ll;\n\t" // lo
+            "madc.hi.u32 lh, yl, wl, lh;\n\t"
+            "mad.lo.cc.s32 ll, yh, vl, ll;\n\t"
+            "madc.hi.s32 lh, yh, vl, lh;\n\t"
+            "mad.lo.cc.u32 ll, ml, %5, ll;\n\t"
+            "madc.hi.u32 lh, ml, %5, lh;\n\t"
+            "mad.lo.cc.s32 ll, mh, %4, ll;\n\t"
+            "madc.hi.s32 lh, mh, %4, lh;\n\t"
+            "mov.b64 %0, {ll, lh};\n\t"
+            "}"
+            : "=l"(t)
+            : "l"(y), "l"(w.x), "l"(w.y), "r"(c4), "r"(p20), "l"(add));
+        return t;
+    }
+    __device__ __forceinline__ uint64_t mul_canon(uint64_t y, ulonglong2 w) const
+    {
+        return canon_pos(mul(y, w, 16 * q));  // -10 * 2^50 + 16 q > 0
+    }
+    __device__ __forceinline__ uint64_t sub(uint64_t x, uint64_t y, uint64_t = 0) const { return x - y; }
+    // a value congruent to x, > -2^36 and < 2^52 + 2^36 (< 5 q), for any signed x
+    __device__ __forceinline__ uint64_t fold(uint64_t x) const
+    {
+        const int64_t h = (int32_t)(x >> 32) >> 20;  // x >> 52
+        return (x & ((1ull << 52) - 1)) + (uint64_t)(h * (int64_t)c4);
+    }
+    // canonical residue of x >= 0: the fold at 2^50 leaves less than 2^50 + 2^36 < 2 q
+    __device__ __forceinline__ uint64_t canon_pos(uint64_t x) const
+    {
+        return csub((x & ((1ull << 50) - 1)) + (uint64_t)(uint32_t)(x >> 50) * c, q);
+    }
+    // canonical residue of any x, |x| <= 2047 q
+    __device__ __forceinline__ uint64_t canon(uint64_t x) const { return canon_pos(x + 2048 * q); }
+};
+
 // Multiply-accumulate of products x*w with x < 2^56, w < 2^50, as three
 // partial sums of 32x32 products:
 //   V = s0 + 2^64 c0 + 2^32 s1 + 2^64 s2,
@@ -210,6 +318,24 @@ __device__ __forceinline__ uint64_t mac_reduce_special(const MacAcc &a, uint64_t
     uint64_t lo, hi;
     mac_value(a, lo, hi);
     return reduce128_special(lo, hi, q, c);
+}
+
+// canonical x*w mod q of a lazy forward-transform value x and a residue w < q.  The
+// folded form's x (|x| < 2^60) is first brought into [0, 2^53), so that x*w < 2^104.
+__device__ __forceinline__ uint64_t mul_slot(const TwArith<false> &ar, uint64_t x, uint64_t w, uint64_t r64,
+                                             uint64_t r64_s)
+{
+    MacAcc a;
+    mac_zero(a);
+    mac_add(a, x, w);
+    return mac_reduce(a, ar.q, ar.nq, r64, r64_s, ar.ones);
+}
+__device__ __forceinline__ uint64_t mul_slot(const TwArith<true> &ar, uint64_t x, uint64_t w, uint64_t, uint64_t)
+{
+    MacAcc a;
+    mac_zero(a);
+    mac_add(a, ar.fold(x + 2048 * ar.q), w);
+    return mac_reduce_special(a, ar.q, ar.c);
 }
 
 }  // namespace hc

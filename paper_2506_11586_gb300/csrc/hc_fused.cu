@@ -74,7 +74,7 @@ __device__ __forceinline__ bool wait_for(const uint32_t *ctr, uint32_t target, i
     return *s_ok != 0;
 }
 
-template <class Cfg, int NS>
+template <class Cfg, int NS, bool SP>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
 k_conv_fused(const __grid_constant__ FusedLayersT<NS> P, uint32_t *cnt, int *err)
 {
@@ -118,7 +118,7 @@ k_conv_fused(const __grid_constant__ FusedLayersT<NS> P, uint32_t *cnt, int *err
             const uint32_t local = t - ly.t_fwd;
             const uint32_t limb = local / (2 * ly.I), poly = local % (2 * ly.I);
             const size_t off = ((size_t)poly * L + limb) * N;
-            fwd_task<Cfg>(dsm, ly.in + off, const_cast<uint64_t *>(sg.X) + off, 0, sg.limbs[limb], tid);
+            fwd_task<Cfg, SP>(dsm, ly.in + off, const_cast<uint64_t *>(sg.X) + off, 0, sg.limbs[limb], tid);
             signal_done(cnt + ly.c_fwd + limb);
         } else if (phase == 1) {  // one MAC chunk
             const uint32_t local = t - ly.t_mac;
@@ -140,16 +140,16 @@ k_conv_fused(const __grid_constant__ FusedLayersT<NS> P, uint32_t *cnt, int *err
                 break;
             }
             uint64_t *y = sg.Y + ((size_t)poly * L + limb) * N;
-            inv_task<Cfg, true>(dsm, y, y, 0, sg.limbs[limb], tid);
+            inv_task<Cfg, SP, true>(dsm, y, y, 0, sg.limbs[limb], tid);
         }
     }
 }
 
-template <int LOGN, int V, int NS>
+template <int LOGN, int V, int NS, bool SP>
 hc_status run_fused(FusedLayersT<NS> &P, size_t smem, uint32_t ctr_words, uint32_t *ctr, int *err, cudaStream_t s)
 {
     using Cfg = typename FusedShape<LOGN, V>::Cfg;
-    auto kern = k_conv_fused<Cfg, NS>;
+    auto kern = k_conv_fused<Cfg, NS, SP>;
     static std::atomic<uint32_t> attr_done{0};
     int dev = 0;
     cudaGetDevice(&dev);
@@ -190,7 +190,7 @@ hc_status run_fused(FusedLayersT<NS> &P, size_t smem, uint32_t ctr_words, uint32
     return e == cudaSuccess ? HC_OK : cuda_error(e, "launch k_conv_fused");
 }
 
-template <int LOGN, int V, int NS>
+template <int LOGN, int V, int NS, bool SP>
 hc_status fused_for_ns(const ConvJob *jobs, size_t n, uint32_t *ctr, cudaStream_t s)
 {
     FusedLayersT<NS> P{};
@@ -198,7 +198,7 @@ hc_status fused_for_ns(const ConvJob *jobs, size_t n, uint32_t *ctr, cudaStream_
     uint32_t words = 1;  // [0]: the task counter
     const ConvJob *idx[NS];
     for (size_t i = 0; i < n; ++i) {
-        if (jobs[i].ctx->logN != (uint32_t)LOGN || !jobs[i].blocked) continue;
+        if (jobs[i].ctx->logN != (uint32_t)LOGN || !jobs[i].blocked || jobs[i].ctx->fold != SP) continue;
         if (P.n == (uint32_t)NS) return set_error(HC_ERR_UNSUPPORTED, "too many layers for one fused launch");
         idx[P.n] = &jobs[i];
         FusedLayer &ly = P.s[P.n++];
@@ -230,23 +230,27 @@ hc_status fused_for_ns(const ConvJob *jobs, size_t n, uint32_t *ctr, cudaStream_
     }
     if (t > 0xffffffffu) return set_error(HC_ERR_INVALID_ARG, "fused launch too large");
     P.total = (uint32_t)t;
-    return run_fused<LOGN, V, NS>(P, smem, words, ctr, timeout_flag(idx[0]->ctx), s);
+    return run_fused<LOGN, V, NS, SP>(P, smem, words, ctr, timeout_flag(idx[0]->ctx), s);
 }
 
-template <int LOGN>
+template <int LOGN, bool SP>
 hc_status fused_for(const ConvJob *jobs, size_t n, uint32_t *ctr, cudaStream_t s)
 {
     size_t count = 0;
-    const ConvJob *first = nullptr;
     for (size_t i = 0; i < n; ++i)
-        if (jobs[i].ctx->logN == (uint32_t)LOGN && jobs[i].blocked) {
-            if (!first) first = &jobs[i];
-            ++count;
-        }
-    if (!first) return HC_OK;
+        if (jobs[i].ctx->logN == (uint32_t)LOGN && jobs[i].blocked && jobs[i].ctx->fold == SP) ++count;
+    if (!count) return HC_OK;
     // one layer: a one-entry table keeps the kernel's parameter block small
-    return count == 1 ? fused_for_ns<LOGN, 1, 1>(jobs, n, ctr, s)
-                      : fused_for_ns<LOGN, 1, kFusedMaxLayers>(jobs, n, ctr, s);
+    return count == 1 ? fused_for_ns<LOGN, 1, 1, SP>(jobs, n, ctr, s)
+                      : fused_for_ns<LOGN, 1, kFusedMaxLayers, SP>(jobs, n, ctr, s);
+}
+
+// the folded contexts' layers, then the others', in stream order on the same counters
+template <int LOGN>
+hc_status fused_both(const ConvJob *jobs, size_t n, uint32_t *ctr, cudaStream_t s)
+{
+    const hc_status st = fused_for<LOGN, true>(jobs, n, ctr, s);
+    return st == HC_OK ? fused_for<LOGN, false>(jobs, n, ctr, s) : st;
 }
 
 }  // namespace
@@ -266,9 +270,9 @@ size_t fused_counter_words(const ConvJob *jobs, size_t n, uint32_t logN)
 hc_status launch_conv_fused(const ConvJob *jobs, size_t n, uint32_t logN, uint32_t *ctr, cudaStream_t s)
 {
     switch (logN) {
-    case 12: return fused_for<12>(jobs, n, ctr, s);
-    case 13: return fused_for<13>(jobs, n, ctr, s);
-    case 14: return fused_for<14>(jobs, n, ctr, s);
+    case 12: return fused_both<12>(jobs, n, ctr, s);
+    case 13: return fused_both<13>(jobs, n, ctr, s);
+    case 14: return fused_both<14>(jobs, n, ctr, s);
     default: return set_error(HC_ERR_UNSUPPORTED, "unsupported degree");
     }
 }

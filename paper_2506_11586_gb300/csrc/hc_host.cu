@@ -166,6 +166,12 @@ uint64_t min_primitive_2n_root(uint64_t q, uint32_t N)
 
 uint64_t shoup_companion(uint64_t w, uint64_t q) { return (uint64_t)(((u128)w << 64) / q); }
 
+ulonglong2 fold_twiddle(uint64_t w, uint64_t q)
+{
+    auto cut = [](uint64_t a) { return (a & 0xfffff) | (a >> 20) << 32; };
+    return make_ulonglong2(cut(w), cut((uint64_t)(((u128)w << 32) % q)));
+}
+
 void delta_residues(const uint64_t *moduli, uint32_t L, uint64_t t, uint64_t *out)
 {
     // Q = prod q_i as little-endian 64-bit words (L <= 8 limbs of < 50 bits: < 7 words)

@@ -21,7 +21,9 @@ constexpr uint32_t kMagicGaloisKey = 0x4843474Bu;  // 'HCGK'
 constexpr uint32_t kMagicDead = 0xDEADDEADu;
 
 // Per-limb constants and twiddle tables, device-resident, read through the
-// read-only path.  Every Shoup companion w' = floor(w * 2^64 / q).
+// read-only path.  Every Shoup companion w' = floor(w * 2^64 / q).  Twiddles
+// (tw_f, tw_i, tw_r, ninv, ninvw) are {w, w'} pairs, or in folded form
+// (fold_twiddle) in contexts with hc_ctx::fold.
 struct LimbConst {
     uint64_t q;
     uint64_t r64, r64_s;      // 2^64 mod q, companion
@@ -92,6 +94,7 @@ struct hc_ctx {
     void *d_tables;           // twiddle storage (owned)
     size_t table_bytes;
     int *d_flag;              // device error flag for checked mode (owned)
+    bool fold;                // every limb is 2^50 - c, c < 2^22: folded twiddles, SP kernels
     uint8_t variant[hc::KK_COUNT];  // launch-shape variant per kernel family
 };
 
@@ -229,6 +232,9 @@ uint64_t min_primitive_2n_root(uint64_t q, uint32_t N);
 // floor(prod(moduli) / t) mod q_i for every limb (exact multi-precision)
 void delta_residues(const uint64_t *moduli, uint32_t L, uint64_t t, uint64_t *out);
 uint64_t shoup_companion(uint64_t w, uint64_t q);
+// folded form of a twiddle w < q: w and v = w * 2^32 mod q, each as {low 20 bits, rest}
+// in the low and high 32 bits of one word
+ulonglong2 fold_twiddle(uint64_t w, uint64_t q);
 uint32_t bit_reverse(uint32_t k, uint32_t logn);
 
 // ---- kernel launchers (hc_kernels.cu) -------------------------------------------
@@ -245,6 +251,7 @@ struct NttSeg {
     const LimbConst *limbs;
     uint32_t L, n_groups, cta_begin;
     uint32_t Lc = 0, limb0 = 0;  // limbs [limb0, limb0 + Lc) only (Lc = 0: all L); L stays the layout stride
+    uint32_t fold = 0;           // the context's twiddle form; one form per launch (launch_ntt_ct_segs)
 };
 __host__ __device__ inline uint32_t seg_limbs(const NttSeg &s) { return s.Lc ? s.Lc : s.L; }
 constexpr int kMaxSegs = 48;
@@ -353,6 +360,7 @@ struct MixItem {
     const LimbConst *limbs;
     uint32_t L, logN;
 };
+// (items of one launch share the twiddle form)
 // work unit code: item << 4 | limb << 1 | component
 constexpr uint32_t mix_unit(uint32_t item, uint32_t limb, uint32_t comp) { return item << 4 | limb << 1 | comp; }
 // components per unit at ring degree 2^logN (2: both in one unit, 1: one unit per component)
@@ -360,7 +368,7 @@ constexpr uint32_t mix_comps_per_unit(uint32_t logN) { return logN >= 14 ? 1 : 2
 // persistent launch over n_units units (sorted by cost, most expensive first);
 // *next must be 0 when the launch starts
 hc_status launch_product_mixed(const MixItem *items, const uint32_t *units, uint32_t n_units, uint32_t *next,
-                               cudaStream_t s);
+                               bool fold, cudaStream_t s);
 
 // transform kinds that take a segment table (pseudo-kinds, variant of FWDCT / INVCT),
 // and the inverse transform with the server step's output epilogue (variant of INV)
@@ -379,7 +387,7 @@ struct LaunchArgs {
     bool accumulate;
     const ExtractArgs *ex;
 };
-template <int LOGN>
+template <int LOGN, bool SP>
 hc_status launch_n(const hc_ctx *ctx, int kind, int variant, const LaunchArgs &a, cudaStream_t s);
 
 // default launch variant of a kernel family at ring degree 2^logn
@@ -393,7 +401,8 @@ hc_status launch_ntt_inv(const hc_ctx *ctx, const uint64_t *in, uint64_t *out, s
 // inverse NTT of n_ct ciphertexts [n][2][L][N] (canonical NTT domain in, coefficients out)
 hc_status launch_ntt_inv_ct(const hc_ctx *ctx, const uint64_t *in, uint64_t *out, size_t n_ct, cudaStream_t s);
 // multi-segment forward / inverse transforms of ciphertexts (all segments share
-// ctx's N and launch variant; n_groups counts ciphertexts)
+// ctx's N and launch variant; n_groups counts ciphertexts); one launch per twiddle
+// form that occurs
 hc_status launch_ntt_ct_segs(const hc_ctx *ctx, const NttSegs &segs, bool inverse, cudaStream_t s);
 // conv MAC blocked over coefficient chunks: Y[m*B+b] = sum_g W[m*G+g] . X[g*B+b] (NTT domain)
 hc_status launch_mac_conv(const hc_ctx *ctx, const uint64_t *x_ntt, const uint64_t *w_ntt, uint64_t *y,

@@ -1,6 +1,6 @@
 // hc_kernels.cuh -- sm_103a kernels of the HE-convolution hot path, their
-// launch shapes and launchers.  Instantiated once per ring degree in
-// hc_kernels_n12.cu / _n13.cu / _n14.cu (compiled in parallel).
+// launch shapes and launchers.  Instantiated once per ring degree and twiddle form
+// (SP, see hc_ntt.cuh) in hc_kernels_n12.cu / _n12f.cu ... _n14f.cu (compiled in parallel).
 //
 //   k_ntt_fwd   forward NTT of NP polynomials per CTA (in place or out of place)
 //   k_ntt_inv   inverse NTT, NP polynomials per CTA
@@ -96,27 +96,24 @@ __device__ __forceinline__ void load_round0(uint64_t (&x)[Cfg::NP][Cfg::C], cons
 // Forward NTT of NP polynomials (src + p*pstride, p < NP) into dst (same
 // strides), canonical output, stored through shared memory as coalesced
 // 16-byte pairs.  One CTA task.
-template <class Cfg>
+template <class Cfg, bool SP>
 __device__ __forceinline__ void fwd_task(uint64_t *sm, const uint64_t *src, uint64_t *dst, size_t pstride,
                                          const LimbConst &lc, int tid)
 {
     constexpr int NP = Cfg::NP, C = Cfg::C, T = Cfg::T, N = Cfg::N;
-    const uint64_t q = lc.q;
     uint64_t x[NP][C];
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
 #pragma unroll
         for (int r = 0; r < C; ++r) x[p][r] = __ldg(src + p * pstride + tid + r * T);
     }
-    fwd_transform<Cfg>(x, sm, lc.tw_f, lc.tw_r, q, tid);
-
-    const uint32_t ones = (uint32_t)lc.one_s;
-    const uint64_t nq = 0ull - q;
+    const TwArith<SP> ar = tw_arith<SP>(lc);
+    fwd_transform<Cfg>(x, sm, lc, ar, tid);
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < C; ++r) {
 #pragma unroll
-        for (int p = 0; p < NP; ++p) sm[p * N + spos<Cfg>(tid * C + r)] = canon3(reduce_lazy(x[p][r], ones, nq), q);
+        for (int p = 0; p < NP; ++p) sm[p * N + spos<Cfg>(tid * C + r)] = ar.canon(x[p][r]);
     }
     __syncthreads();
 #pragma unroll
@@ -136,7 +133,7 @@ __device__ __forceinline__ void fwd_task(uint64_t *sm, const uint64_t *src, uint
 // Inverse NTT of NP polynomials (src + p*pstride) into dst (may equal src).
 // COHERENT loads bypass the non-coherent read-only path, for inputs written
 // earlier by other CTAs of the same launch.  One CTA task.
-template <class Cfg, bool COHERENT = false>
+template <class Cfg, bool SP, bool COHERENT = false>
 __device__ __forceinline__ void inv_core(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_t *sm, const uint64_t *src,
                                          size_t pstride, const LimbConst &lc, int tid)
 {
@@ -155,16 +152,16 @@ __device__ __forceinline__ void inv_core(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_
         }
     }
     load_round0<Cfg>(x, sm, tid);
-    inv_transform<Cfg>(x, sm, lc, lc.tw_i, tid);
+    inv_transform<Cfg>(x, sm, lc, tw_arith<SP>(lc), tid);
 }
 
-template <class Cfg, bool COHERENT = false>
+template <class Cfg, bool SP, bool COHERENT = false>
 __device__ __forceinline__ void inv_task(uint64_t *sm, const uint64_t *src, uint64_t *dst, size_t pstride,
                                          const LimbConst &lc, int tid)
 {
     constexpr int NP = Cfg::NP, C = Cfg::C;
     uint64_t x[NP][C];
-    inv_core<Cfg, COHERENT>(x, sm, src, pstride, lc, tid);
+    inv_core<Cfg, SP, COHERENT>(x, sm, src, pstride, lc, tid);
     // the transform's results are read by no later kernel of the layer: streaming
     // stores (evict first), so that L2 keeps what the next kernels read
 #pragma unroll
@@ -175,7 +172,7 @@ __device__ __forceinline__ void inv_task(uint64_t *sm, const uint64_t *src, uint
     }
 }
 
-template <class Cfg, int NS>
+template <class Cfg, int NS, bool SP>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
 k_ntt_fwd(const __grid_constant__ NttSegsT<NS> segs)
 {
@@ -184,10 +181,10 @@ k_ntt_fwd(const __grid_constant__ NttSegsT<NS> segs)
     const uint32_t local = blockIdx.x - sg.cta_begin;
     const uint32_t limb = sg.limb0 + local / sg.n_groups, grp = local % sg.n_groups;
     const size_t off = ((size_t)grp * Cfg::NP * sg.L + limb) * Cfg::N;
-    fwd_task<Cfg>(sm, sg.in + off, sg.out + off, (size_t)sg.L * Cfg::N, sg.limbs[limb], threadIdx.x);
+    fwd_task<Cfg, SP>(sm, sg.in + off, sg.out + off, (size_t)sg.L * Cfg::N, sg.limbs[limb], threadIdx.x);
 }
 
-template <class Cfg, int NS>
+template <class Cfg, int NS, bool SP>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
 k_ntt_inv(const __grid_constant__ NttSegsT<NS> segs)
 {
@@ -196,14 +193,14 @@ k_ntt_inv(const __grid_constant__ NttSegsT<NS> segs)
     const uint32_t local = blockIdx.x - sg.cta_begin;
     const uint32_t limb = sg.limb0 + local / sg.n_groups, grp = local % sg.n_groups;
     const size_t off = ((size_t)grp * Cfg::NP * sg.L + limb) * Cfg::N;
-    inv_task<Cfg>(sm, sg.in + off, sg.out + off, (size_t)sg.L * Cfg::N, sg.limbs[limb], threadIdx.x);
+    inv_task<Cfg, SP>(sm, sg.in + off, sg.out + off, (size_t)sg.L * Cfg::N, sg.limbs[limb], threadIdx.x);
 }
 
 // Inverse NTT of a layer's outputs with the server step's epilogue (Sec. 7, Sec.
 // 6.2: only the output coefficients of c0 go back, masked): one CTA per output
 // polynomial (limb-major).  c1 is stored in full; c0 goes through shared memory
 // and only its S output slots are written, each minus Delta * mask.
-template <class Cfg>
+template <class Cfg, bool SP>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
 k_ntt_inv_extract(const __grid_constant__ ExtractArgs ex, const LimbConst *__restrict__ limbs, uint32_t L)
 {
@@ -215,7 +212,7 @@ k_ntt_inv_extract(const __grid_constant__ ExtractArgs ex, const LimbConst *__res
     const uint32_t o = pi >> 1, comp = pi & 1;
     const LimbConst &lc = limbs[limb];
     uint64_t x[1][Cfg::C];
-    inv_core<Cfg>(x, sm, ex.y + ((size_t)pi * L + limb) * Cfg::N, 0, lc, tid);
+    inv_core<Cfg, SP>(x, sm, ex.y + ((size_t)pi * L + limb) * Cfg::N, 0, lc, tid);
     if (comp) {
         uint64_t *d = ex.c1 + ((size_t)o * L + limb) * Cfg::N;
 #pragma unroll
@@ -249,7 +246,7 @@ k_ntt_inv_extract(const __grid_constant__ ExtractArgs ex, const LimbConst *__res
 // ---------------------------------------------------------------------------
 // group = one output and NP of its components; limb-major item order so that
 // consecutive CTAs (consecutive outputs) share weight polynomials in L2.
-template <class Cfg>
+template <class Cfg, bool SP>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
 k_mac_intt(const uint64_t *__restrict__ ct_ntt, const uint64_t *__restrict__ pt_ntt,
            const uint32_t *__restrict__ term_ptr, const uint32_t *__restrict__ terms,
@@ -301,7 +298,7 @@ k_mac_intt(const uint64_t *__restrict__ ct_ntt, const uint64_t *__restrict__ pt_
     }
     uint64_t x[NP][C];
     load_round0<Cfg>(x, sm, tid);
-    inv_transform<Cfg>(x, sm, lc, lc.tw_i, tid);
+    inv_transform<Cfg>(x, sm, lc, tw_arith<SP>(lc), tid);
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
         uint64_t *dst = out + (((size_t)o * 2 + comp0 + p) * L + limb) * N;
@@ -339,7 +336,7 @@ __device__ __forceinline__ void unrotate(ulonglong2 (&t)[V], uint32_t rho)
     });
 }
 
-template <class Cfg, int NS>
+template <class Cfg, int NS, bool SP>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
 k_ntt_inv_tma(const __grid_constant__ NttSegsT<NS> segs, uint32_t total, int *err)
 {
@@ -404,7 +401,7 @@ k_ntt_inv_tma(const __grid_constant__ NttSegsT<NS> segs, uint32_t total, int *er
             x[0][2 * j] = t[j].x;
             x[0][2 * j + 1] = t[j].y;
         }
-        inv_transform<Cfg>(x, buf, lc, lc.tw_i, tid);
+        inv_transform<Cfg>(x, buf, lc, tw_arith<SP>(lc), tid);
         unsigned long long *dst = reinterpret_cast<unsigned long long *>(sg.out + ((size_t)poly * sg.L + limb) * N);
 #pragma unroll
         for (int r = 0; r < C; ++r) __stcs(dst + inv_out_elem<Cfg>(tid, r), (unsigned long long)x[0][r]);  // as inv_task
@@ -424,7 +421,7 @@ k_ntt_inv_tma(const __grid_constant__ NttSegsT<NS> segs, uint32_t total, int *er
 // next unit's cp.async copies into it (8-byte words, coalesced in global
 // memory, swizzled in shared memory), so that the next load overlaps the last
 // round and the stores.
-template <class Cfg, int NS>
+template <class Cfg, int NS, bool SP>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
 k_ntt_inv_pf(const __grid_constant__ NttSegsT<NS> segs, uint32_t total)
 {
@@ -470,7 +467,8 @@ k_ntt_inv_pf(const __grid_constant__ NttSegsT<NS> segs, uint32_t total)
 #pragma unroll
         for (int r = 0; r < C; ++r) x[0][r] = sm[spos<Cfg>(tid * C + r)];
         const uint32_t next = u + G;
-        inv_transform<Cfg>(x, sm, lc, lc.tw_i, tid, [&] {
+        const TwArith<SP> ar = tw_arith<SP>(lc);
+        inv_transform<Cfg>(x, sm, lc, ar, tid, [&] {
             __syncthreads();  // the last exchange has been read by every thread
             if (next < total) prefetch(next);
         });
@@ -489,7 +487,7 @@ k_ntt_inv_pf(const __grid_constant__ NttSegsT<NS> segs, uint32_t total)
 // transform of N/2 residues (HCfg) with the full table's twiddles
 // (fwd_transform's HALF mode), then stores half c canonical, as 16-byte pairs.
 // The arithmetic is the one-CTA transform's, stage by stage.
-template <class HCfg, int NS>
+template <class HCfg, int NS, bool SP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(HCfg::T, HCfg::MINB)
 k_ntt_fwd_pair(const __grid_constant__ NttSegsT<NS> segs)
 {
@@ -507,27 +505,26 @@ k_ntt_fwd_pair(const __grid_constant__ NttSegsT<NS> segs)
     const size_t off = ((size_t)poly * sg.L + limb) * (2 * (size_t)NH);
     const uint64_t *src = sg.in + off;
     const LimbConst &lc = sg.limbs[limb];
-    const uint64_t q = lc.q, nq = 0ull - q, q4 = 4 * q;
     const ulonglong2 w = __ldg(lc.tw_f + 1);
     const uint32_t to0 = cluster_map(sm, 0), to1 = cluster_map(sm, 1);
     cluster_sync();  // both CTAs are running before either writes into the other
+    const TwArith<SP> ar = tw_arith<SP>(lc);
 #pragma unroll
     for (int r = 0; r < C / 2; ++r) {
         const uint32_t j = rank * (NH / 2) + tid + r * T;  // < NH
         const uint64_t X = __ldg(src + j), Y = __ldg(src + j + NH);
-        const uint64_t t = shoup_lazy(Y, w.x, w.y, nq);   // < 4q
+        const uint64_t t = ar.mul(Y, w);
         st_cluster_u64(to0 + j * 8, X + t);
-        st_cluster_u64(to1 + j * 8, X - t + q4);
+        st_cluster_u64(to1 + j * 8, ar.sub(X, t));
     }
     cluster_sync();  // the halves are complete; no remote access after this point
     uint64_t x[1][C];
 #pragma unroll
     for (int r = 0; r < C; ++r) x[0][r] = sm[tid + r * T];
-    fwd_transform<HCfg, 0, true>(x, sm, lc.tw_f, nullptr, q, tid, 2 + (int)rank);
-    const uint32_t ones = (uint32_t)lc.one_s;
+    fwd_rounds<HCfg, 0, true>(x, sm, lc.tw_f, nullptr, ar, tid, 2 + (int)rank);
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < C; ++r) sm[spos<HCfg>(tid * C + r)] = canon3(reduce_lazy(x[0][r], ones, nq), q);
+    for (int r = 0; r < C; ++r) sm[spos<HCfg>(tid * C + r)] = ar.canon(x[0][r]);
     __syncthreads();
     ulonglong2 *d = reinterpret_cast<ulonglong2 *>(sg.out + off + (size_t)rank * NH);
 #pragma unroll
@@ -548,7 +545,7 @@ k_ntt_fwd_pair(const __grid_constant__ NttSegsT<NS> segs)
 // for j in [c N/4, (c+1) N/4), reading both halves through distributed shared
 // memory, and stores both outputs; a last cluster barrier keeps each CTA's
 // shared memory alive until its peer has read it.
-template <class HCfg, int NS>
+template <class HCfg, int NS, bool SP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(HCfg::T, HCfg::MINB)
 k_ntt_inv_pair(const __grid_constant__ NttSegsT<NS> segs)
 {
@@ -565,7 +562,6 @@ k_ntt_inv_pair(const __grid_constant__ NttSegsT<NS> segs)
     const uint32_t limb = sg.limb0 + local / sg.n_groups, poly = local % sg.n_groups;
     const size_t off = ((size_t)poly * sg.L + limb) * (2 * (size_t)NH);
     const LimbConst &lc = sg.limbs[limb];
-    const uint64_t q = lc.q, nq = 0ull - q;
     // half c: coalesced 16-byte loads into shared memory, then the round-0 layout
     const ulonglong2 *s2 = reinterpret_cast<const ulonglong2 *>(sg.in + off + (size_t)rank * NH);
 #pragma unroll
@@ -577,20 +573,22 @@ k_ntt_inv_pair(const __grid_constant__ NttSegsT<NS> segs)
     }
     uint64_t x[1][C];
     load_round0<HCfg>(x, sm, tid);
-    inv_transform<HCfg, 0, NoHook, true>(x, sm, lc, lc.tw_i, tid, NoHook{}, 2 + (int)rank);
+    const TwArith<SP> ar = tw_arith<SP>(lc);
+    inv_transform<HCfg, true>(x, sm, lc, ar, tid, NoHook{}, 2 + (int)rank);
     __syncthreads();  // the transform's last exchange has been read
 #pragma unroll
     for (int r = 0; r < C; ++r) sm[inv_out_elem<HCfg>(tid, r)] = x[0][r];
     const uint32_t from0 = cluster_map(sm, 0), from1 = cluster_map(sm, 1);
     cluster_sync();  // both halves are in shared memory
-    const uint64_t qs = q << (HCfg::LOGN);  // bound of the last stage's inputs (stage log2 N - 1)
+    const uint64_t qs = ar.q * HCfg::N;  // bound of the last stage's inputs (Shoup)
+    const ulonglong2 wn = make_ulonglong2(lc.ninv, lc.ninv_s), wnw = make_ulonglong2(lc.ninvw, lc.ninvw_s);
     uint64_t *out = sg.out + off;
 #pragma unroll
     for (int r = 0; r < C / 2; ++r) {
         const uint32_t j = rank * (NH / 2) + tid + r * T;  // < NH
         const uint64_t X = ld_cluster_u64(from0 + j * 8), Y = ld_cluster_u64(from1 + j * 8);
-        out[j] = canon4(shoup_lazy(X + Y, lc.ninv, lc.ninv_s, nq), q);
-        out[j + NH] = canon4(shoup_lazy(X - Y + qs, lc.ninvw, lc.ninvw_s, nq), q);
+        out[j] = ar.mul_canon(X + Y, wn);
+        out[j + NH] = ar.mul_canon(ar.sub(X, Y, qs), wnw);
     }
     cluster_sync();  // the peer has read this CTA's half
 }
@@ -600,7 +598,7 @@ k_ntt_inv_pair(const __grid_constant__ NttSegsT<NS> segs)
 // one limb.  ct is the product's ciphertext [2][L][N], pt its NTT-domain
 // plaintext [L][N], out its output ciphertext [2][L][N]:
 //   out[c][limb] (+)= INTT(NTT(ct[c][limb]) . pt[limb])                  (App. C.1)
-template <class Cfg>
+template <class Cfg, bool SP>
 __device__ __forceinline__ void product_task(uint64_t *sm, const uint64_t *__restrict__ ct,
                                              const uint64_t *__restrict__ pt, uint64_t *out, const LimbConst &lc,
                                              uint32_t L, uint32_t limb, uint32_t comp0, bool accumulate)
@@ -616,26 +614,19 @@ __device__ __forceinline__ void product_task(uint64_t *sm, const uint64_t *__res
 #pragma unroll
         for (int r = 0; r < C; ++r) x[p][r] = __ldg(src + tid + r * T);
     }
-    fwd_transform<Cfg>(x, sm, lc.tw_f, lc.tw_r, q, tid);  // lazy values < 57 q, contiguous layout
-
-    const uint64_t nq = 0ull - q, r64 = lc.r64, r64_s = lc.r64_s;
-    const uint32_t ones = (uint32_t)lc.one_s;
+    const TwArith<SP> ar = tw_arith<SP>(lc);
+    fwd_transform<Cfg>(x, sm, lc, ar, tid);  // lazy values, contiguous layout
     const ulonglong2 *wp = reinterpret_cast<const ulonglong2 *>(pt + (size_t)limb * N + tid * C);
 #pragma unroll
     for (int r = 0; r < C / 2; ++r) {
         const ulonglong2 w = __ldg(wp + r);
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-            MacAcc a0, a1;
-            mac_zero(a0);
-            mac_zero(a1);
-            mac_add(a0, x[p][2 * r], w.x);       // x < 2^56 (lazy forward output)
-            mac_add(a1, x[p][2 * r + 1], w.y);
-            x[p][2 * r] = mac_reduce(a0, q, nq, r64, r64_s, ones);
-            x[p][2 * r + 1] = mac_reduce(a1, q, nq, r64, r64_s, ones);
+            x[p][2 * r] = mul_slot(ar, x[p][2 * r], w.x, lc.r64, lc.r64_s);
+            x[p][2 * r + 1] = mul_slot(ar, x[p][2 * r + 1], w.y, lc.r64, lc.r64_s);
         }
     }
-    inv_transform<Cfg>(x, sm, lc, lc.tw_i, tid);
+    inv_transform<Cfg>(x, sm, lc, ar, tid);
 
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
@@ -653,7 +644,7 @@ __device__ __forceinline__ void product_task(uint64_t *sm, const uint64_t *__res
     }
 }
 
-template <class Cfg>
+template <class Cfg, bool SP>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
 k_product(const uint64_t *__restrict__ ct, const uint64_t *__restrict__ pt_ntt,
           const uint32_t *__restrict__ out_index, uint64_t *out, const LimbConst *__restrict__ limbs,
@@ -666,7 +657,7 @@ k_product(const uint64_t *__restrict__ ct, const uint64_t *__restrict__ pt_ntt,
     const uint32_t j = grp / CPG;
     const uint32_t comp0 = (grp % CPG) * Cfg::NP;
     const uint32_t oj = out_index ? __ldg(out_index + j) : j;
-    product_task<Cfg>(sm, ct + (size_t)j * 2 * L * N, pt_ntt + (size_t)j * L * N, out + (size_t)oj * 2 * L * N,
+    product_task<Cfg, SP>(sm, ct + (size_t)j * 2 * L * N, pt_ntt + (size_t)j * L * N, out + (size_t)oj * 2 * L * N,
                       limbs[limb], L, limb, comp0, accumulate != 0);
 }
 
@@ -676,8 +667,8 @@ k_product(const uint64_t *__restrict__ ct, const uint64_t *__restrict__ pt_ntt,
 // ===========================================================================
 namespace detail {
 
-// one cache bit per (kernel family, launch shape, device)
-template <class Cfg, int KIND, class K>
+// one cache bit per (kernel family, launch shape, twiddle form, device)
+template <class Cfg, bool SP, int KIND, class K>
 hc_status prepare(K kernel, size_t smem)
 {
     static std::atomic<uint32_t> done{0};
@@ -716,22 +707,22 @@ inline hc_status after_launch(const char *what)
     return e == cudaSuccess ? HC_OK : cuda_error(e, what);
 }
 
-template <class Cfg, int KIND, int NS>
+template <class Cfg, bool SP, int KIND, int NS>
 hc_status run_ntt_segs(const NttSegsT<NS> &segs, cudaStream_t s, bool inverse)
 {
     uint32_t items = 0;
     for (uint32_t i = 0; i < segs.n; ++i) items = segs.s[i].cta_begin + segs.s[i].n_groups * seg_limbs(segs.s[i]);
     if (items == 0) return HC_OK;
     if (inverse) {
-        auto kern = k_ntt_inv<Cfg, NS>;
-        hc_status st = prepare<Cfg, KIND * 1000 + NS>(kern, Cfg::SMEM_BYTES);
+        auto kern = k_ntt_inv<Cfg, NS, SP>;
+        hc_status st = prepare<Cfg, SP, KIND * 1000 + NS>(kern, Cfg::SMEM_BYTES);
         if (st != HC_OK) return st;
         ProfileScope ps(kname<Cfg>(KK_INV), s);
         kern<<<items, Cfg::T, Cfg::SMEM_BYTES, s>>>(segs);
         return after_launch("k_ntt_inv");
     }
-    auto kern = k_ntt_fwd<Cfg, NS>;
-    hc_status st = prepare<Cfg, KIND * 1000 + NS>(kern, Cfg::SMEM_BYTES);
+    auto kern = k_ntt_fwd<Cfg, NS, SP>;
+    hc_status st = prepare<Cfg, SP, KIND * 1000 + NS>(kern, Cfg::SMEM_BYTES);
     if (st != HC_OK) return st;
     ProfileScope ps(kname<Cfg>(KK_FWD), s);
     kern<<<items, Cfg::T, Cfg::SMEM_BYTES, s>>>(segs);
@@ -740,14 +731,14 @@ hc_status run_ntt_segs(const NttSegsT<NS> &segs, cudaStream_t s, bool inverse)
 
 // persistent TMA-fed inverse NTT: segs' cta_begin are unit offsets (n_groups
 // polynomials x L limbs per segment); one launch of resident CTAs
-template <class Cfg, int NS>
+template <class Cfg, bool SP, int NS>
 hc_status run_ntt_inv_tma(const NttSegsT<NS> &segs, int *err, cudaStream_t s)
 {
     uint32_t total = 0;
     for (uint32_t i = 0; i < segs.n; ++i) total = segs.s[i].cta_begin + segs.s[i].n_groups * seg_limbs(segs.s[i]);
     if (total == 0) return HC_OK;
     constexpr size_t smem = 2 * Cfg::SMEM_BYTES;
-    auto kern = k_ntt_inv_tma<Cfg, NS>;
+    auto kern = k_ntt_inv_tma<Cfg, NS, SP>;
     static std::atomic<int> resident[32];
     int dev = 0;
     cudaGetDevice(&dev);
@@ -768,7 +759,7 @@ hc_status run_ntt_inv_tma(const NttSegsT<NS> &segs, int *err, cudaStream_t s)
     return after_launch("k_ntt_inv_tma");
 }
 
-template <class HCfg, int NS>
+template <class HCfg, bool SP, int NS>
 hc_status run_ntt_inv_pair(const NttSegsT<NS> &segs, cudaStream_t s);
 
 // persistent prefetching inverse NTT: segs' cta_begin are unit offsets
@@ -776,14 +767,14 @@ hc_status run_ntt_inv_pair(const NttSegsT<NS> &segs, cudaStream_t s);
 // With fewer limbs than resident CTAs no CTA would prefetch, and the limbs run
 // as two-CTA clusters (k_ntt_inv_pair, halves of shape PCfg) instead: measured
 // on GB300, 7-14 % lower latency for a few limbs, 11 % higher time for 1536.
-template <class Cfg, class PCfg, int NS>
+template <class Cfg, class PCfg, bool SP, int NS>
 hc_status run_ntt_inv_pf(const NttSegsT<NS> &segs, cudaStream_t s)
 {
     uint32_t total = 0;
     for (uint32_t i = 0; i < segs.n; ++i) total = segs.s[i].cta_begin + segs.s[i].n_groups * seg_limbs(segs.s[i]);
     if (total == 0) return HC_OK;
     constexpr size_t smem = Cfg::SMEM_BYTES;
-    auto kern = k_ntt_inv_pf<Cfg, NS>;
+    auto kern = k_ntt_inv_pf<Cfg, NS, SP>;
     static std::atomic<int> resident[32];
     int dev = 0;
     cudaGetDevice(&dev);
@@ -798,7 +789,7 @@ hc_status run_ntt_inv_pf(const NttSegsT<NS> &segs, cudaStream_t s)
         r = per_sm * sms;
         resident[dev & 31].store(r);
     }
-    if (total < (uint32_t)r) return run_ntt_inv_pair<PCfg>(segs, s);
+    if (total < (uint32_t)r) return run_ntt_inv_pair<PCfg, SP>(segs, s);
     const uint32_t grid = total < (uint32_t)r ? total : (uint32_t)r;
     ProfileScope ps(kname<Cfg>(KK_INV), s);
     kern<<<grid, Cfg::T, smem, s>>>(segs, total);
@@ -807,30 +798,30 @@ hc_status run_ntt_inv_pf(const NttSegsT<NS> &segs, cudaStream_t s)
 
 // forward NTTs by clusters of two CTAs: segs' cta_begin are unit offsets (n_groups
 // polynomials x L limbs per segment); two CTAs per unit
-template <class HCfg, int NS>
+template <class HCfg, bool SP, int NS>
 hc_status run_ntt_fwd_pair(const NttSegsT<NS> &segs, cudaStream_t s)
 {
     uint32_t total = 0;
     for (uint32_t i = 0; i < segs.n; ++i) total = segs.s[i].cta_begin + segs.s[i].n_groups * seg_limbs(segs.s[i]);
     if (total == 0) return HC_OK;
     if (total > 0x3fffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
-    auto kern = k_ntt_fwd_pair<HCfg, NS>;
-    hc_status st = prepare<HCfg, 7000 + NS>(kern, HCfg::SMEM_BYTES);
+    auto kern = k_ntt_fwd_pair<HCfg, NS, SP>;
+    hc_status st = prepare<HCfg, SP, 7000 + NS>(kern, HCfg::SMEM_BYTES);
     if (st != HC_OK) return st;
     ProfileScope ps(kname_of(KK_FWD, HCfg::LOGN + 1), s);
     kern<<<2 * total, HCfg::T, HCfg::SMEM_BYTES, s>>>(segs);
     return after_launch("k_ntt_fwd_pair");
 }
 
-template <class HCfg, int NS>
+template <class HCfg, bool SP, int NS>
 hc_status run_ntt_inv_pair(const NttSegsT<NS> &segs, cudaStream_t s)
 {
     uint32_t total = 0;
     for (uint32_t i = 0; i < segs.n; ++i) total = segs.s[i].cta_begin + segs.s[i].n_groups * seg_limbs(segs.s[i]);
     if (total == 0) return HC_OK;
     if (total > 0x3fffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
-    auto kern = k_ntt_inv_pair<HCfg, NS>;
-    hc_status st = prepare<HCfg, 8000 + NS>(kern, HCfg::SMEM_BYTES);
+    auto kern = k_ntt_inv_pair<HCfg, NS, SP>;
+    hc_status st = prepare<HCfg, SP, 8000 + NS>(kern, HCfg::SMEM_BYTES);
     if (st != HC_OK) return st;
     ProfileScope ps(kname_of(KK_INV, HCfg::LOGN + 1), s);
     kern<<<2 * total, HCfg::T, HCfg::SMEM_BYTES, s>>>(segs);
@@ -846,29 +837,29 @@ inline NttSegs1 one_seg(const hc_ctx *ctx, const uint64_t *in, uint64_t *out, si
     return segs;
 }
 
-template <class Cfg>
+template <class Cfg, bool SP>
 hc_status run_ntt_fwd(const hc_ctx *ctx, const uint64_t *in, uint64_t *out, size_t n_groups, cudaStream_t s)
 {
     if (n_groups == 0) return HC_OK;
     if (n_groups * ctx->L > 0x7fffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
-    return run_ntt_segs<Cfg, KK_FWD>(one_seg(ctx, in, out, n_groups), s, false);
+    return run_ntt_segs<Cfg, SP, KK_FWD>(one_seg(ctx, in, out, n_groups), s, false);
 }
 
-template <class Cfg>
+template <class Cfg, bool SP>
 hc_status run_ntt_inv(const hc_ctx *ctx, const uint64_t *in, uint64_t *out, size_t n_groups, cudaStream_t s)
 {
     if (n_groups == 0) return HC_OK;
     if (n_groups * ctx->L > 0x7fffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
-    return run_ntt_segs<Cfg, KK_INV>(one_seg(ctx, in, out, n_groups), s, true);
+    return run_ntt_segs<Cfg, SP, KK_INV>(one_seg(ctx, in, out, n_groups), s, true);
 }
 
-template <class Cfg>
+template <class Cfg, bool SP>
 hc_status run_mac_intt(const hc_ctx *ctx, const uint64_t *ct_ntt, const uint64_t *pt_ntt, MacTerms terms,
                        uint64_t *out, size_t n_out, cudaStream_t s)
 {
     if (n_out == 0) return HC_OK;
-    auto kern = k_mac_intt<Cfg>;
-    hc_status st = prepare<Cfg, KK_MAC>(kern, Cfg::SMEM_BYTES);
+    auto kern = k_mac_intt<Cfg, SP>;
+    hc_status st = prepare<Cfg, SP, KK_MAC>(kern, Cfg::SMEM_BYTES);
     if (st != HC_OK) return st;
     const size_t n_groups = n_out * (2 / Cfg::NP);
     const size_t items = n_groups * ctx->L;
@@ -879,12 +870,12 @@ hc_status run_mac_intt(const hc_ctx *ctx, const uint64_t *ct_ntt, const uint64_t
     return after_launch("k_mac_intt");
 }
 
-template <class Cfg>
+template <class Cfg, bool SP>
 hc_status run_inv_extract(const hc_ctx *ctx, const ExtractArgs &ex, cudaStream_t s)
 {
     if (ex.O == 0) return HC_OK;
-    auto kern = k_ntt_inv_extract<Cfg>;
-    hc_status st = prepare<Cfg, KK_INV_EXTRACT>(kern, Cfg::SMEM_BYTES);
+    auto kern = k_ntt_inv_extract<Cfg, SP>;
+    hc_status st = prepare<Cfg, SP, KK_INV_EXTRACT>(kern, Cfg::SMEM_BYTES);
     if (st != HC_OK) return st;
     const uint32_t Lc = ex.Lc ? ex.Lc : ctx->L;
     if (ex.limb0 + Lc > ctx->L) return set_error(HC_ERR_INVALID_ARG, "limb range out of bounds");
@@ -895,13 +886,13 @@ hc_status run_inv_extract(const hc_ctx *ctx, const ExtractArgs &ex, cudaStream_t
     return after_launch("k_ntt_inv_extract");
 }
 
-template <class Cfg>
+template <class Cfg, bool SP>
 hc_status run_product(const hc_ctx *ctx, const uint64_t *ct, const uint64_t *pt_ntt, const uint32_t *out_index,
                       uint64_t *out, size_t n, bool accumulate, cudaStream_t s)
 {
     if (n == 0) return HC_OK;
-    auto kern = k_product<Cfg>;
-    hc_status st = prepare<Cfg, KK_PROD>(kern, Cfg::SMEM_BYTES);
+    auto kern = k_product<Cfg, SP>;
+    hc_status st = prepare<Cfg, SP, KK_PROD>(kern, Cfg::SMEM_BYTES);
     if (st != HC_OK) return st;
     const size_t n_groups = n * (2 / Cfg::NP);
     const size_t items = n_groups * ctx->L;
@@ -914,7 +905,7 @@ hc_status run_product(const hc_ctx *ctx, const uint64_t *ct, const uint64_t *pt_
 
 }  // namespace detail
 
-template <int LOGN, int V>
+template <int LOGN, int V, bool SP>
 hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaStream_t s)
 {
     using Fused = VCfg<LOGN, V, false>;
@@ -922,9 +913,9 @@ hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaS
     if constexpr (use_inv_tma<LOGN, V> || use_inv_pf<LOGN, V>) {
         auto run = [&](const auto &segs) {
             if constexpr (use_inv_tma<LOGN, V>)
-                return detail::run_ntt_inv_tma<typename InvTma<LOGN>::Cfg>(segs, timeout_flag(ctx), s);
+                return detail::run_ntt_inv_tma<typename InvTma<LOGN>::Cfg, SP>(segs, timeout_flag(ctx), s);
             else
-                return detail::run_ntt_inv_pf<typename InvPf<LOGN>::Cfg, typename FwdPair<LOGN>::Cfg>(segs, s);
+                return detail::run_ntt_inv_pf<typename InvPf<LOGN>::Cfg, typename FwdPair<LOGN>::Cfg, SP>(segs, s);
         };
         if (kind == KK_INV || kind == KK_INVCT) {
             const size_t polys = kind == KK_INV ? a.n : 2 * a.n;
@@ -949,7 +940,7 @@ hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaS
             const size_t polys = kind == KK_FWD ? a.n : 2 * a.n;
             if (polys == 0) return HC_OK;
             if (polys * ctx->L > 0x7fffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
-            return detail::run_ntt_fwd_pair<HC>(detail::one_seg(ctx, a.in, a.out, polys), s);
+            return detail::run_ntt_fwd_pair<HC, SP>(detail::one_seg(ctx, a.in, a.out, polys), s);
         }
         if (kind == KK_FWDCT_SEGS) {
             NttSegs segs = *a.segs;
@@ -959,14 +950,14 @@ hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaS
                 segs.s[i].cta_begin = begin;
                 begin += segs.s[i].n_groups * seg_limbs(segs.s[i]);
             }
-            return detail::run_ntt_fwd_pair<HC>(segs, s);
+            return detail::run_ntt_fwd_pair<HC, SP>(segs, s);
         }
     }
     switch (kind) {
-    case KK_FWD: return detail::run_ntt_fwd<Single>(ctx, a.in, a.out, a.n, s);
-    case KK_INV: return detail::run_ntt_inv<Single>(ctx, a.in, a.out, a.n, s);
-    case KK_FWDCT: return detail::run_ntt_fwd<Fused>(ctx, a.in, a.out, a.n * (2 / Fused::NP), s);
-    case KK_INVCT: return detail::run_ntt_inv<Fused>(ctx, a.in, a.out, a.n * (2 / Fused::NP), s);
+    case KK_FWD: return detail::run_ntt_fwd<Single, SP>(ctx, a.in, a.out, a.n, s);
+    case KK_INV: return detail::run_ntt_inv<Single, SP>(ctx, a.in, a.out, a.n, s);
+    case KK_FWDCT: return detail::run_ntt_fwd<Fused, SP>(ctx, a.in, a.out, a.n * (2 / Fused::NP), s);
+    case KK_INVCT: return detail::run_ntt_inv<Fused, SP>(ctx, a.in, a.out, a.n * (2 / Fused::NP), s);
     case KK_FWDCT_SEGS:
     case KK_INVCT_SEGS: {
         // segment n_groups are given in ciphertexts; scale to CTAs of this shape
@@ -977,30 +968,30 @@ hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaS
             segs.s[i].cta_begin = begin;
             begin += segs.s[i].n_groups * seg_limbs(segs.s[i]);
         }
-        return kind == KK_FWDCT_SEGS ? detail::run_ntt_segs<Fused, KK_FWDCT>(segs, s, false)
-                                     : detail::run_ntt_segs<Fused, KK_INVCT>(segs, s, true);
+        return kind == KK_FWDCT_SEGS ? detail::run_ntt_segs<Fused, SP, KK_FWDCT>(segs, s, false)
+                                     : detail::run_ntt_segs<Fused, SP, KK_INVCT>(segs, s, true);
     }
-    case KK_MAC: return detail::run_mac_intt<Fused>(ctx, a.in, a.pt, a.terms, a.out, a.n, s);
-    case KK_PROD: return detail::run_product<Fused>(ctx, a.in, a.pt, a.out_index, a.out, a.n, a.accumulate, s);
+    case KK_MAC: return detail::run_mac_intt<Fused, SP>(ctx, a.in, a.pt, a.terms, a.out, a.n, s);
+    case KK_PROD: return detail::run_product<Fused, SP>(ctx, a.in, a.pt, a.out_index, a.out, a.n, a.accumulate, s);
     case KK_INV_EXTRACT:
         // variant 2 of the inverse kinds is persistent at N >= 8192; the epilogue
         // kernel (one output limb per CTA, shared memory busy until its last store)
         // takes the best one-CTA shape there, variant 1's
         if constexpr (V == 2 && LOGN >= 13)
-            return detail::run_inv_extract<VCfg<LOGN, 1, true>>(ctx, *a.ex, s);
+            return detail::run_inv_extract<VCfg<LOGN, 1, true>, SP>(ctx, *a.ex, s);
         else
-            return detail::run_inv_extract<Single>(ctx, *a.ex, s);
+            return detail::run_inv_extract<Single, SP>(ctx, *a.ex, s);
     default: return set_error(HC_ERR_INVALID_ARG, "unknown kernel kind %d", kind);
     }
 }
 
-template <int LOGN>
+template <int LOGN, bool SP>
 hc_status launch_n(const hc_ctx *ctx, int kind, int variant, const LaunchArgs &a, cudaStream_t s)
 {
     switch (variant) {
-    case 0: return launch_variant<LOGN, 0>(ctx, kind, a, s);
-    case 1: return launch_variant<LOGN, 1>(ctx, kind, a, s);
-    case 2: return launch_variant<LOGN, 2>(ctx, kind, a, s);
+    case 0: return launch_variant<LOGN, 0, SP>(ctx, kind, a, s);
+    case 1: return launch_variant<LOGN, 1, SP>(ctx, kind, a, s);
+    case 2: return launch_variant<LOGN, 2, SP>(ctx, kind, a, s);
     default: return set_error(HC_ERR_INVALID_ARG, "unknown launch variant %d", variant);
     }
 }

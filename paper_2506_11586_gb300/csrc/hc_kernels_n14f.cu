@@ -1,0 +1,6 @@
+// hc_kernels_n14f.cu -- kernels and launchers for N = 16384, folded twiddles (see hc_kernels.cuh).
+#include "hc_kernels.cuh"
+
+namespace hc {
+template hc_status launch_n<14, true>(const hc_ctx *, int, int, const LaunchArgs &, cudaStream_t);
+}  // namespace hc

@@ -272,10 +272,11 @@ hc_status dispatch(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaStream_
                   : kind == KK_INVCT_SEGS  ? ctx->variant[KK_INVCT]
                   : kind == KK_INV_EXTRACT ? ctx->variant[KK_INVCT]
                                            : ctx->variant[kind];
+    const bool fold = a.segs ? a.segs->s[0].fold != 0 : ctx->fold;
     switch (ctx->logN) {
-    case 12: return launch_n<12>(ctx, kind, v, a, s);
-    case 13: return launch_n<13>(ctx, kind, v, a, s);
-    case 14: return launch_n<14>(ctx, kind, v, a, s);
+    case 12: return fold ? launch_n<12, true>(ctx, kind, v, a, s) : launch_n<12, false>(ctx, kind, v, a, s);
+    case 13: return fold ? launch_n<13, true>(ctx, kind, v, a, s) : launch_n<13, false>(ctx, kind, v, a, s);
+    case 14: return fold ? launch_n<14, true>(ctx, kind, v, a, s) : launch_n<14, false>(ctx, kind, v, a, s);
     default: return set_error(HC_ERR_UNSUPPORTED, "unsupported N = %u", ctx->N);
     }
 }
@@ -327,9 +328,17 @@ hc_status launch_ntt_inv_ct(const hc_ctx *ctx, const uint64_t *in, uint64_t *out
 
 hc_status launch_ntt_ct_segs(const hc_ctx *ctx, const NttSegs &segs, bool inverse, cudaStream_t s)
 {
-    LaunchArgs a{};
-    a.segs = &segs;
-    return dispatch(ctx, inverse ? KK_INVCT_SEGS : KK_FWDCT_SEGS, a, s);
+    for (uint32_t fold = 0; fold < 2; ++fold) {
+        NttSegs part{};
+        for (uint32_t i = 0; i < segs.n; ++i)
+            if (segs.s[i].fold == fold) part.s[part.n++] = segs.s[i];
+        if (part.n == 0) continue;
+        LaunchArgs a{};
+        a.segs = &part;
+        hc_status st = dispatch(ctx, inverse ? KK_INVCT_SEGS : KK_FWDCT_SEGS, a, s);
+        if (st != HC_OK) return st;
+    }
+    return HC_OK;
 }
 
 hc_status launch_mac_intt(const hc_ctx *ctx, const uint64_t *ct_ntt, const uint64_t *pt_ntt, MacTerms terms,

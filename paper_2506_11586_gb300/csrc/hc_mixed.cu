@@ -25,6 +25,7 @@ static_assert(mix_comps_per_unit(12) == MixCfg12::NP && mix_comps_per_unit(13) =
               "unit split must match the per-degree shapes");
 constexpr size_t kMixSmem = MixCfg13::SMEM_BYTES > MixCfg14::SMEM_BYTES ? MixCfg13::SMEM_BYTES : MixCfg14::SMEM_BYTES;
 
+template <bool SP>
 __global__ void __launch_bounds__(kMixThreads, 1)
 k_product_mixed(const MixItem *__restrict__ items, const uint32_t *__restrict__ units, uint32_t n_units,
                 uint32_t *next)
@@ -42,30 +43,28 @@ k_product_mixed(const MixItem *__restrict__ items, const uint32_t *__restrict__ 
         const uint32_t limb = (code >> 1) & 7, comp = code & 1;
         const LimbConst &lc = it.limbs[limb];
         if (it.logN == 12)
-            product_task<MixCfg12>(sm, it.ct, it.pt, it.out, lc, it.L, limb, 0, false);
+            product_task<MixCfg12, SP>(sm, it.ct, it.pt, it.out, lc, it.L, limb, 0, false);
         else if (it.logN == 13)
-            product_task<MixCfg13>(sm, it.ct, it.pt, it.out, lc, it.L, limb, 0, false);
+            product_task<MixCfg13, SP>(sm, it.ct, it.pt, it.out, lc, it.L, limb, 0, false);
         else
-            product_task<MixCfg14>(sm, it.ct, it.pt, it.out, lc, it.L, limb, comp, false);
+            product_task<MixCfg14, SP>(sm, it.ct, it.pt, it.out, lc, it.L, limb, comp, false);
     }
 }
 
-}  // namespace
-
-hc_status launch_product_mixed(const MixItem *items, const uint32_t *units, uint32_t n_units, uint32_t *next,
-                               cudaStream_t s)
+template <bool SP>
+hc_status run_mixed(const MixItem *items, const uint32_t *units, uint32_t n_units, uint32_t *next, cudaStream_t s)
 {
-    if (n_units == 0) return HC_OK;
+    auto kern = k_product_mixed<SP>;
     static std::atomic<uint32_t> attr_done{0};
     static std::atomic<int> grid_cache[32];
     int dev = 0;
     cudaGetDevice(&dev);
     const uint32_t bit = 1u << (dev & 31);
     if (!(attr_done.load() & bit)) {
-        cudaError_t e = cudaFuncSetAttribute(k_product_mixed, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMixSmem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMixSmem);
         if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute(k_product_mixed)");
         int per_sm = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_product_mixed, kMixThreads, kMixSmem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kMixThreads, kMixSmem);
         if (e != cudaSuccess) return cuda_error(e, "occupancy(k_product_mixed)");
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return cuda_error(e, "cudaDeviceGetAttribute");
@@ -76,10 +75,19 @@ hc_status launch_product_mixed(const MixItem *items, const uint32_t *units, uint
     const uint32_t resident = (uint32_t)grid_cache[dev & 31].load();
     const uint32_t grid = n_units < resident ? n_units : resident;
     ProfileScope ps("k_product_mixed", s);
-    k_product_mixed<<<grid, kMixThreads, kMixSmem, s>>>(items, units, n_units, next);
+    kern<<<grid, kMixThreads, kMixSmem, s>>>(items, units, n_units, next);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "launch k_product_mixed");
     return HC_OK;
+}
+
+}  // namespace
+
+hc_status launch_product_mixed(const MixItem *items, const uint32_t *units, uint32_t n_units, uint32_t *next,
+                               bool fold, cudaStream_t s)
+{
+    if (n_units == 0) return HC_OK;
+    return fold ? run_mixed<true>(items, units, n_units, next, s) : run_mixed<false>(items, units, n_units, next, s);
 }
 
 }  // namespace hc

@@ -14,12 +14,23 @@
 // N / 2^(s+1) groups, group i uses psi^-rev(N/2^(s+1) + i); N^-1 is merged
 // into the last stage.
 //
-// Lazy bounds (q < 2^50, N <= 2^14; shoup_lazy returns values < 4q):
-//   forward: inputs < q; each stage adds 4q -> outputs < (4 log2 N + 1) q < 2^56
-//   inverse: inputs < q; stage 0 corrects its products to < 2q, so stage-s
+// Twiddle products (TwArith): limbs with q = 2^50 - c, c < 2^22 (SP), multiply by
+// folding, on signed lazy values; the others by Shoup's method, on unsigned ones.  A
+// context whose limbs are all of that kind holds its tables in the folded form (16
+// bytes per twiddle either way) and its launches take the SP kernels.  Both forms in one
+// kernel, chosen per CTA, cost the folded one registers: 112.8 instead of 97.7 us for
+// 1536 inverse transforms at N = 8192.
+// Lazy bounds (q < 2^50, N <= 2^14; products < 4q by Shoup, |.| <= 35 q folded):
+//   forward: inputs < q; each stage adds a product -> outputs < (4 log2 N + 1) q < 2^56
+//            by Shoup, |.| <= (35 log2 N + 1) q < 2^59 folded
+//   inverse, Shoup: inputs < q; stage 0 corrects its products to < 2q, so stage-s
 //            inputs are < 2^s q and X - Y + 2^s q < 2^(s+1) q <= 2^64; the last
 //            stage's Shoup steps (N^-1 merged) and two corrections give
 //            canonical output.
+//   inverse, folded: sums double and products restart at 35 q, so within a round only
+//            the registers that were sums throughout, or were products in the first
+//            stages, grow large; those above what the next round may take
+//            (inv_fold_limit) are folded below 5 q: at most four of a round's 32.
 // Twiddle loads: in the inverse's first round and the forward's last round
 // every thread needs its own twiddles (N/2 distinct ones in the inverse's
 // first stage); read from the natural tables a warp's 32 loads would hit 32
@@ -108,16 +119,15 @@ __device__ __forceinline__ void static_for(F &&f)
 // transform's first stage (see k_ntt_fwd_pair): local stage s, group i uses the
 // full table's entry tmul*2^s + i, tmul = 2 + the half's index; every round
 // reads the natural table.
-template <class Cfg, int R, int SIG, bool HALF = false>
+template <class Cfg, int R, int SIG, bool HALF, bool SP>
 __device__ __forceinline__ void fwd_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const ulonglong2 *__restrict__ tw,
-                                          const ulonglong2 *__restrict__ twr, uint64_t q, int v, int g0, int tid,
-                                          int tmul = 1)
+                                          const ulonglong2 *__restrict__ twr, const TwArith<SP> &ar, int v, int g0,
+                                          int tid, int tmul)
 {
     using RS = RoundShape<Cfg, R>;
     static_assert(Cfg::LOGC >= 3 && Cfg::LOGC <= 5, "last-round tables exist for LOGC = 3, 4, 5");
     constexpr int half = RS::KK >> (SIG + 1);
     constexpr bool last = R == Cfg::NROUNDS - 1 && !HALF;  // every thread has its own twiddles (g0 = tid*SUBS + v)
-    const uint64_t nq = 0ull - q, q4 = 4 * q;
 #pragma unroll
     for (int lam = 0; lam < (1 << SIG); ++lam) {
         // last round: the rearranged table, stage S0 + SIG at [2^(S0+SIG) - 2^S0],
@@ -132,17 +142,17 @@ __device__ __forceinline__ void fwd_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const 
 #pragma unroll
             for (int p = 0; p < Cfg::NP; ++p) {
                 const uint64_t X = x[p][j];
-                const uint64_t t = shoup_lazy(x[p][j + half], w.x, w.y, nq);  // < 4q
+                const uint64_t t = ar.mul(x[p][j + half], w);
                 x[p][j] = X + t;
-                x[p][j + half] = X - t + q4;
+                x[p][j + half] = ar.sub(X, t);
             }
         }
     }
 }
 
-template <class Cfg, int R, bool HALF = false>
+template <class Cfg, int R, bool HALF, bool SP>
 __device__ __forceinline__ void fwd_round(uint64_t (&x)[Cfg::NP][Cfg::C], const ulonglong2 *__restrict__ tw,
-                                          const ulonglong2 *__restrict__ twr, uint64_t q, int tid, int tmul = 1)
+                                          const ulonglong2 *__restrict__ twr, const TwArith<SP> &ar, int tid, int tmul)
 {
     using RS = RoundShape<Cfg, R>;
     constexpr int S = Cfg::N >> (RS::S0 + RS::K);
@@ -150,7 +160,7 @@ __device__ __forceinline__ void fwd_round(uint64_t (&x)[Cfg::NP][Cfg::C], const 
         constexpr int v = decltype(vc)::value;
         const int g0 = (tid * RS::SUBS + v) / S;
         static_for<0, RS::K>([&](auto sc) {
-            fwd_stage<Cfg, R, decltype(sc)::value, HALF>(x, tw, twr, q, v, g0, tid, tmul);
+            fwd_stage<Cfg, R, decltype(sc)::value, HALF, SP>(x, tw, twr, ar, v, g0, tid, tmul);
         });
     });
 }
@@ -160,19 +170,71 @@ __device__ __forceinline__ void fwd_round(uint64_t (&x)[Cfg::NP][Cfg::C], const 
 // transform's last stage (see k_ntt_inv_pair): stage s, group i uses the full
 // table's entry tmul*(N >> (s+1)) + i (N this transform's size, tmul = 2 + the
 // half's index); every round reads the natural table and no stage is the last.
-template <class Cfg, int R, int SIG, bool HALF = false>
-__device__ __forceinline__ void inv_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const LimbConst &lc,
-                                          const ulonglong2 *__restrict__ tw, int v, int blk, int tmul = 1)
+// Bounds, in multiples of q, of the folded form (values in the Shoup form follow 2^s).
+// Between rounds a register may hold at most inv_fold_limit: the next round's K stages
+// double it K - 1 times before the last X - Y, which must stay below 2^63 in magnitude,
+// and 2 * 4096 q < 2^63.
+template <class Cfg, int R, bool HALF>
+constexpr uint64_t inv_fold_limit()
+{
+    if constexpr (R + 1 < Cfg::NROUNDS)
+        return 4096u >> (RoundShape<Cfg, R + 1>::K - 1);
+    else
+        return 4096u;  // HALF: one more stage, by the caller
+}
+// register j (of a sub-transform) after a round of K stages on inputs <= b q: j = 0 was a
+// sum in every stage; else j's top bit is the stage of its last product
+constexpr uint64_t inv_reg_bound(uint64_t b, int K, int j)
+{
+    if (j == 0) return b << K;
+    int h = 0;
+    while ((j >> h) > 1) ++h;
+    return kFoldMax << (K - 1 - h);
+}
+template <class Cfg, int R, bool HALF>
+constexpr uint64_t inv_in_bound()  // inputs of round R
+{
+    if constexpr (R == 0) {
+        return 1;
+    } else {
+        uint64_t m = 0;
+        for (int j = 0; j < RoundShape<Cfg, R - 1>::KK; ++j) {
+            uint64_t b = inv_reg_bound(inv_in_bound<Cfg, R - 1, HALF>(), RoundShape<Cfg, R - 1>::K, j);
+            if (b > inv_fold_limit<Cfg, R - 1, HALF>()) b = 5;
+            if (b > m) m = b;
+        }
+        return m;
+    }
+}
+// bound of the inputs of stage SIG of round R
+template <class Cfg, int R, int SIG, bool HALF, bool SP>
+constexpr uint64_t inv_stage_bound()
+{
+    if constexpr (!SP) {
+        return 1ull << (RoundShape<Cfg, R>::S0 + SIG);
+    } else {
+        const uint64_t b = inv_in_bound<Cfg, R, HALF>() << SIG;
+        const uint64_t p = SIG > 0 ? kFoldMax << (SIG - 1) : 0;
+        return b > p ? b : p;
+    }
+}
+
+template <class Cfg, int R, int SIG, bool HALF, bool SP>
+__device__ __forceinline__ void inv_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const LimbConst &lc, const TwArith<SP> &ar,
+                                          const ulonglong2 *__restrict__ tw, int v, int blk, int tmul)
 {
     using RS = RoundShape<Cfg, R>;
     static_assert(Cfg::LOGC >= 3 && Cfg::LOGC <= 5, "first-round tables exist for LOGC = 3, 4, 5");
     constexpr int s = RS::S0 + SIG;  // global stage
     constexpr int dist = 1 << SIG;
     constexpr int ngrp = RS::KK >> (SIG + 1);
-    const uint64_t q = lc.q, nq = 0ull - q;
-    const uint64_t qs = q << s;       // bound of the stage's inputs
+    constexpr uint64_t bound = inv_stage_bound<Cfg, R, SIG, HALF, SP>();
+    static_assert(bound <= (SP ? 4096 : 8192), "differences must fit 64 bits");
+    const uint64_t q = ar.q;
+    const uint64_t qs = q * bound;    // bound of the stage's inputs
     if constexpr (s == Cfg::LOGN - 1 && !HALF) {
         // last stage: N^-1 merged into both outputs, canonical result
+        const ulonglong2 wn = make_ulonglong2(lc.ninv, lc.ninv_s), wnw = make_ulonglong2(lc.ninvw, lc.ninvw_s);
 #pragma unroll
         for (int grp = 0; grp < ngrp; ++grp) {
 #pragma unroll
@@ -181,8 +243,8 @@ __device__ __forceinline__ void inv_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const 
 #pragma unroll
                 for (int p = 0; p < Cfg::NP; ++p) {
                     const uint64_t X = x[p][j], Y = x[p][j + dist];
-                    x[p][j] = canon4(shoup_lazy(X + Y, lc.ninv, lc.ninv_s, nq), q);
-                    x[p][j + dist] = canon4(shoup_lazy(X - Y + qs, lc.ninvw, lc.ninvw_s, nq), q);
+                    x[p][j] = ar.mul_canon(X + Y, wn);
+                    x[p][j + dist] = ar.mul_canon(ar.sub(X, Y, qs), wnw);
                 }
             }
         }
@@ -202,17 +264,17 @@ __device__ __forceinline__ void inv_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const 
                 for (int p = 0; p < Cfg::NP; ++p) {
                     const uint64_t X = x[p][j], Y = x[p][j + dist];
                     x[p][j] = X + Y;
-                    const uint64_t t = shoup_lazy(X - Y + qs, w.x, w.y, nq);  // < 4q
-                    x[p][j + dist] = (s == 0) ? csub(t, 2 * q) : t;
+                    const uint64_t t = ar.mul(ar.sub(X, Y, qs), w);
+                    x[p][j + dist] = !SP && s == 0 ? csub(t, 2 * q) : t;
                 }
             }
         }
     }
 }
 
-template <class Cfg, int R, bool HALF = false>
-__device__ __forceinline__ void inv_round(uint64_t (&x)[Cfg::NP][Cfg::C], const LimbConst &lc,
-                                          const ulonglong2 *__restrict__ tw, int tid, int tmul = 1)
+template <class Cfg, int R, bool HALF, bool SP>
+__device__ __forceinline__ void inv_round(uint64_t (&x)[Cfg::NP][Cfg::C], const LimbConst &lc, const TwArith<SP> &ar,
+                                          const ulonglong2 *__restrict__ tw, int tid, int tmul)
 {
     using RS = RoundShape<Cfg, R>;
     constexpr int S = 1 << RS::S0;
@@ -220,8 +282,15 @@ __device__ __forceinline__ void inv_round(uint64_t (&x)[Cfg::NP][Cfg::C], const 
         constexpr int v = decltype(vc)::value;
         const int blk = (tid + v * Cfg::T) / S;
         static_for<0, RS::K>([&](auto sc) {
-            inv_stage<Cfg, R, decltype(sc)::value, HALF>(x, lc, tw, v, blk, tmul);
+            inv_stage<Cfg, R, decltype(sc)::value, HALF, SP>(x, lc, ar, tw, v, blk, tmul);
         });
+        if constexpr (SP && (R + 1 < Cfg::NROUNDS || HALF))
+            static_for<0, RS::KK>([&](auto jc) {
+                constexpr int j = decltype(jc)::value;
+                if constexpr (inv_reg_bound(inv_in_bound<Cfg, R, HALF>(), RS::K, j) > inv_fold_limit<Cfg, R, HALF>())
+#pragma unroll
+                    for (int p = 0; p < Cfg::NP; ++p) x[p][v * RS::KK + j] = ar.fold(x[p][v * RS::KK + j]);
+            });
     });
 }
 
@@ -303,16 +372,23 @@ __device__ __forceinline__ void inv_exchange(uint64_t (&x)[Cfg::NP][Cfg::C], uin
 // ---- whole transforms -----------------------------------------------------------
 // forward: x holds the round-0 layout (element tid + r*T) on entry and the
 // last-round layout (element tid*C + r, contiguous) on exit.
-template <class Cfg, int R = 0, bool HALF = false>
-__device__ __forceinline__ void fwd_transform(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_t *sm,
-                                              const ulonglong2 *__restrict__ tw, const ulonglong2 *__restrict__ twr,
-                                              uint64_t q, int tid, int tmul = 1)
+template <class Cfg, int R, bool HALF, bool SP>
+__device__ __forceinline__ void fwd_rounds(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_t *sm,
+                                           const ulonglong2 *__restrict__ tw, const ulonglong2 *__restrict__ twr,
+                                           const TwArith<SP> &ar, int tid, int tmul)
 {
-    fwd_round<Cfg, R, HALF>(x, tw, twr, q, tid, tmul);
+    fwd_round<Cfg, R, HALF, SP>(x, tw, twr, ar, tid, tmul);
     if constexpr (R + 1 < Cfg::NROUNDS) {
         fwd_exchange<Cfg, R>(x, sm, tid);
-        fwd_transform<Cfg, R + 1, HALF>(x, sm, tw, twr, q, tid, tmul);
+        fwd_rounds<Cfg, R + 1, HALF, SP>(x, sm, tw, twr, ar, tid, tmul);
     }
+}
+
+template <class Cfg, bool SP>
+__device__ __forceinline__ void fwd_transform(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_t *sm, const LimbConst &lc,
+                                              const TwArith<SP> &ar, int tid)
+{
+    fwd_rounds<Cfg, 0, false, SP>(x, sm, lc.tw_f, lc.tw_r, ar, tid, 1);
 }
 
 struct NoHook {
@@ -327,17 +403,30 @@ struct NoHook {
 // are its reads of the round-0 layout, element tid*C + r).  hook() runs (in every thread) right before the last
 // round, once this transform has finished with shared memory: after its last
 // exchange, or after the caller's reads when there is one round only.
-template <class Cfg, int R = 0, class Hook = NoHook, bool HALF = false>
-__device__ __forceinline__ void inv_transform(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_t *sm,
-                                              const LimbConst &lc, const ulonglong2 *__restrict__ tw,
-                                              int tid, const Hook &hook = Hook{}, int tmul = 1)
+template <class Cfg, int R, class Hook, bool HALF, bool SP>
+__device__ __forceinline__ void inv_rounds(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_t *sm, const LimbConst &lc,
+                                           const TwArith<SP> &ar, int tid, const Hook &hook, int tmul)
 {
     if constexpr (R + 1 == Cfg::NROUNDS) hook();
-    inv_round<Cfg, R, HALF>(x, lc, tw, tid, tmul);
+    inv_round<Cfg, R, HALF, SP>(x, lc, ar, lc.tw_i, tid, tmul);
     if constexpr (R + 1 < Cfg::NROUNDS) {
         inv_exchange<Cfg, R>(x, sm, tid);
-        inv_transform<Cfg, R + 1, Hook, HALF>(x, sm, lc, tw, tid, hook, tmul);
+        inv_rounds<Cfg, R + 1, Hook, HALF, SP>(x, sm, lc, ar, tid, hook, tmul);
     }
+}
+
+template <class Cfg, bool HALF = false, bool SP, class Hook = NoHook>
+__device__ __forceinline__ void inv_transform(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_t *sm, const LimbConst &lc,
+                                              const TwArith<SP> &ar, int tid, const Hook &hook = Hook{}, int tmul = 1)
+{
+    inv_rounds<Cfg, 0, Hook, HALF, SP>(x, sm, lc, ar, tid, hook, tmul);
+}
+
+// the limb's arithmetic (SP as its context's tables, hc_ctx::fold)
+template <bool SP>
+__device__ __forceinline__ TwArith<SP> tw_arith(const LimbConst &lc)
+{
+    return TwArith<SP>(lc.q, lc.special_c, lc.one_s);
 }
 
 }  // namespace hc

@@ -42,7 +42,7 @@ struct hc_plan {
     MixItem *d_items = nullptr;
     uint32_t *d_units = nullptr;
     uint32_t *d_next = nullptr;
-    uint32_t n_units = 0;
+    uint32_t n_units = 0, n_units_fold = 0;  // units of folded contexts first
     uint64_t n_products = 0, alg_bytes = 0;
     uint32_t n_launches = 0;
     uint32_t runs = 0;
@@ -112,52 +112,81 @@ hc_status run_batched(hc_plan *p, cudaStream_t s)
 {
     hc_status st = launch_conv_jobs(p->convs.data(), p->convs.size(), s, p->d_ctr, p->ctr_words);
     if (st != HC_OK) return st;
-    // every standalone product, one persistent launch
+    // every standalone product, one persistent launch per twiddle form that occurs
     if (p->n_units) {
-        HC_CUDA_TRY(cudaMemsetAsync(p->d_next, 0, sizeof(uint32_t), s));
-        st = launch_product_mixed(p->d_items, p->d_units, p->n_units, p->d_next, s);
+        HC_CUDA_TRY(cudaMemsetAsync(p->d_next, 0, 2 * sizeof(uint32_t), s));
+        st = launch_product_mixed(p->d_items, p->d_units, p->n_units_fold, p->d_next, true, s);
+        if (st != HC_OK) return st;
+        st = launch_product_mixed(p->d_items, p->d_units + p->n_units_fold, p->n_units - p->n_units_fold,
+                                  p->d_next + 1, false, s);
         if (st != HC_OK) return st;
     }
     return HC_OK;
 }
 
-// kernels one batched run launches (the fused form counts one per degree)
+// transform launches (one per twiddle form present) of consecutive groups of kMaxSegs
+// of the jobs that `take` selects; with_mac: plus one MAC launch per group
+template <class F>
+uint32_t count_groups(const hc_plan *p, F take, uint32_t transforms, bool with_mac)
+{
+    uint32_t n = 0, in_group = 0;
+    bool form[2] = {false, false};
+    auto close = [&] {
+        if (in_group) n += transforms * ((uint32_t)form[0] + (uint32_t)form[1]) + (with_mac ? 1 : 0);
+        in_group = 0;
+        form[0] = form[1] = false;
+    };
+    for (const PlanConv &c : p->convs) {
+        if (!take(c)) continue;
+        form[c.ctx->fold ? 1 : 0] = true;
+        if (++in_group == (uint32_t)kMaxSegs) close();
+    }
+    close();
+    return n;
+}
+
+// kernels one batched run launches (the fused form counts one per degree and twiddle form)
 uint32_t count_launches(const hc_plan *p)
 {
     uint32_t n = 0, fit = 0;
-    uint32_t per_n[3] = {0, 0, 0}, per_n_fit[3] = {0, 0, 0};
     bool fused[3] = {false, false, false};
-    for (int d = 0; d < 3; ++d) {
-        uint32_t cnt = 0;
+    for (uint32_t d = 0; d < 3; ++d) {
+        uint32_t cnt = 0, maxl = 0;
         const PlanConv *first = nullptr;
+        bool form[2] = {false, false};
         for (const PlanConv &c : p->convs)
-            if (c.ctx->logN == (uint32_t)(12 + d) && c.blocked) {
+            if (c.ctx->logN == 12 + d && c.blocked) {
                 if (!first) first = &c;
+                form[c.ctx->fold ? 1 : 0] = true;
+                if (c.ctx->L > maxl) maxl = c.ctx->L;
                 ++cnt;
             }
-        fused[d] = first && first->ctx->variant[KK_CONV] == 1 && cnt <= (uint32_t)kFusedMaxLayers && p->d_ctr;
-        if (fused[d]) ++n;
-        if (first && first->ctx->variant[KK_CONV] == 2 && !fused[d]) {
-            uint32_t maxl = 0;
-            for (const PlanConv &c : p->convs)
-                if (c.ctx->logN == (uint32_t)(12 + d) && c.blocked && c.ctx->L > maxl) maxl = c.ctx->L;
-            n += 3 * maxl * ((cnt + kMaxSegs - 1) / kMaxSegs);
-            fused[d] = true;  // counted here, not below
+        if (!first) continue;
+        if (first->ctx->variant[KK_CONV] == 2) {
+            for (uint32_t l = 0; l < maxl; ++l)
+                n += count_groups(p, [&](const PlanConv &c) { return c.ctx->logN == 12 + d && c.blocked && c.ctx->L > l; },
+                                  2, true);
+            fused[d] = true;
+        } else if (first->ctx->variant[KK_CONV] == 1 && cnt <= (uint32_t)kFusedMaxLayers && p->d_ctr) {
+            n += (uint32_t)form[0] + (uint32_t)form[1];
+            fused[d] = true;
         }
     }
+    auto rest = [&](const PlanConv &c) { return !(c.blocked && fused[c.ctx->logN - 12]); };
     for (const PlanConv &c : p->convs) {
-        if (c.blocked && fused[c.ctx->logN - 12]) continue;
-        ++per_n[c.ctx->logN - 12];
-        if (c.blocked) {
-            ++per_n_fit[c.ctx->logN - 12];
+        if (!rest(c)) continue;
+        if (c.blocked)
             ++fit;
-        } else {
+        else
             ++n;  // fused MAC + INTT
-        }
     }
-    for (int i = 0; i < 3; ++i) n += (per_n[i] + kMaxSegs - 1) / kMaxSegs + (per_n_fit[i] + kMaxSegs - 1) / kMaxSegs;
+    for (uint32_t d = 0; d < 3; ++d) {
+        n += count_groups(p, [&](const PlanConv &c) { return c.ctx->logN == 12 + d && rest(c); }, 1, false);
+        n += count_groups(p, [&](const PlanConv &c) { return c.ctx->logN == 12 + d && rest(c) && c.blocked; }, 1, false);
+    }
     n += (fit + kMaxSegs - 1) / kMaxSegs;
-    if (p->n_units) ++n;
+    if (p->n_units_fold) ++n;
+    if (p->n_units > p->n_units_fold) ++n;
     return n;
 }
 
@@ -361,11 +390,13 @@ hc_status launch_limb_chains(const ConvJob *jobs, size_t n, uint32_t logN, cudaS
                 NttSeg f{c.in, c.ntt, c.ctx->d_limbs, c.ctx->L, c.w->I, 0};
                 f.Lc = 1;
                 f.limb0 = l;
+                f.fold = c.ctx->fold;
                 fwd.s[fwd.n++] = f;
                 if (!c.ex) {
                     NttSeg v{c.out, c.out, c.ctx->d_limbs, c.ctx->L, c.w->O, 0};
                     v.Lc = 1;
                     v.limb0 = l;
+                    v.fold = c.ctx->fold;
                     inv.s[inv.n++] = v;
                 }
                 MacLayer ly{c.ntt, job_weights(c), c.out, c.w->G, c.w->B, c.w->Mp};
@@ -454,7 +485,8 @@ hc_status launch_conv_jobs(const ConvJob *jobs, size_t n, cudaStream_t s, uint32
                 const ConvJob &c = jobs[i];
                 if (c.ctx->logN != logN || done(c)) continue;
                 if (!first) first = c.ctx;
-                segs.s[segs.n++] = NttSeg{c.in, c.ntt, c.ctx->d_limbs, c.ctx->L, c.w->I, 0};
+                segs.s[segs.n] = NttSeg{c.in, c.ntt, c.ctx->d_limbs, c.ctx->L, c.w->I, 0};
+                segs.s[segs.n++].fold = c.ctx->fold;
             }
             if (segs.n && (segs.n == kMaxSegs || i == n)) {
                 hc_status st = launch_ntt_ct_segs(first, segs, false, s);
@@ -492,7 +524,8 @@ hc_status launch_conv_jobs(const ConvJob *jobs, size_t n, cudaStream_t s, uint32
                 const ConvJob &c = jobs[i];
                 if (c.ctx->logN != logN || !c.blocked || done(c)) continue;
                 if (!first) first = c.ctx;
-                segs.s[segs.n++] = NttSeg{c.out, c.out, c.ctx->d_limbs, c.ctx->L, c.w->O, 0};
+                segs.s[segs.n] = NttSeg{c.out, c.out, c.ctx->d_limbs, c.ctx->L, c.w->O, 0};
+                segs.s[segs.n++].fold = c.ctx->fold;
             }
             if (segs.n && (segs.n == kMaxSegs || i == n)) {
                 hc_status st = launch_ntt_ct_segs(first, segs, true, s);
@@ -554,6 +587,7 @@ hc_status hc_plan_create(const hc_work_item *items, size_t n, hc_plan **out)
     p->device = dev;
     size_t scratch_words = 0;
     std::vector<MixItem> mix;
+    std::vector<bool> mix_fold;
     for (const hc_work_item &it : its) {
         const hc_ctx *c = it.ctx;
         if (std::find(p->ctxs.begin(), p->ctxs.end(), c) == p->ctxs.end()) p->ctxs.push_back(c);
@@ -569,6 +603,7 @@ hc_status hc_plan_create(const hc_work_item *items, size_t n, hc_plan **out)
             for (size_t j = 0; j < it.n; ++j)
                 mix.push_back(MixItem{it.d_ct_in + j * ct_words(c), it.d_pt_ntt + j * (size_t)c->L * c->N,
                                       it.d_ct_out + j * ct_words(c), c->d_limbs, c->L, c->logN});
+            mix_fold.resize(mix.size(), c->fold);
             p->n_products += it.n;
             p->alg_bytes += nl * 5ull * it.n;
         }
@@ -577,15 +612,19 @@ hc_status hc_plan_create(const hc_work_item *items, size_t n, hc_plan **out)
         hc_free(p);
         return set_error(HC_ERR_INVALID_ARG, "more than 2^28 standalone products");
     }
-    // units in cost order: larger ring degree first (stable: item order within a degree)
+    // units in cost order: larger ring degree first (stable: item order within a degree),
+    // folded contexts' units before the others'
     std::vector<uint32_t> units;
-    for (uint32_t logN = 14; logN >= 12; --logN)
-        for (uint32_t j = 0; j < mix.size(); ++j) {
-            if (mix[j].logN != logN) continue;
-            const uint32_t step = mix_comps_per_unit(logN);
-            for (uint32_t limb = 0; limb < mix[j].L; ++limb)
-                for (uint32_t comp = 0; comp < 2; comp += step) units.push_back(mix_unit(j, limb, comp));
-        }
+    for (int fold = 1; fold >= 0; --fold) {
+        for (uint32_t logN = 14; logN >= 12; --logN)
+            for (uint32_t j = 0; j < mix.size(); ++j) {
+                if (mix[j].logN != logN || mix_fold[j] != (fold == 1)) continue;
+                const uint32_t step = mix_comps_per_unit(logN);
+                for (uint32_t limb = 0; limb < mix[j].L; ++limb)
+                    for (uint32_t comp = 0; comp < 2; comp += step) units.push_back(mix_unit(j, limb, comp));
+            }
+        if (fold) p->n_units_fold = (uint32_t)units.size();
+    }
     p->n_units = (uint32_t)units.size();
 
     for (const PlanConv &c : p->convs) p->ctr_words += conv_counter_bound(c.ctx, c.w);
