@@ -112,6 +112,21 @@ __device__ __forceinline__ uint64_t ld_cluster_u64(uint32_t addr)
     return v;
 }
 
+// ---- programmatic dependent launch ------------------------------------------------
+// The next kernel of the stream, if it was launched with the programmatic attribute,
+// may start once every CTA of this grid has come here (or ended) ...
+__device__ __forceinline__ void pdl_launch_dependents()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// ... and waits here until the grids before it have ended and their stores are visible.
+// Returns at once in a kernel launched without the attribute.
+__device__ __forceinline__ void pdl_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // per-thread asynchronous 8-byte global -> shared copy (completes with cp_async_wait_all)
 __device__ __forceinline__ void cp_async8(void *dst, const void *src)
 {

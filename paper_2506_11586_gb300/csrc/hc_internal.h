@@ -132,6 +132,17 @@ struct hc_weights {
 
 namespace hc {
 
+// the key switch of n rotated ciphertexts over the moduli of Q*p_sp (hc_keyswitch.cuh)
+struct KsArgs {
+    const uint64_t *a;     // [n][2][L][N]; component 1: the permuted c1, canonical
+    const uint64_t *key;   // [L][2][L+1][N], NTT domain
+    uint64_t *u;           // [n][2][L+1][N], coefficient domain
+    const LimbConst *lqp;  // [L+1]
+    uint32_t L;
+};
+template <int LOGN, bool SP>
+hc_status launch_ks_n(const KsArgs &a, size_t n, uint32_t sms, cudaStream_t s);
+
 // inverse transform with the server step's output epilogue (ExtractArgs)
 hc_status launch_inv_extract(const hc_ctx *ctx, const ExtractArgs &ex, cudaStream_t s);
 // the output slot table of w (built once per weights handle)

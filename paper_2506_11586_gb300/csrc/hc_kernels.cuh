@@ -69,17 +69,6 @@ __device__ __forceinline__ const NttSeg &find_seg(const NttSegsT<NS> &segs)
     return segs.s[i];
 }
 
-// ---------------------------------------------------------------------------
-// store the last inverse-round layout: slot r = v*KK + j holds element
-// tid + T*(v + j*SUBS)  (coalesced across the warp)
-template <class Cfg>
-__device__ __forceinline__ int inv_out_elem(int tid, int r)
-{
-    using RS = RoundShape<Cfg, Cfg::NROUNDS - 1>;
-    const int v = r >> RS::K, j = r & (RS::KK - 1);
-    return tid + Cfg::T * (v + j * RS::SUBS);
-}
-
 // after the block has filled shared memory: x[p][r] = element tid*C + r
 // (the inverse transform's round-0 layout)
 template <class Cfg>
@@ -458,7 +447,7 @@ k_ntt_inv_pf(const __grid_constant__ NttSegsT<NS> segs, uint32_t total)
     if (u < total) prefetch(u);
     for (; u < total; u += G) {
         cp_async_wait_all();
-        xsync<true>();  // the warp's copies of its block of this unit have landed
+        __syncwarp();  // the warp's copies of its block of this unit have landed
         uint32_t si, limb, poly;
         locate(u, si, limb, poly);
         const NttSeg &sg = segs.s[si];
@@ -485,7 +474,7 @@ k_ntt_inv_pf(const __grid_constant__ NttSegsT<NS> segs, uint32_t total)
 // both at position j (distributed shared memory); after a cluster barrier the
 // halves are independent and CTA c runs stages 1 .. log2 N - 1 on half c as a
 // transform of N/2 residues (HCfg) with the full table's twiddles
-// (fwd_transform's HALF mode), then stores half c canonical, as 16-byte pairs.
+// (the engine's PART mode), then stores half c canonical, as 16-byte pairs.
 // The arithmetic is the one-CTA transform's, stage by stage.
 template <class HCfg, int NS, bool SP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(HCfg::T, HCfg::MINB)
@@ -521,7 +510,7 @@ k_ntt_fwd_pair(const __grid_constant__ NttSegsT<NS> segs)
     uint64_t x[1][C];
 #pragma unroll
     for (int r = 0; r < C; ++r) x[0][r] = sm[tid + r * T];
-    fwd_rounds<HCfg, 0, true>(x, sm, lc.tw_f, nullptr, ar, tid, 2 + (int)rank);
+    fwd_rounds<HCfg, 0, 1>(x, sm, lc.tw_f, nullptr, ar, tid, 2 + (int)rank);
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < C; ++r) sm[spos<HCfg>(tid * C + r)] = ar.canon(x[0][r]);
@@ -539,8 +528,8 @@ k_ntt_fwd_pair(const __grid_constant__ NttSegsT<NS> segs)
 
 // Inverse NTT of one polynomial limb by a cluster of two CTAs: CTA c runs
 // stages 0 .. log2 N - 2 on half c (positions [c N/2, (c+1) N/2)) as a
-// transform of N/2 residues with the full table's twiddles (inv_transform's
-// HALF mode) and leaves the half in its shared memory in natural order; after a
+// transform of N/2 residues with the full table's twiddles (the engine's
+// PART mode) and leaves the half in its shared memory in natural order; after a
 // cluster barrier it computes the last stage (pairs j, j + N/2, N^-1 merged)
 // for j in [c N/4, (c+1) N/4), reading both halves through distributed shared
 // memory, and stores both outputs; a last cluster barrier keeps each CTA's
@@ -574,7 +563,7 @@ k_ntt_inv_pair(const __grid_constant__ NttSegsT<NS> segs)
     uint64_t x[1][C];
     load_round0<HCfg>(x, sm, tid);
     const TwArith<SP> ar = tw_arith<SP>(lc);
-    inv_transform<HCfg, true>(x, sm, lc, ar, tid, NoHook{}, 2 + (int)rank);
+    inv_transform<HCfg, 1>(x, sm, lc, ar, tid, NoHook{}, 2 + (int)rank);
     __syncthreads();  // the transform's last exchange has been read
 #pragma unroll
     for (int r = 0; r < C; ++r) sm[inv_out_elem<HCfg>(tid, r)] = x[0][r];

@@ -1,0 +1,7 @@
+// hc_keyswitch_n12.cu -- key-switch kernels for N = 4096 (see hc_keyswitch.cuh).
+#include "hc_keyswitch.cuh"
+
+namespace hc {
+template hc_status launch_ks_n<12, false>(const KsArgs &, size_t, uint32_t, cudaStream_t);
+template hc_status launch_ks_n<12, true>(const KsArgs &, size_t, uint32_t, cudaStream_t);
+}  // namespace hc

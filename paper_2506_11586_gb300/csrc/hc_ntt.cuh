@@ -50,12 +50,13 @@
 
 namespace hc {
 
-template <int LOGN_, int LOGC_, int NP_, int MINB_ = 1>
+template <int LOGN_, int LOGC_, int NP_, int MINB_ = 1, int GROUPS_ = 1>
 struct NttCfg {
     static constexpr int LOGN = LOGN_;
     static constexpr int LOGC = LOGC_;
     static constexpr int NP = NP_;
     static constexpr int MINB = MINB_;  // CTAs per SM the register budget is sized for
+    static constexpr int GROUPS = GROUPS_;  // groups of T threads that run transforms of their own side by side
     static constexpr int N = 1 << LOGN;
     static constexpr int C = 1 << LOGC;
     static constexpr int T = N / C;
@@ -115,11 +116,11 @@ __device__ __forceinline__ void static_for(F &&f)
 }
 
 // ---- one forward round: K Cooley-Tukey stages in registers ---------------------
-// HALF: the transform is one half of a transform of twice the size, after that
-// transform's first stage (see k_ntt_fwd_pair): local stage s, group i uses the
-// full table's entry tmul*2^s + i, tmul = 2 + the half's index; every round
-// reads the natural table.
-template <class Cfg, int R, int SIG, bool HALF, bool SP>
+// PART > 0: the transform is one of the 2^PART parts of a larger transform after that
+// transform's first PART stages (see k_ntt_fwd_pair, k_ks_switch): local stage s,
+// group i uses the full table's entry tmul*2^s + i, tmul = 2^PART + the part's
+// index; every round reads the natural table.
+template <class Cfg, int R, int SIG, int PART, bool SP>
 __device__ __forceinline__ void fwd_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const ulonglong2 *__restrict__ tw,
                                           const ulonglong2 *__restrict__ twr, const TwArith<SP> &ar, int v, int g0,
                                           int tid, int tmul)
@@ -127,7 +128,7 @@ __device__ __forceinline__ void fwd_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const 
     using RS = RoundShape<Cfg, R>;
     static_assert(Cfg::LOGC >= 3 && Cfg::LOGC <= 5, "last-round tables exist for LOGC = 3, 4, 5");
     constexpr int half = RS::KK >> (SIG + 1);
-    constexpr bool last = R == Cfg::NROUNDS - 1 && !HALF;  // every thread has its own twiddles (g0 = tid*SUBS + v)
+    constexpr bool last = R == Cfg::NROUNDS - 1 && PART == 0;  // every thread has its own twiddles (g0 = tid*SUBS + v)
 #pragma unroll
     for (int lam = 0; lam < (1 << SIG); ++lam) {
         // last round: the rearranged table, stage S0 + SIG at [2^(S0+SIG) - 2^S0],
@@ -135,7 +136,7 @@ __device__ __forceinline__ void fwd_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const 
         const ulonglong2 w =
             last ? __ldg(twr + (size_t)(3 + Cfg::LOGC - 3) * Cfg::N + ((1 << (RS::S0 + SIG)) - (1 << RS::S0)) +
                          ((v << SIG) + lam) * Cfg::T + tid)
-                 : __ldg(tw + ((HALF ? tmul : 1) << (RS::S0 + SIG)) + (g0 << SIG) + lam);
+                 : __ldg(tw + ((PART ? tmul : 1) << (RS::S0 + SIG)) + (g0 << SIG) + lam);
 #pragma unroll
         for (int jj = 0; jj < half; ++jj) {
             const int j = v * RS::KK + lam * 2 * half + jj;
@@ -150,7 +151,7 @@ __device__ __forceinline__ void fwd_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const 
     }
 }
 
-template <class Cfg, int R, bool HALF, bool SP>
+template <class Cfg, int R, int PART, bool SP>
 __device__ __forceinline__ void fwd_round(uint64_t (&x)[Cfg::NP][Cfg::C], const ulonglong2 *__restrict__ tw,
                                           const ulonglong2 *__restrict__ twr, const TwArith<SP> &ar, int tid, int tmul)
 {
@@ -160,27 +161,28 @@ __device__ __forceinline__ void fwd_round(uint64_t (&x)[Cfg::NP][Cfg::C], const 
         constexpr int v = decltype(vc)::value;
         const int g0 = (tid * RS::SUBS + v) / S;
         static_for<0, RS::K>([&](auto sc) {
-            fwd_stage<Cfg, R, decltype(sc)::value, HALF, SP>(x, tw, twr, ar, v, g0, tid, tmul);
+            fwd_stage<Cfg, R, decltype(sc)::value, PART, SP>(x, tw, twr, ar, v, g0, tid, tmul);
         });
     });
 }
 
 // ---- one inverse round: K Gentleman-Sande stages in registers ------------------
-// HALF: the transform is one half of a transform of twice the size, before that
-// transform's last stage (see k_ntt_inv_pair): stage s, group i uses the full
-// table's entry tmul*(N >> (s+1)) + i (N this transform's size, tmul = 2 + the
-// half's index); every round reads the natural table and no stage is the last.
+// PART > 0: the transform is one of the 2^PART parts of a larger transform, before
+// that transform's last PART stages (see k_ntt_inv_pair, k_ks_switch): stage s, group
+// i uses the full table's entry tmul*(N >> (s+1)) + i (N this transform's size, tmul =
+// 2^PART + the part's index); every round reads the natural table and no stage is the
+// last.
 // Bounds, in multiples of q, of the folded form (values in the Shoup form follow 2^s).
 // Between rounds a register may hold at most inv_fold_limit: the next round's K stages
 // double it K - 1 times before the last X - Y, which must stay below 2^63 in magnitude,
 // and 2 * 4096 q < 2^63.
-template <class Cfg, int R, bool HALF>
+template <class Cfg, int R, int PART>
 constexpr uint64_t inv_fold_limit()
 {
     if constexpr (R + 1 < Cfg::NROUNDS)
         return 4096u >> (RoundShape<Cfg, R + 1>::K - 1);
     else
-        return 4096u;  // HALF: one more stage, by the caller
+        return 4096u >> (PART > 0 ? PART - 1 : 0);  // PART more stages, by the caller
 }
 // register j (of a sub-transform) after a round of K stages on inputs <= b q: j = 0 was a
 // sum in every stage; else j's top bit is the stage of its last product
@@ -191,7 +193,7 @@ constexpr uint64_t inv_reg_bound(uint64_t b, int K, int j)
     while ((j >> h) > 1) ++h;
     return kFoldMax << (K - 1 - h);
 }
-template <class Cfg, int R, bool HALF>
+template <class Cfg, int R, int PART>
 constexpr uint64_t inv_in_bound()  // inputs of round R
 {
     if constexpr (R == 0) {
@@ -199,27 +201,27 @@ constexpr uint64_t inv_in_bound()  // inputs of round R
     } else {
         uint64_t m = 0;
         for (int j = 0; j < RoundShape<Cfg, R - 1>::KK; ++j) {
-            uint64_t b = inv_reg_bound(inv_in_bound<Cfg, R - 1, HALF>(), RoundShape<Cfg, R - 1>::K, j);
-            if (b > inv_fold_limit<Cfg, R - 1, HALF>()) b = 5;
+            uint64_t b = inv_reg_bound(inv_in_bound<Cfg, R - 1, PART>(), RoundShape<Cfg, R - 1>::K, j);
+            if (b > inv_fold_limit<Cfg, R - 1, PART>()) b = 5;
             if (b > m) m = b;
         }
         return m;
     }
 }
 // bound of the inputs of stage SIG of round R
-template <class Cfg, int R, int SIG, bool HALF, bool SP>
+template <class Cfg, int R, int SIG, int PART, bool SP>
 constexpr uint64_t inv_stage_bound()
 {
     if constexpr (!SP) {
         return 1ull << (RoundShape<Cfg, R>::S0 + SIG);
     } else {
-        const uint64_t b = inv_in_bound<Cfg, R, HALF>() << SIG;
+        const uint64_t b = inv_in_bound<Cfg, R, PART>() << SIG;
         const uint64_t p = SIG > 0 ? kFoldMax << (SIG - 1) : 0;
         return b > p ? b : p;
     }
 }
 
-template <class Cfg, int R, int SIG, bool HALF, bool SP>
+template <class Cfg, int R, int SIG, int PART, bool SP>
 __device__ __forceinline__ void inv_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const LimbConst &lc, const TwArith<SP> &ar,
                                           const ulonglong2 *__restrict__ tw, int v, int blk, int tmul)
 {
@@ -228,11 +230,11 @@ __device__ __forceinline__ void inv_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const 
     constexpr int s = RS::S0 + SIG;  // global stage
     constexpr int dist = 1 << SIG;
     constexpr int ngrp = RS::KK >> (SIG + 1);
-    constexpr uint64_t bound = inv_stage_bound<Cfg, R, SIG, HALF, SP>();
+    constexpr uint64_t bound = inv_stage_bound<Cfg, R, SIG, PART, SP>();
     static_assert(bound <= (SP ? 4096 : 8192), "differences must fit 64 bits");
     const uint64_t q = ar.q;
     const uint64_t qs = q * bound;    // bound of the stage's inputs
-    if constexpr (s == Cfg::LOGN - 1 && !HALF) {
+    if constexpr (s == Cfg::LOGN - 1 && PART == 0) {
         // last stage: N^-1 merged into both outputs, canonical result
         const ulonglong2 wn = make_ulonglong2(lc.ninv, lc.ninv_s), wnw = make_ulonglong2(lc.ninvw, lc.ninvw_s);
 #pragma unroll
@@ -254,9 +256,9 @@ __device__ __forceinline__ void inv_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const 
             // first round: blk is the thread index, and the rearranged table gives the
             // warp consecutive entries; later rounds share each twiddle across threads
             const ulonglong2 w =
-                R == 0 && !HALF
+                R == 0 && PART == 0
                     ? __ldg(lc.tw_r + (size_t)(Cfg::LOGC - 3) * Cfg::N + (Cfg::N - (Cfg::N >> s)) + grp * Cfg::T + blk)
-                    : __ldg(tw + (HALF ? tmul : 1) * (Cfg::N >> (s + 1)) + blk * ngrp + grp);
+                    : __ldg(tw + (PART ? tmul : 1) * (Cfg::N >> (s + 1)) + blk * ngrp + grp);
 #pragma unroll
             for (int jj = 0; jj < dist; ++jj) {
                 const int j = v * RS::KK + grp * 2 * dist + jj;
@@ -272,7 +274,7 @@ __device__ __forceinline__ void inv_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const 
     }
 }
 
-template <class Cfg, int R, bool HALF, bool SP>
+template <class Cfg, int R, int PART, bool SP>
 __device__ __forceinline__ void inv_round(uint64_t (&x)[Cfg::NP][Cfg::C], const LimbConst &lc, const TwArith<SP> &ar,
                                           const ulonglong2 *__restrict__ tw, int tid, int tmul)
 {
@@ -282,12 +284,12 @@ __device__ __forceinline__ void inv_round(uint64_t (&x)[Cfg::NP][Cfg::C], const 
         constexpr int v = decltype(vc)::value;
         const int blk = (tid + v * Cfg::T) / S;
         static_for<0, RS::K>([&](auto sc) {
-            inv_stage<Cfg, R, decltype(sc)::value, HALF, SP>(x, lc, ar, tw, v, blk, tmul);
+            inv_stage<Cfg, R, decltype(sc)::value, PART, SP>(x, lc, ar, tw, v, blk, tmul);
         });
-        if constexpr (SP && (R + 1 < Cfg::NROUNDS || HALF))
+        if constexpr (SP && (R + 1 < Cfg::NROUNDS || PART > 0))
             static_for<0, RS::KK>([&](auto jc) {
                 constexpr int j = decltype(jc)::value;
-                if constexpr (inv_reg_bound(inv_in_bound<Cfg, R, HALF>(), RS::K, j) > inv_fold_limit<Cfg, R, HALF>())
+                if constexpr (inv_reg_bound(inv_in_bound<Cfg, R, PART>(), RS::K, j) > inv_fold_limit<Cfg, R, PART>())
 #pragma unroll
                     for (int p = 0; p < Cfg::NP; ++p) x[p][v * RS::KK + j] = ar.fold(x[p][v * RS::KK + j]);
             });
@@ -319,13 +321,25 @@ constexpr bool fwd_round_local()
 {
     return Cfg::LOGN - R * Cfg::LOGC <= 5 + Cfg::LOGC;
 }
-template <bool WARP>
+// the threads of one transform: the CTA, or one of its groups (named barriers 1 ...)
+template <class Cfg>
+__device__ __forceinline__ void group_sync()
+{
+    if constexpr (Cfg::GROUPS == 1)
+        __syncthreads();
+    else  // barrier numbers as constants: a register would reserve all sixteen
+        static_for<0, Cfg::GROUPS>([](auto gc) {
+            constexpr int g = decltype(gc)::value;
+            if (threadIdx.x / Cfg::T == g) asm volatile("bar.sync %0, %1;" ::"n"(1 + g), "n"(Cfg::T) : "memory");
+        });
+}
+template <class Cfg, bool WARP>
 __device__ __forceinline__ void xsync()
 {
     if constexpr (WARP && HC_WARP_LOCAL_XCHG)
         __syncwarp();
     else
-        __syncthreads();
+        group_sync<Cfg>();
 }
 
 // ---- exchanges through shared memory ---------------------------------------------
@@ -333,14 +347,14 @@ template <class Cfg, int RFROM>
 __device__ __forceinline__ void fwd_exchange(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_t *sm, int tid)
 {
     constexpr bool local = fwd_round_local<Cfg, RFROM>() && fwd_round_local<Cfg, RFROM + 1>();
-    xsync<local>();
+    xsync<Cfg, local>();
 #pragma unroll
     for (int r = 0; r < Cfg::C; ++r) {
         const int e = spos<Cfg>(fwd_elem<Cfg, RFROM>(tid, r));
 #pragma unroll
         for (int p = 0; p < Cfg::NP; ++p) sm[p * Cfg::SW + e] = x[p][r];
     }
-    xsync<local>();
+    xsync<Cfg, local>();
 #pragma unroll
     for (int r = 0; r < Cfg::C; ++r) {
         const int e = spos<Cfg>(fwd_elem<Cfg, RFROM + 1>(tid, r));
@@ -353,14 +367,14 @@ template <class Cfg, int RFROM>
 __device__ __forceinline__ void inv_exchange(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_t *sm, int tid)
 {
     constexpr bool local = inv_round_local<Cfg, RFROM>() && inv_round_local<Cfg, RFROM + 1>();
-    xsync<local>();
+    xsync<Cfg, local>();
 #pragma unroll
     for (int r = 0; r < Cfg::C; ++r) {
         const int e = spos<Cfg>(inv_elem<Cfg, RFROM>(tid, r));
 #pragma unroll
         for (int p = 0; p < Cfg::NP; ++p) sm[p * Cfg::SW + e] = x[p][r];
     }
-    xsync<local>();
+    xsync<Cfg, local>();
 #pragma unroll
     for (int r = 0; r < Cfg::C; ++r) {
         const int e = spos<Cfg>(inv_elem<Cfg, RFROM + 1>(tid, r));
@@ -372,15 +386,15 @@ __device__ __forceinline__ void inv_exchange(uint64_t (&x)[Cfg::NP][Cfg::C], uin
 // ---- whole transforms -----------------------------------------------------------
 // forward: x holds the round-0 layout (element tid + r*T) on entry and the
 // last-round layout (element tid*C + r, contiguous) on exit.
-template <class Cfg, int R, bool HALF, bool SP>
+template <class Cfg, int R, int PART, bool SP>
 __device__ __forceinline__ void fwd_rounds(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_t *sm,
                                            const ulonglong2 *__restrict__ tw, const ulonglong2 *__restrict__ twr,
                                            const TwArith<SP> &ar, int tid, int tmul)
 {
-    fwd_round<Cfg, R, HALF, SP>(x, tw, twr, ar, tid, tmul);
+    fwd_round<Cfg, R, PART, SP>(x, tw, twr, ar, tid, tmul);
     if constexpr (R + 1 < Cfg::NROUNDS) {
         fwd_exchange<Cfg, R>(x, sm, tid);
-        fwd_rounds<Cfg, R + 1, HALF, SP>(x, sm, tw, twr, ar, tid, tmul);
+        fwd_rounds<Cfg, R + 1, PART, SP>(x, sm, tw, twr, ar, tid, tmul);
     }
 }
 
@@ -403,23 +417,33 @@ struct NoHook {
 // are its reads of the round-0 layout, element tid*C + r).  hook() runs (in every thread) right before the last
 // round, once this transform has finished with shared memory: after its last
 // exchange, or after the caller's reads when there is one round only.
-template <class Cfg, int R, class Hook, bool HALF, bool SP>
+template <class Cfg, int R, class Hook, int PART, bool SP>
 __device__ __forceinline__ void inv_rounds(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_t *sm, const LimbConst &lc,
                                            const TwArith<SP> &ar, int tid, const Hook &hook, int tmul)
 {
     if constexpr (R + 1 == Cfg::NROUNDS) hook();
-    inv_round<Cfg, R, HALF, SP>(x, lc, ar, lc.tw_i, tid, tmul);
+    inv_round<Cfg, R, PART, SP>(x, lc, ar, lc.tw_i, tid, tmul);
     if constexpr (R + 1 < Cfg::NROUNDS) {
         inv_exchange<Cfg, R>(x, sm, tid);
-        inv_rounds<Cfg, R + 1, Hook, HALF, SP>(x, sm, lc, ar, tid, hook, tmul);
+        inv_rounds<Cfg, R + 1, Hook, PART, SP>(x, sm, lc, ar, tid, hook, tmul);
     }
 }
 
-template <class Cfg, bool HALF = false, bool SP, class Hook = NoHook>
+template <class Cfg, int PART = 0, bool SP, class Hook = NoHook>
 __device__ __forceinline__ void inv_transform(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_t *sm, const LimbConst &lc,
                                               const TwArith<SP> &ar, int tid, const Hook &hook = Hook{}, int tmul = 1)
 {
-    inv_rounds<Cfg, 0, Hook, HALF, SP>(x, sm, lc, ar, tid, hook, tmul);
+    inv_rounds<Cfg, 0, Hook, PART, SP>(x, sm, lc, ar, tid, hook, tmul);
+}
+
+// the last inverse-round layout: slot r = v*KK + j holds element
+// tid + T*(v + j*SUBS)  (coalesced across the warp)
+template <class Cfg>
+__device__ __forceinline__ int inv_out_elem(int tid, int r)
+{
+    using RS = RoundShape<Cfg, Cfg::NROUNDS - 1>;
+    const int v = r >> RS::K, j = r & (RS::KK - 1);
+    return tid + Cfg::T * (v + j * RS::SUBS);
 }
 
 // the limb's arithmetic (SP as its context's tables, hc_ctx::fold)

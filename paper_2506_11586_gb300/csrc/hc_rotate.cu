@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "hc_arith.cuh"
+#include "hc_async.cuh"
 #include "hc_internal.h"
 
 // per ciphertext limb i: p_sp mod q_i, p_sp^-1 mod q_i with its Shoup companion
@@ -31,7 +32,7 @@ struct hc_galois_key {
     const hc_ctx *ctx;     // ciphertext context: q_0 .. q_{L-1}
     hc_ctx *qp;            // owned: q_0 .. q_{L-1}, p_sp
     int device;
-    uint32_t g, ginv;      // Galois element and its inverse mod 2N
+    uint32_t g;            // Galois element
     uint64_t special;
     uint64_t *d_key;       // [L][2][L+1][N], NTT domain over Q*p_sp
     ModDown *d_md;         // [L]
@@ -47,97 +48,71 @@ __device__ __forceinline__ uint64_t reduce_any(uint64_t v, const LimbConst &lc)
     return canon3(reduce_lazy(v, (uint32_t)lc.one_s, 0ull - lc.q), lc.q);
 }
 
-// The three kernels below run on 2-D grids: blockIdx.y walks the rows (one
-// polynomial limb of the output per row, the row's indices decoded once per
-// block), x the N coefficients (N a power of two, so no division per element).
-constexpr uint32_t kKsBlock = 256;
+// The elementwise half of a rotation: division by p_sp, the sums, and the permutation the
+// next key switch wants its input in.  With a = sigma(c) of the ciphertext c being rotated
+// (already permuted),
+//   w[ct][comp][i] = (comp == 0 ? a[ct][0][i] : 0) + (u_i - [u_sp]) / p_sp  (+ add) mod q_i
+// is the rotated ciphertext, and out = sigma_g(w): coefficient k goes to k*g mod 2N, negated
+// past N (g = 1: as it stands).  DIVIDE false: w = a, both components.  Reads are 16-byte
+// and coalesced; the permutation is on the stores, each word stored once, where gathering
+// it in the key switch would read every word L+1 times in 32-byte sectors.
+// 2-D grid: y walks the rows (one polynomial limb each), x the N / 2 pairs of coefficients.
+constexpr uint32_t kKsBlock = 128;
 
-// digits of sigma_g(c1): dig[ct][j][i][k] = sigma_g(c1)[j][k] mod m_i over the L+1
-// moduli m_i of Q*p_sp (gather: output coefficient k takes source k*ginv mod 2N);
-// rows (ct, j)
-__global__ void k_ks_digits(const uint64_t *__restrict__ ct, uint64_t *__restrict__ dig,
-                            const LimbConst *__restrict__ lq, const LimbConst *__restrict__ lqp, uint32_t L,
-                            uint32_t N, uint32_t ginv, uint32_t rows)
+template <bool DIVIDE>
+__global__ void __launch_bounds__(kKsBlock)
+k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *out,
+           const LimbConst *__restrict__ lq, const ModDown *__restrict__ md, uint64_t special, uint32_t L, uint32_t N,
+           uint32_t g, uint32_t rows)
 {
-    const uint32_t k = blockIdx.x * kKsBlock + threadIdx.x;
-    const uint32_t mask2 = 2 * N - 1;
-    const uint32_t src = (uint32_t)(((uint64_t)k * ginv) & mask2);
-    for (uint32_t r = blockIdx.y; r < rows; r += gridDim.y) {
-        const uint32_t c = r / L, j = r - c * L;
-        const uint64_t qj = lq[j].q;
-        const uint64_t *c1 = ct + ((size_t)(c * 2 + 1) * L + j) * N;
-        const uint64_t v = src < N ? c1[src] : negmod(c1[src - N], qj);
-        uint64_t *d = dig + (size_t)r * (L + 1) * N + k;
-        for (uint32_t i = 0; i <= L; ++i) d[(size_t)i * N] = i == j ? v : reduce_any(v, lqp[i]);
-    }
-}
-
-// u[ct][comp][i][k] = sum_j dig[ct][j][i][k] * key[j][comp][i][k] mod m_i (NTT domain);
-// rows (ct, i)
-__global__ void k_ks_mac(const uint64_t *__restrict__ dig, const uint64_t *__restrict__ key,
-                         uint64_t *__restrict__ u, const LimbConst *__restrict__ lqp, uint32_t L, uint32_t N,
-                         uint32_t rows)
-{
-    const uint32_t k = blockIdx.x * kKsBlock + threadIdx.x;
-    const uint32_t L1 = L + 1;
-    for (uint32_t r = blockIdx.y; r < rows; r += gridDim.y) {
-        const uint32_t c = r / L1, i = r - c * L1;
-        const LimbConst &lc = lqp[i];
-        const uint64_t q = lc.q, nq = 0ull - q;
-        MacAcc a0, a1;
-        mac_zero(a0);
-        mac_zero(a1);
-        for (uint32_t j = 0; j < L; ++j) {
-            const uint64_t x = dig[((size_t)(c * L + j) * L1 + i) * N + k];
-            mac_add(a0, x, key[((size_t)(j * 2) * L1 + i) * N + k]);
-            mac_add(a1, x, key[((size_t)(j * 2 + 1) * L1 + i) * N + k]);
-        }
-        const uint32_t ones = (uint32_t)lc.one_s;
-        u[((size_t)(c * 2) * L1 + i) * N + k] = mac_reduce(a0, q, nq, lc.r64, lc.r64_s, ones);
-        u[((size_t)(c * 2 + 1) * L1 + i) * N + k] = mac_reduce(a1, q, nq, lc.r64, lc.r64_s, ones);
-    }
-}
-
-// out[ct][comp][i][k] = (comp == 0 ? sigma_g(c0)[i][k] : 0) + (u_i - [u_sp]) / p_sp
-//                       (+ add[ct][comp][i][k] when add is given) mod q_i;  rows (ct, comp, i)
-// (add may be out itself: each element is read before it is written, by the same thread)
-__global__ void k_ks_mod_down(const uint64_t *__restrict__ ct, const uint64_t *__restrict__ u, uint64_t *out,
-                              const uint64_t *add, const LimbConst *__restrict__ lq,
-                              const ModDown *__restrict__ md, uint64_t special, uint32_t L, uint32_t N,
-                              uint32_t ginv, uint32_t rows)
-{
-    const uint32_t k = blockIdx.x * kKsBlock + threadIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();
+    const uint32_t k = 2 * (blockIdx.x * kKsBlock + threadIdx.x);
     const uint32_t mask2 = 2 * N - 1, L1 = L + 1;
     const uint64_t half = (special - 1) / 2;
-    const uint32_t src = (uint32_t)(((uint64_t)k * ginv) & mask2);
+    const uint32_t d0 = (uint32_t)((uint64_t)k * g) & mask2, d1 = (d0 + g) & mask2;
     for (uint32_t r = blockIdx.y; r < rows; r += gridDim.y) {
         const uint32_t cc = r / L, i = r - cc * L;  // cc = ct * 2 + comp
-        const uint32_t comp = cc & 1;
         const LimbConst &lc = lq[i];
         const uint64_t q = lc.q;
-        const uint64_t ui = u[((size_t)cc * L1 + i) * N + k];
-        const uint64_t usp = u[((size_t)cc * L1 + L) * N + k];
-        const uint64_t rsp = reduce_any(usp, lc);  // usp mod q_i
-        // the centered residue: usp - p_sp when usp > (p_sp - 1) / 2
-        const uint64_t pm = md[i].p_mod_q;
-        const uint64_t cen = usp > half ? (rsp >= pm ? rsp - pm : rsp + q - pm) : rsp;
-        const uint64_t diff = ui >= cen ? ui - cen : ui + q - cen;
-        uint64_t v = canon4(shoup_lazy(diff, md[i].pinv, md[i].pinv_s, 0ull - q), q);
-        if (comp == 0) {
-            const uint64_t *c0 = ct + ((size_t)cc * L + i) * N;
-            const uint64_t a = src < N ? c0[src] : negmod(c0[src - N], q);
-            v = csub(v + a, q);
+        auto ld2 = [](const uint64_t *p) { return __ldcg(reinterpret_cast<const ulonglong2 *>(p)); };
+        ulonglong2 v;
+        if constexpr (DIVIDE) {
+            const ulonglong2 ui = ld2(u + ((size_t)cc * L1 + i) * N + k), us = ld2(u + ((size_t)cc * L1 + L) * N + k);
+            const uint64_t pm = md[i].p_mod_q, pinv = md[i].pinv, pinv_s = md[i].pinv_s;
+            auto div = [&](uint64_t x, uint64_t usp) {
+                const uint64_t rsp = reduce_any(usp, lc);  // usp mod q_i
+                // the centered residue: usp - p_sp when usp > (p_sp - 1) / 2
+                const uint64_t cen = usp > half ? (rsp >= pm ? rsp - pm : rsp + q - pm) : rsp;
+                const uint64_t diff = x >= cen ? x - cen : x + q - cen;
+                return canon4(shoup_lazy(diff, pinv, pinv_s, 0ull - q), q);
+            };
+            if (add) {
+                const ulonglong2 b = ld2(add + (size_t)r * N + k);
+                v.x = csub(div(ui.x, us.x) + b.x, q);
+                v.y = csub(div(ui.y, us.y) + b.y, q);
+            } else {
+                v.x = div(ui.x, us.x);
+                v.y = div(ui.y, us.y);
+            }
+            if (!(cc & 1)) {
+                const ulonglong2 b = ld2(a + (size_t)r * N + k);
+                v.x = csub(v.x + b.x, q);
+                v.y = csub(v.y + b.y, q);
+            }
+        } else if (((uintptr_t)a & 15) == 0) {
+            v = ld2(a + (size_t)r * N + k);
+        } else {  // the caller's input on an odd word
+            v = make_ulonglong2(__ldcg((const unsigned long long *)a + (size_t)r * N + k), __ldcg((const unsigned long long *)a + (size_t)r * N + k + 1));
         }
-        const size_t o = (size_t)r * N + k;
-        if (add) v = csub(v + add[o], q);
-        out[o] = v;
+        uint64_t *o = out + (size_t)r * N;
+        if (g == 1 && ((uintptr_t)out & 15) == 0) {
+            *reinterpret_cast<ulonglong2 *>(o + k) = v;
+        } else {
+            o[d0 & (N - 1)] = d0 < N ? v.x : negmod(v.x, q);
+            o[d1 & (N - 1)] = d1 < N ? v.y : negmod(v.y, q);
+        }
     }
-}
-
-// grid of one of the kernels above: N / kKsBlock blocks across, rows (at most 65535) down
-dim3 ks_grid(uint32_t N, size_t rows)
-{
-    return dim3(N / kKsBlock, (unsigned)(rows < 65535 ? (rows ? rows : 1) : 65535));
 }
 
 // term list of mn outputs with one term each: output o = ciphertext o mod m times
@@ -179,41 +154,80 @@ struct Buf {
 
 bool key_ok(const hc_galois_key *k) { return k && k->magic == kMagicGaloisKey; }
 
-// out = rotate(in) (+ add, elementwise, when given; add may equal out, not in)
-hc_status rotate_into(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *in, uint64_t *out, size_t n,
-                      cudaStream_t s, const uint64_t *add = nullptr)
+// Device scratch of a chain of rotations of n ciphertexts: two permuted ciphertext buffers
+// (one read while the other is written) and the key switch's result.
+struct RotateScratch {
+    Buf mem;
+    uint64_t *a[2], *u;
+    explicit RotateScratch(cudaStream_t s) : mem(s) {}
+    hc_status alloc(const hc_ctx *ctx, size_t n, bool chain, cudaStream_t s)
+    {
+        const size_t ct = n * 2 * ctx->L * (size_t)ctx->N, ks = n * 2 * (ctx->L + 1) * (size_t)ctx->N;
+        if (n * 2 * (ctx->L + 1) > 0xffffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
+        mem.p = dev_alloc(((chain ? 2 : 1) * ct + ks) * 8, s);
+        if (!mem.p) return set_error(HC_ERR_OOM, "scratch allocation failed");
+        a[0] = (uint64_t *)mem.p;
+        a[1] = chain ? a[0] + ct : nullptr;
+        u = a[0] + (chain ? 2 : 1) * ct;
+        return HC_OK;
+    }
+};
+
+// out = sigma_g(a), or with u = sigma_g of the rotation that a, u (+ add) finish
+hc_status ks_apply(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *a, const uint64_t *u,
+                   const uint64_t *add, uint64_t *out, uint32_t g, size_t n, cudaStream_t s)
 {
-    const uint32_t L = ctx->L, N = ctx->N;
-    const size_t dig_words = n * L * (L + 1) * (size_t)N, u_words = n * 2 * (L + 1) * (size_t)N;
-    Buf dig(s), u(s);
-    dig.p = dev_alloc(dig_words * 8, s);
-    u.p = dev_alloc(u_words * 8, s);
-    if (!dig.p || !u.p) return set_error(HC_ERR_OOM, "scratch allocation failed");
-    uint64_t *dd = (uint64_t *)dig.p, *uu = (uint64_t *)u.p;
-    if ((size_t)n * 2 * (L + 1) > 0xffffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
-    {
-        ProfileScope ps("k_ks_digits", s);
-        const uint32_t rows = (uint32_t)(n * L);
-        k_ks_digits<<<ks_grid(N, rows), kKsBlock, 0, s>>>(in, dd, ctx->d_limbs, key->qp->d_limbs, L, N, key->ginv,
-                                                         rows);
-        HC_CUDA_TRY(cudaGetLastError());
+    const uint32_t rows = (uint32_t)(n * 2 * ctx->L);
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctx->N / 2 / kKsBlock, rows < 65535 ? rows : 65535);
+    cfg.blockDim = dim3(kKsBlock);
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = u ? 1 : 0;  // the first kernel of a chain follows other launches as usual
+    ProfileScope ps("k_ks_apply", s);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, u ? k_ks_apply<true> : k_ks_apply<false>, a, u, add, out,
+                                             (const LimbConst *)ctx->d_limbs, (const ModDown *)key->d_md, key->special,
+                                             ctx->L, ctx->N, g, rows);
+    return e == cudaSuccess ? HC_OK : cuda_error(e, "launch k_ks_apply");
+}
+
+// u = key switch of the permuted ciphertexts a
+hc_status ks_switch(const hc_galois_key *key, const uint64_t *a, uint64_t *u, size_t n, cudaStream_t s)
+{
+    const hc_ctx *qp = key->qp;
+    const KsArgs args{a, key->d_key, u, qp->d_limbs, qp->L - 1};
+    switch (qp->logN) {
+    case 12: return qp->fold ? launch_ks_n<12, true>(args, n, qp->sms, s) : launch_ks_n<12, false>(args, n, qp->sms, s);
+    case 13: return qp->fold ? launch_ks_n<13, true>(args, n, qp->sms, s) : launch_ks_n<13, false>(args, n, qp->sms, s);
+    case 14: return qp->fold ? launch_ks_n<14, true>(args, n, qp->sms, s) : launch_ks_n<14, false>(args, n, qp->sms, s);
+    default: return set_error(HC_ERR_UNSUPPORTED, "unsupported N = %u", qp->N);
     }
-    hc_status st = launch_ntt_fwd(key->qp, dd, dd, n * L, s);  // digits: n*L polys over Q*p_sp
+}
+
+// acc = prods[steps];  acc = rot_{key(i)}(acc) + prods[i], i = steps-1 .. 0;  out = acc
+// (prods [steps + 1][n][2][L][N]).  Each step is two launches: the key switch, then the
+// division and the addition, whose stores are already permuted for the next step.
+template <class KeyAt>
+hc_status rotate_chain(const hc_ctx *ctx, const KeyAt &key_at, const uint64_t *prods, uint32_t steps, size_t n,
+                       uint64_t *out, cudaStream_t s)
+{
+    RotateScratch sc(s);
+    hc_status st = sc.alloc(ctx, n, steps > 1, s);
     if (st != HC_OK) return st;
-    {
-        ProfileScope ps("k_ks_mac", s);
-        const uint32_t rows = (uint32_t)(n * (L + 1));
-        k_ks_mac<<<ks_grid(N, rows), kKsBlock, 0, s>>>(dd, key->d_key, uu, key->qp->d_limbs, L, N, rows);
-        HC_CUDA_TRY(cudaGetLastError());
+    const size_t step = n * 2 * ctx->L * (size_t)ctx->N;
+    const hc_galois_key *key = key_at(steps - 1);
+    st = ks_apply(ctx, key, prods + (size_t)steps * step, nullptr, nullptr, sc.a[0], key->g, n, s);
+    for (uint32_t i = steps, b = 0; st == HC_OK && i-- > 0; b ^= 1) {
+        st = ks_switch(key, sc.a[b], sc.u, n, s);
+        if (st != HC_OK) break;
+        const hc_galois_key *next = i ? key_at(i - 1) : nullptr;
+        st = ks_apply(ctx, key, sc.a[b], sc.u, prods + (size_t)i * step, i ? sc.a[b ^ 1] : out, next ? next->g : 1, n, s);
+        key = next;
     }
-    st = launch_ntt_inv(key->qp, uu, uu, 2 * n, s);
-    if (st != HC_OK) return st;
-    ProfileScope ps("k_ks_mod_down", s);
-    const uint32_t rows = (uint32_t)(n * 2 * L);
-    k_ks_mod_down<<<ks_grid(N, rows), kKsBlock, 0, s>>>(in, uu, out, add, ctx->d_limbs, key->d_md, key->special, L,
-                                                        N, key->ginv, rows);
-    HC_CUDA_TRY(cudaGetLastError());
-    return HC_OK;
+    return st;
 }
 
 }  // namespace
@@ -265,9 +279,6 @@ hc_status hc_galois_key_create(const hc_ctx *ctx, uint64_t special_prime, uint32
     k->qp = qp;
     k->device = ctx->device;
     k->g = galois_elt;
-    uint32_t ginv = 1;
-    while ((uint64_t)ginv * galois_elt % (2 * N) != 1) ginv += 2;  // odd residues form a group mod 2N
-    k->ginv = ginv;
     k->special = special_prime;
     std::vector<ModDown> md(L);
     for (uint32_t i = 0; i < L; ++i) {
@@ -315,7 +326,12 @@ hc_status hc_ct_rotate(const hc_ctx *ctx, const hc_galois_key *key, const uint64
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
     hc_status st = check_inputs(ctx, d_ct_in, 2 * n_ct, s);
     if (st != HC_OK) return st;
-    return rotate_into(ctx, key, d_ct_in, d_ct_out, n_ct, s);
+    RotateScratch sc(s);
+    st = sc.alloc(ctx, n_ct, false, s);
+    if (st == HC_OK) st = ks_apply(ctx, key, d_ct_in, nullptr, nullptr, sc.a[0], key->g, n_ct, s);
+    if (st == HC_OK) st = ks_switch(key, sc.a[0], sc.u, n_ct, s);
+    if (st == HC_OK) st = ks_apply(ctx, key, sc.a[0], sc.u, nullptr, d_ct_out, 1, n_ct, s);
+    return st;
 }
 
 hc_status hc_mac_rotate_many(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *d_ct, uint32_t m,
@@ -333,7 +349,7 @@ hc_status hc_mac_rotate_many(const hc_ctx *ctx, const hc_galois_key *key, const 
     // The products x_j * w_i do not depend on the accumulators: all m*n run first, in
     // one launch (forward NTT of the x_j once, then one MAC + inverse NTT per product);
     // the chain then only rotates and adds, all m accumulators per step, the add fused
-    // into the key switch's last kernel:
+    // into the division kernel:
     //   P_i = x * w_i (m ciphertexts);  acc = P_{n-1};  acc = rot(acc) + P_i, i = n-2 .. 0.
     const uint32_t L = ctx->L, N = ctx->N;
     const size_t ct_words = (size_t)2 * L * N, mn = (size_t)m * n;
@@ -350,16 +366,7 @@ hc_status hc_mac_rotate_many(const hc_ctx *ctx, const hc_galois_key *key, const 
     uint64_t *first = n == 1 ? d_out : prods;  // P_0 of a one-term iteration is the result
     st = launch_mac_intt(ctx, ctn, d_w_ntt, MacTerms{term_ptr, terms}, first, mn, s);
     if (st != HC_OK || n == 1) return st;
-    const size_t step = (size_t)m * ct_words;
-    const uint64_t *acc = prods + (size_t)(n - 1) * step;
-    for (uint32_t i = n - 1; i-- > 0;) {
-        uint64_t *pi = prods + (size_t)i * step;
-        uint64_t *dst = i == 0 ? d_out : pi;
-        st = rotate_into(ctx, key, acc, dst, m, s, pi);
-        if (st != HC_OK) return st;
-        acc = dst;
-    }
-    return HC_OK;
+    return rotate_chain(ctx, [&](uint32_t) { return key; }, prods, n - 1, m, d_out, s);
 }
 
 hc_status hc_mac_rotate(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *d_ct, const uint64_t *d_w_ntt,
@@ -424,7 +431,7 @@ hc_status hc_zp_conv(const hc_ctx *ctx, const hc_conv_desc *desc, const hc_galoi
     // P_{y,i} = sum_c x_c * w_{y,i,c}: forward NTT of the C inputs once, then one MAC +
     // inverse NTT launch over the kk*Y outputs (ordered [i][y], so that the chain's step
     // i rotates all Y accumulators at once); the chain then rotates and adds, the add
-    // fused into the key switch's last kernel:
+    // fused into the division's kernel:
     //   acc = P_{kk-1};  acc = rot^(step_i)(acc) + P_i, i = kk-2 .. 0.
     const size_t ct_words = (size_t)2 * L * N;
     const size_t prod_words = kk > 1 ? (size_t)n_out * ct_words : 0;
@@ -440,18 +447,9 @@ hc_status hc_zp_conv(const hc_ctx *ctx, const hc_conv_desc *desc, const hc_galoi
     HC_CUDA_TRY(cudaGetLastError());
     st = launch_mac_intt(ctx, ctn, d_w_ntt, MacTerms{term_ptr, terms}, kk == 1 ? d_ct_out : prods, n_out, s);
     if (st != HC_OK || kk == 1) return st;
-    const size_t step = (size_t)Y * ct_words;
-    const uint64_t *acc = prods + (size_t)(kk - 1) * step;
-    for (uint32_t i = kk - 1; i-- > 0;) {
-        // offsets i and i + 1 lie in one kernel row unless i + 1 starts a new one
-        const hc_galois_key *key = (i + 1) % desc->kw == 0 ? key_row : key_1;
-        uint64_t *pi = prods + (size_t)i * step;
-        uint64_t *dst = i == 0 ? d_ct_out : pi;
-        st = rotate_into(ctx, key, acc, dst, Y, s, pi);
-        if (st != HC_OK) return st;
-        acc = dst;
-    }
-    return HC_OK;
+    // offsets i and i + 1 lie in one kernel row unless i + 1 starts a new one
+    auto key_at = [&](uint32_t i) { return (i + 1) % desc->kw == 0 ? key_row : key_1; };
+    return rotate_chain(ctx, key_at, prods, kk - 1, Y, d_ct_out, s);
 }
 
 }  // extern "C"
