@@ -320,6 +320,83 @@ __device__ __forceinline__ uint64_t mac_reduce_special(const MacAcc &a, uint64_t
     return reduce128_special(lo, hi, q, c);
 }
 
+// ---- sums of products of canonical residues --------------------------------------------
+// Residues below 2^50 cut at 2^25, x = x0 + 2^25 x1: a sum of products is
+//   V = s0 + 2^25 (sm - s0 - s2) + 2^50 s2,
+//   s0 = sum x0 w0,  s2 = sum x1 w1,  sm = sum (x0 + x1)(w0 + w1)      (Karatsuba 1962),
+// three wide multiply-adds a product and, because the halves leave room, no carries:
+// s0, s2 < G 2^50 and sm < G 2^52 fit 64 bits for G < 4096 terms.  MacAcc's cut at 2^32
+// takes four and a carry chain.
+struct MacAcc25 {
+    uint64_t s0, s2, sm;
+};
+constexpr uint32_t kCut25 = (1u << 25) - 1;
+constexpr uint32_t kMacSpecialTerms = 256;  // most terms mac25_reduce_special takes
+
+__device__ __forceinline__ void mac25_zero(MacAcc25 &a) { a.s0 = a.s2 = a.sm = 0; }
+
+// x = {x0, x1} in the low and high 32 bits
+__device__ __forceinline__ uint64_t split25(uint64_t x)
+{
+    const uint32_t lo = (uint32_t)x, hi = (uint32_t)(x >> 32);
+    return (uint64_t)(__funnelshift_r(lo, hi, 25)) << 32 | (lo & kCut25);
+}
+
+// a += b * c, in place: by halves, because the compiler gives mad.wide.u32's result a
+// fresh register pair and moves it back
+__device__ __forceinline__ void mad_wide(uint64_t &a, uint32_t b, uint32_t c)
+{
+    asm("{\n\t"
+        ".reg .u32 l, h;\n\t"
+        "mov.b64 {l, h}, %0;\n\t"
+        "mad.lo.cc.u32 l, %1, %2, l;\n\t"
+        "madc.hi.u32 h, %1, %2, h;\n\t"
+        "mov.b64 %0, {l, h};\n\t"
+        "}"
+        : "+l"(a)
+        : "r"(b), "r"(c));
+}
+
+// both operands split
+__device__ __forceinline__ void mac25_add(MacAcc25 &a, uint64_t x, uint32_t xs, uint64_t w, uint32_t ws)
+{
+    mad_wide(a.s0, (uint32_t)x, (uint32_t)w);
+    mad_wide(a.s2, (uint32_t)(x >> 32), (uint32_t)(w >> 32));
+    mad_wide(a.sm, xs, ws);
+}
+
+// canonical V mod q, any q < 2^50
+__device__ __forceinline__ uint64_t mac25_reduce(const MacAcc25 &a, uint64_t q, uint64_t nq, uint64_t r64,
+                                                 uint64_t r64_s, uint32_t ones)
+{
+    const uint64_t s1 = a.sm - a.s0 - a.s2;
+    const uint64_t t = a.s0 + (s1 << 25), lo = t + (a.s2 << 50);
+    const uint64_t hi = (s1 >> 39) + (a.s2 >> 14) + (t < a.s0) + (lo < t);
+    return reduce128(lo, hi, q, nq, r64, r64_s, ones);
+}
+
+// canonical V mod q for q = 2^50 - c, 0 < c < 2^22, at most 256 terms.  s0 < 2^58 and
+// s1 < 2^59; with s1 = l + 2^25 h, V = s0 + 2^25 l + c (s2 + h) (mod q), and with
+// s2 + h = tl + 2^28 th, th < 2^31, and u = c th = ul + 2^22 uh, 2^28 u = 2^28 ul + c uh:
+//   V = s0 + 2^25 l + c tl + 2^28 ul + c uh < 2^58 + 2^54,
+// whose fold at 2^50 leaves less than 2^50 + 2^31 < 2 q.  p25, p28: powers of two the
+// compiler does not see through, for the shifted sums on the multiply pipe.
+__device__ __forceinline__ uint64_t mac25_reduce_special(const MacAcc25 &a, uint64_t q, uint32_t c, uint32_t p25,
+                                                         uint32_t p28)
+{
+    const uint64_t s1 = a.sm - a.s0 - a.s2;
+    const uint64_t t = a.s2 + (s1 >> 25);
+    const uint64_t u = (uint64_t)(uint32_t)(t >> 28) * c;
+    uint64_t r = a.s0;
+    mad_wide(r, (uint32_t)s1 & kCut25, p25);
+    mad_wide(r, (uint32_t)t & ((1u << 28) - 1), c);
+    mad_wide(r, (uint32_t)u & ((1u << 22) - 1), p28);
+    mad_wide(r, (uint32_t)(u >> 22), c);
+    uint64_t v = r & ((1ull << 50) - 1);
+    mad_wide(v, (uint32_t)(r >> 50), c);
+    return csub(v, q);
+}
+
 // canonical x*w mod q of a lazy forward-transform value x and a residue w < q.  The
 // folded form's x (|x| < 2^60) is first brought into [0, 2^53), so that x*w < 2^104.
 __device__ __forceinline__ uint64_t mul_slot(const TwArith<false> &ar, uint64_t x, uint64_t w, uint64_t r64,

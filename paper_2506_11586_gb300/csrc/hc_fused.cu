@@ -80,14 +80,11 @@ k_conv_fused(const __grid_constant__ FusedLayersT<NS> P, uint32_t *cnt, int *err
 {
     constexpr int T = Cfg::T, N = Cfg::N;
     extern __shared__ __align__(16) uint64_t dsm[];
-    __shared__ __align__(8) uint64_t bars[1 + kMacStages];
+    __shared__ __align__(8) uint64_t bars[kMacBars];
     __shared__ uint32_t s_task;
     __shared__ int s_ok;
     const int tid = threadIdx.x;
-    if (tid == 0) {
-        for (int i = 0; i < 1 + kMacStages; ++i) mbar_init(&bars[i], 1);
-        mbar_fence_init();
-    }
+    if (tid == 0) mac_bars_init<T>(bars);
     MacRing ring{0, 0};
     uint32_t *next = cnt;
     for (;;) {
@@ -203,7 +200,7 @@ hc_status fused_for_ns(const ConvJob *jobs, size_t n, uint32_t *ctr, cudaStream_
         idx[P.n] = &jobs[i];
         FusedLayer &ly = P.s[P.n++];
         const ConvJob &j = jobs[i];
-        ly.mac = make_mac_seg(j.ctx, j.ntt, job_weights(j), j.out, j.w->G, j.w->B, j.w->Mp, kMacKC);
+        ly.mac = make_mac_seg(j.ctx, j.ntt, job_weights(j), j.out, j.w->G, j.w->B, j.w->Mp, true);
         ly.in = j.in;
         ly.I = j.w->I;
         ly.O = j.w->O;
@@ -261,7 +258,7 @@ size_t fused_counter_words(const ConvJob *jobs, size_t n, uint32_t logN)
     for (size_t i = 0; i < n; ++i) {
         if (jobs[i].ctx->logN != logN || !jobs[i].blocked) continue;
         const MacSeg sg = make_mac_seg(jobs[i].ctx, jobs[i].ntt, job_weights(jobs[i]), jobs[i].out, jobs[i].w->G,
-                                       jobs[i].w->B, jobs[i].w->Mp, kMacKC);
+                                       jobs[i].w->B, jobs[i].w->Mp, true);
         words += jobs[i].ctx->L * (1 + sg.groups);
     }
     return words ? words + 1 : 0;

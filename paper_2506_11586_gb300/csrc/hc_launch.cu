@@ -60,16 +60,19 @@ int default_variant(int kind, uint32_t logn)
 }
 
 // ---------------------------------------------------------------------------
-// Blocked convolution MAC (the task in hc_mac.cuh): one task per CTA; the
+// Blocked convolution MAC (the tasks in hc_mac.cuh): one task per CTA; the
 // CTAs of a launch cover the (chunk, limb, channel group) tasks of every
-// segment (layer) of the table.
+// segment (layer) of the table.  Layers of one or two blocks stream their weights
+// (chunks of kMacStreamKC slots; figures at mac_stream_task), the others, whose rows share
+// a weight four times and more, take them through the shared-memory ring.
 constexpr int kMacThreads = 256;
+constexpr uint32_t kMacStreamKC = 128;
 
-template <int KC, int NS>
-__global__ void __launch_bounds__(kMacThreads)
+template <int NS>
+__global__ void __launch_bounds__(kMacThreads, 4)
 k_mac_conv(const __grid_constant__ MacSegsT<NS> segs, int *err)
 {
-    __shared__ __align__(8) uint64_t bars[1 + kMacStages];
+    __shared__ __align__(8) uint64_t bars[kMacBars];
     extern __shared__ __align__(16) uint64_t dsm[];
     uint32_t si = 0;
     while (si + 1 < segs.n && blockIdx.x >= segs.s[si + 1].cta_begin) ++si;
@@ -79,18 +82,23 @@ k_mac_conv(const __grid_constant__ MacSegsT<NS> segs, int *err)
     const uint32_t lc = seg_limbs(sg);
     const uint32_t limb = sg.limb0 + rest % lc;
     const uint32_t m0 = (rest / lc) * sg.MB, m1 = min(sg.M, m0 + sg.MB);
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < 1 + kMacStages; ++i) mbar_init(&bars[i], 1);
-        mbar_fence_init();
+    if (sg.KC == kMacStreamKC) {
+        if (sg.B == 1)
+            mac_stream_task<kMacStreamKC, kMacThreads, 2, 2>(sg, chunk, limb, m0, m1, dsm);
+        else
+            mac_stream_task<kMacStreamKC, kMacThreads, 1, 4>(sg, chunk, limb, m0, m1, dsm);
+        return;
     }
+    if (threadIdx.x == 0) mac_bars_init<kMacThreads>(bars);
     __syncthreads();
     MacRing ring{0, 0};
-    mac_task<KC, kMacThreads>(sg, chunk, limb, m0, m1, dsm, bars, ring, err);
+    mac_task<kMacKC, kMacThreads>(sg, chunk, limb, m0, m1, dsm, bars, ring, err);
 }
 
-// launch variants of the blocked MAC: (slots per chunk, weight rows per stage)
-constexpr uint32_t kMacVariantKC[kNumVariants] = {64, 64, 64};
-constexpr uint32_t kMacStageRows[kNumVariants] = {8, 16, 32};
+// launch variants of the blocked MAC: weight rows per ring stage, waves of CTAs of a
+// streamed layer
+constexpr uint32_t kMacStageRows[kNumVariants] = {16, 32, 64};
+constexpr uint32_t kMacStreamWaves[kNumVariants] = {4, 2, 8};
 constexpr size_t kMacSmemCap = 200 * 1024;
 
 static size_t mac_smem(uint32_t G, uint32_t B, uint32_t MS, uint32_t kc)
@@ -102,20 +110,20 @@ static size_t mac_smem(uint32_t G, uint32_t B, uint32_t MS, uint32_t kc)
 static uint32_t mac_stage_channels(uint32_t G, uint32_t B, uint32_t M, int variant, uint32_t kc)
 {
     uint32_t ms = kMacStageRows[variant] / G;
-    if (ms < 1) ms = 1;
+    ms = ms < 2 ? 2 : ms & ~1u;  // the tiles take channel pairs
     if (ms > M) ms = M;
-    while (ms > 1 && mac_smem(G, B, ms, kc) > kMacSmemCap / 2) --ms;  // keep two CTAs per SM where possible
+    while (ms > 2 && mac_smem(G, B, ms, kc) > kMacSmemCap / 2) ms -= ms & 1 ? 1 : 2;  // two CTAs per SM where possible
+    if (mac_smem(G, B, ms, kc) > kMacSmemCap) ms = 1;
     return ms;
 }
 
 // fill the launch geometry of one segment: enough CTAs for about `waves` waves of
-// the layer's full work (all L limbs)
+// the layer's full work (all L limbs).  ring: through the weight ring whatever B is.
 MacSeg make_mac_seg(const hc_ctx *ctx, const uint64_t *x, const uint64_t *w, uint64_t *y, uint32_t G, uint32_t B,
-                    uint32_t M, uint32_t kc, uint32_t waves)
+                    uint32_t M, bool ring, uint32_t waves)
 {
     int v = ctx->variant[KK_MACB];
-    if (v >= kNumVariants) v = 1;  // shapes the tensor-core MAC does not take: stages of 16 rows
-    if (kc == 0) kc = kMacVariantKC[v];
+    if (v >= kNumVariants) v = 1;  // shapes the tensor-core MAC does not take: stages of 32 rows
     MacSeg sg{};
     sg.X = x;
     sg.W = w;
@@ -126,28 +134,31 @@ MacSeg make_mac_seg(const hc_ctx *ctx, const uint64_t *x, const uint64_t *w, uin
     sg.G = G;
     sg.B = B;
     sg.M = M;
-    sg.KC = kc;
-    sg.MS = mac_stage_channels(G, B, M, v, kc);
+    // streamed: the input chunk alone, at least four CTAs per SM
+    const bool stream = !ring && B <= 2 && mac_smem(G, B, 0, kMacStreamKC) <= kMacSmemCap / 4;
+    const uint32_t kc = sg.KC = stream ? kMacStreamKC : kMacKC;
+    sg.MS = stream ? 0 : mac_stage_channels(G, B, M, v, kc);
     const size_t smem = mac_smem(G, B, sg.MS, kc);
     const uint32_t per_sm = (uint32_t)(kMacSmemCap / smem) < 4 ? (uint32_t)(kMacSmemCap / smem) : 4;
     sg.chunks = ctx->N / kc;
-    const uint32_t target = ctx->sms * (per_sm ? per_sm : 1) * waves;
+    const uint32_t target = ctx->sms * (per_sm ? per_sm : 1) * (stream ? waves * kMacStreamWaves[v] / 4 : waves);
     const uint32_t want = (target + sg.chunks * ctx->L - 1) / (sg.chunks * ctx->L);
     const uint32_t groups = want < 1 ? 1 : (want > M ? M : want);
     sg.MB = (M + groups - 1) / groups;
-    sg.MB = (sg.MB + sg.MS - 1) / sg.MS * sg.MS;  // whole stages per CTA
+    const uint32_t unit = stream ? kMacThreads / kMacStreamKC * (B == 1 ? 2 : 1) : sg.MS;
+    sg.MB = (sg.MB + unit - 1) / unit * unit;  // whole stages, or whole passes of the row groups, per CTA
     sg.groups = (M + sg.MB - 1) / sg.MB;
     return sg;
 }
 
-template <int KC, int NS>
-static hc_status run_mac_segs_kc(MacSegsT<NS> &segs, size_t smem, int *err, cudaStream_t s)
+template <int NS>
+static hc_status run_mac_segs(MacSegsT<NS> &segs, size_t smem, int *err, cudaStream_t s)
 {
     static std::atomic<uint32_t> attr_done{0};
     int dev = 0;
     cudaGetDevice(&dev);
     if (!(attr_done.load() & (1u << (dev & 31)))) {
-        cudaError_t e = cudaFuncSetAttribute(k_mac_conv<KC, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(k_mac_conv<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kMacSmemCap);
         if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute(k_mac_conv)");
         attr_done.fetch_or(1u << (dev & 31));
@@ -159,16 +170,8 @@ static hc_status run_mac_segs_kc(MacSegsT<NS> &segs, size_t smem, int *err, cuda
     }
     if (begin == 0) return HC_OK;
     ProfileScope ps("k_mac_conv", s);
-    k_mac_conv<KC, NS><<<begin, kMacThreads, smem, s>>>(segs, err);
+    k_mac_conv<NS><<<begin, kMacThreads, smem, s>>>(segs, err);
     return after_launch_status("k_mac_conv");
-}
-
-// every segment of one launch has the same chunk width
-template <int NS>
-static hc_status run_mac_segs(MacSegsT<NS> &segs, size_t smem, int *err, cudaStream_t s)
-{
-    return segs.s[0].KC == 32 ? run_mac_segs_kc<32, NS>(segs, smem, err, s)
-                              : run_mac_segs_kc<64, NS>(segs, smem, err, s);
 }
 
 size_t mac_seg_smem(const MacSeg &sg)
@@ -216,8 +219,6 @@ hc_status launch_mac_conv_layers(const hc_ctx *const *ctxs, const MacLayer *laye
         size_t smem = 0;
         const size_t r1 = r0 + kMaxSegs < rest.size() ? r0 + kMaxSegs : rest.size();
         const size_t i0 = rest[r0];
-        const int v0 = ctxs[i0]->variant[KK_MACB];
-        const uint32_t kc = kMacVariantKC[v0 < kNumVariants ? v0 : 1];  // one chunk width per launch
         for (size_t ri = r0; ri < r1; ++ri) {
             const size_t i = rest[ri];
             const MacLayer &ly = layers[i];
@@ -225,7 +226,7 @@ hc_status launch_mac_conv_layers(const hc_ctx *const *ctxs, const MacLayer *laye
             // one limb's launch of the per-limb chains runs beside the other limbs' MACs:
             // fewer, longer CTAs (each loads its input chunk once for more channels)
             // measured faster there (2 waves: 0.240 vs 0.250 ms on the 56x56x64 layer)
-            segs.s[segs.n] = make_mac_seg(ctxs[i], ly.x, ly.w, ly.y, ly.G, ly.B, ly.M, kc, ly.Lc ? 2 : 4);
+            segs.s[segs.n] = make_mac_seg(ctxs[i], ly.x, ly.w, ly.y, ly.G, ly.B, ly.M, false, ly.Lc ? 2 : 4);
             segs.s[segs.n].Lc = ly.Lc;
             segs.s[segs.n].limb0 = ly.limb0;
             const size_t sm = mac_seg_smem(segs.s[segs.n++]);
