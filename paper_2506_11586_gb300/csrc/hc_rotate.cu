@@ -56,6 +56,7 @@ __device__ __forceinline__ uint64_t reduce_any(uint64_t v, const LimbConst &lc)
 // past N (g = 1: as it stands).  DIVIDE false: w = a, both components.  Reads are 16-byte
 // and coalesced; the permutation is on the stores, each word stored once, where gathering
 // it in the key switch would read every word L+1 times in 32-byte sectors.
+// a's ciphertexts lie a_ct ciphertexts apart, add's add_ct.
 // 2-D grid: y walks the rows (one polynomial limb each), x the N / 2 pairs of coefficients.
 constexpr uint32_t kKsBlock = 128;
 
@@ -63,7 +64,7 @@ template <bool DIVIDE>
 __global__ void __launch_bounds__(kKsBlock)
 k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *out,
            const LimbConst *__restrict__ lq, const ModDown *__restrict__ md, uint64_t special, uint32_t L, uint32_t N,
-           uint32_t g, uint32_t rows)
+           uint32_t g, uint32_t rows, uint32_t a_ct, uint32_t add_ct)
 {
     pdl_launch_dependents();
     pdl_wait();
@@ -75,6 +76,7 @@ k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *
         const uint32_t cc = r / L, i = r - cc * L;  // cc = ct * 2 + comp
         const LimbConst &lc = lq[i];
         const uint64_t q = lc.q;
+        auto strided = [&](uint32_t by) { return ((size_t)(cc >> 1) * by * 2 * L + (cc & 1) * L + i) * N + k; };
         auto ld2 = [](const uint64_t *p) { return __ldcg(reinterpret_cast<const ulonglong2 *>(p)); };
         ulonglong2 v;
         if constexpr (DIVIDE) {
@@ -88,7 +90,7 @@ k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *
                 return canon4(shoup_lazy(diff, pinv, pinv_s, 0ull - q), q);
             };
             if (add) {
-                const ulonglong2 b = ld2(add + (size_t)r * N + k);
+                const ulonglong2 b = ld2(add + strided(add_ct));
                 v.x = csub(div(ui.x, us.x) + b.x, q);
                 v.y = csub(div(ui.y, us.y) + b.y, q);
             } else {
@@ -101,9 +103,10 @@ k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *
                 v.y = csub(v.y + b.y, q);
             }
         } else if (((uintptr_t)a & 15) == 0) {
-            v = ld2(a + (size_t)r * N + k);
+            v = ld2(a + strided(a_ct));
         } else {  // the caller's input on an odd word
-            v = make_ulonglong2(__ldcg((const unsigned long long *)a + (size_t)r * N + k), __ldcg((const unsigned long long *)a + (size_t)r * N + k + 1));
+            const unsigned long long *p = (const unsigned long long *)a + strided(a_ct);
+            v = make_ulonglong2(__ldcg(p), __ldcg(p + 1));
         }
         uint64_t *o = out + (size_t)r * N;
         if (g == 1 && ((uintptr_t)out & 15) == 0) {
@@ -115,31 +118,17 @@ k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *
     }
 }
 
-// term list of mn outputs with one term each: output o = ciphertext o mod m times
-// plaintext o / m
-__global__ void k_outer_terms(uint32_t *term_ptr, uint32_t *terms, uint32_t m, uint32_t mn)
-{
-    for (uint32_t o = blockIdx.x * blockDim.x + threadIdx.x; o <= mn; o += gridDim.x * blockDim.x) {
-        term_ptr[o] = o;
-        if (o < mn) {
-            terms[2 * o] = o % m;
-            terms[2 * o + 1] = o / m;
-        }
-    }
-}
-
-// term list of a Z_P convolution's products: output o = i*Y + y (kernel offset i,
-// output ciphertext y) sums the C terms (input c, weight plaintext (y*kk + i)*C + c)
-__global__ void k_conv_terms(uint32_t *term_ptr, uint32_t *terms, uint32_t Y, uint32_t kk, uint32_t C,
-                             uint32_t n_out)
+// term list of a batch of products: output o = m*B + b sums the G terms (input g*B + b,
+// plaintext m*G + g)
+__global__ void k_product_terms(uint32_t *term_ptr, uint32_t *terms, uint32_t G, uint32_t B, uint32_t n_out)
 {
     for (uint32_t o = blockIdx.x * blockDim.x + threadIdx.x; o <= n_out; o += gridDim.x * blockDim.x) {
-        term_ptr[o] = o * C;
+        term_ptr[o] = o * G;
         if (o < n_out) {
-            const uint32_t i = o / Y, y = o % Y;
-            for (uint32_t c = 0; c < C; ++c) {
-                terms[2 * (o * C + c)] = c;
-                terms[2 * (o * C + c) + 1] = (y * kk + i) * C + c;
+            const uint32_t m = o / B, b = o % B;
+            for (uint32_t g = 0; g < G; ++g) {
+                terms[2 * (o * G + g)] = g * B + b;
+                terms[2 * (o * G + g) + 1] = m * G + g;
             }
         }
     }
@@ -173,9 +162,33 @@ struct RotateScratch {
     }
 };
 
+// out[m*B + b] = INTT(sum_g x[g*B + b] . w[m*G + g]), x forward transformed.  The blocked
+// MAC reads each weight once and sums at the multiply pipe's rate, and the inverse
+// transforms run as a launch of their own; k_mac_intt, which reads its terms word by word
+// from each output's CTA, stays for what does not fit or is not aligned.  Measured on GB300,
+// N = 8192, L = 3: a layer of 288 outputs of 16 terms and its rotations 1011 us with
+// k_mac_intt (376 us of it), 929 so; an iteration of 16 products 281 and 271 us.
+hc_status products(const hc_ctx *ctx, const uint64_t *x, const uint64_t *w, uint32_t G, uint32_t B, uint32_t M,
+                   uint64_t *out, cudaStream_t s)
+{
+    const uint32_t n_out = M * B;
+    if (mac_conv_fits(G, B) && (((uintptr_t)w | (uintptr_t)out) & 15) == 0) {
+        const hc_status st = launch_mac_conv(ctx, x, w, out, G, B, M, s);
+        return st == HC_OK ? launch_ntt_inv_ct(ctx, out, out, n_out, s) : st;
+    }
+    Buf tmp(s);
+    tmp.p = dev_alloc(((size_t)n_out + 1 + 2 * (size_t)n_out * G) * sizeof(uint32_t), s);
+    if (!tmp.p) return set_error(HC_ERR_OOM, "scratch allocation failed");
+    uint32_t *term_ptr = (uint32_t *)tmp.p, *terms = term_ptr + n_out + 1;
+    k_product_terms<<<(n_out + 256) / 256, 256, 0, s>>>(term_ptr, terms, G, B, n_out);
+    HC_CUDA_TRY(cudaGetLastError());
+    return launch_mac_intt(ctx, x, w, MacTerms{term_ptr, terms}, out, n_out, s);
+}
+
 // out = sigma_g(a), or with u = sigma_g of the rotation that a, u (+ add) finish
 hc_status ks_apply(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *a, const uint64_t *u,
-                   const uint64_t *add, uint64_t *out, uint32_t g, size_t n, cudaStream_t s)
+                   const uint64_t *add, uint64_t *out, uint32_t g, size_t n, cudaStream_t s, uint32_t a_ct = 1,
+                   uint32_t add_ct = 1)
 {
     const uint32_t rows = (uint32_t)(n * 2 * ctx->L);
     cudaLaunchAttribute attr{};
@@ -190,7 +203,7 @@ hc_status ks_apply(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *
     ProfileScope ps("k_ks_apply", s);
     const cudaError_t e = cudaLaunchKernelEx(&cfg, u ? k_ks_apply<true> : k_ks_apply<false>, a, u, add, out,
                                              (const LimbConst *)ctx->d_limbs, (const ModDown *)key->d_md, key->special,
-                                             ctx->L, ctx->N, g, rows);
+                                             ctx->L, ctx->N, g, rows, a_ct, add_ct);
     return e == cudaSuccess ? HC_OK : cuda_error(e, "launch k_ks_apply");
 }
 
@@ -207,24 +220,24 @@ hc_status ks_switch(const hc_galois_key *key, const uint64_t *a, uint64_t *u, si
     }
 }
 
-// acc = prods[steps];  acc = rot_{key(i)}(acc) + prods[i], i = steps-1 .. 0;  out = acc
-// (prods [steps + 1][n][2][L][N]).  Each step is two launches: the key switch, then the
+// acc = P_steps;  acc = rot_{key(i)}(acc) + P_i, i = steps-1 .. 0;  out = acc.  Ciphertext j
+// of P_i is prods[i*by_i + j*by_j].  Each step is two launches: the key switch, then the
 // division and the addition, whose stores are already permuted for the next step.
 template <class KeyAt>
-hc_status rotate_chain(const hc_ctx *ctx, const KeyAt &key_at, const uint64_t *prods, uint32_t steps, size_t n,
-                       uint64_t *out, cudaStream_t s)
+hc_status rotate_chain(const hc_ctx *ctx, const KeyAt &key_at, const uint64_t *prods, uint32_t by_i,
+                       uint32_t by_j, uint32_t steps, size_t n, uint64_t *out, cudaStream_t s)
 {
     RotateScratch sc(s);
     hc_status st = sc.alloc(ctx, n, steps > 1, s);
     if (st != HC_OK) return st;
-    const size_t step = n * 2 * ctx->L * (size_t)ctx->N;
+    const size_t step = (size_t)by_i * 2 * ctx->L * ctx->N;
     const hc_galois_key *key = key_at(steps - 1);
-    st = ks_apply(ctx, key, prods + (size_t)steps * step, nullptr, nullptr, sc.a[0], key->g, n, s);
+    st = ks_apply(ctx, key, prods + steps * step, nullptr, nullptr, sc.a[0], key->g, n, s, by_j);
     for (uint32_t i = steps, b = 0; st == HC_OK && i-- > 0; b ^= 1) {
         st = ks_switch(key, sc.a[b], sc.u, n, s);
         if (st != HC_OK) break;
         const hc_galois_key *next = i ? key_at(i - 1) : nullptr;
-        st = ks_apply(ctx, key, sc.a[b], sc.u, prods + (size_t)i * step, i ? sc.a[b ^ 1] : out, next ? next->g : 1, n, s);
+        st = ks_apply(ctx, key, sc.a[b], sc.u, prods + i * step, i ? sc.a[b ^ 1] : out, next ? next->g : 1, n, s, 1, by_j);
         key = next;
     }
     return st;
@@ -347,26 +360,22 @@ hc_status hc_mac_rotate_many(const hc_ctx *ctx, const hc_galois_key *key, const 
     if (st == HC_OK) st = check_inputs(ctx, d_w_ntt, n, s);
     if (st != HC_OK) return st;
     // The products x_j * w_i do not depend on the accumulators: all m*n run first, in
-    // one launch (forward NTT of the x_j once, then one MAC + inverse NTT per product);
+    // one batch (forward NTT of the x_j once, then the products and their inverse NTTs);
     // the chain then only rotates and adds, all m accumulators per step, the add fused
     // into the division kernel:
     //   P_i = x * w_i (m ciphertexts);  acc = P_{n-1};  acc = rot(acc) + P_i, i = n-2 .. 0.
     const uint32_t L = ctx->L, N = ctx->N;
     const size_t ct_words = (size_t)2 * L * N, mn = (size_t)m * n;
-    const size_t term_words = (3 * mn + 1 + 1) / 2;  // mn + 1 offsets and 2mn indices, as uint32
     Buf tmp(s);
-    tmp.p = dev_alloc(((mn + m) * ct_words + term_words) * 8, s);
+    tmp.p = dev_alloc((mn + m) * ct_words * 8, s);
     if (!tmp.p) return set_error(HC_ERR_OOM, "scratch allocation failed");
     uint64_t *ctn = (uint64_t *)tmp.p, *prods = ctn + (size_t)m * ct_words;  // prods [n][m][2][L][N]
-    uint32_t *term_ptr = reinterpret_cast<uint32_t *>(prods + mn * ct_words), *terms = term_ptr + mn + 1;
     st = launch_ntt_fwd(ctx, d_ct, ctn, (size_t)2 * m, s);
     if (st != HC_OK) return st;
-    k_outer_terms<<<(unsigned)((mn + 256) / 256), 256, 0, s>>>(term_ptr, terms, m, (uint32_t)mn);
-    HC_CUDA_TRY(cudaGetLastError());
     uint64_t *first = n == 1 ? d_out : prods;  // P_0 of a one-term iteration is the result
-    st = launch_mac_intt(ctx, ctn, d_w_ntt, MacTerms{term_ptr, terms}, first, mn, s);
+    st = products(ctx, ctn, d_w_ntt, 1, m, n, first, s);
     if (st != HC_OK || n == 1) return st;
-    return rotate_chain(ctx, [&](uint32_t) { return key; }, prods, n - 1, m, d_out, s);
+    return rotate_chain(ctx, [&](uint32_t) { return key; }, prods, m, 1, n - 1, m, d_out, s);
 }
 
 hc_status hc_mac_rotate(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *d_ct, const uint64_t *d_w_ntt,
@@ -428,28 +437,24 @@ hc_status hc_zp_conv(const hc_ctx *ctx, const hc_conv_desc *desc, const hc_galoi
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
     st = check_inputs(ctx, d_ct_in, (size_t)2 * C, s);
     if (st != HC_OK) return st;
-    // P_{y,i} = sum_c x_c * w_{y,i,c}: forward NTT of the C inputs once, then one MAC +
-    // inverse NTT launch over the kk*Y outputs (ordered [i][y], so that the chain's step
-    // i rotates all Y accumulators at once); the chain then rotates and adds, the add
+    // P_{y,i} = sum_c x_c * w_{y,i,c}: forward NTT of the C inputs once, then the products
+    // and inverse NTTs of the kk*Y outputs (ordered [y][i], as the weights); the chain then
+    // rotates and adds, all Y accumulators per step, the add
     // fused into the division's kernel:
     //   acc = P_{kk-1};  acc = rot^(step_i)(acc) + P_i, i = kk-2 .. 0.
     const size_t ct_words = (size_t)2 * L * N;
     const size_t prod_words = kk > 1 ? (size_t)n_out * ct_words : 0;
-    const size_t term_words = ((size_t)n_out + 1 + 2 * (size_t)n_out * C + 1) / 2;
     Buf tmp(s);
-    tmp.p = dev_alloc(((size_t)C * ct_words + prod_words + term_words) * 8, s);
+    tmp.p = dev_alloc(((size_t)C * ct_words + prod_words) * 8, s);
     if (!tmp.p) return set_error(HC_ERR_OOM, "scratch allocation failed");
-    uint64_t *ctn = (uint64_t *)tmp.p, *prods = ctn + (size_t)C * ct_words;
-    uint32_t *term_ptr = reinterpret_cast<uint32_t *>(prods + prod_words), *terms = term_ptr + n_out + 1;
+    uint64_t *ctn = (uint64_t *)tmp.p, *prods = ctn + (size_t)C * ct_words;  // prods [Y][kk][2][L][N]
     st = launch_ntt_fwd(ctx, d_ct_in, ctn, (size_t)2 * C, s);
     if (st != HC_OK) return st;
-    k_conv_terms<<<(n_out + 256) / 256, 256, 0, s>>>(term_ptr, terms, Y, kk, C, n_out);
-    HC_CUDA_TRY(cudaGetLastError());
-    st = launch_mac_intt(ctx, ctn, d_w_ntt, MacTerms{term_ptr, terms}, kk == 1 ? d_ct_out : prods, n_out, s);
+    st = products(ctx, ctn, d_w_ntt, C, 1, n_out, kk == 1 ? d_ct_out : prods, s);
     if (st != HC_OK || kk == 1) return st;
     // offsets i and i + 1 lie in one kernel row unless i + 1 starts a new one
     auto key_at = [&](uint32_t i) { return (i + 1) % desc->kw == 0 ? key_row : key_1; };
-    return rotate_chain(ctx, key_at, prods, kk - 1, Y, d_ct_out, s);
+    return rotate_chain(ctx, key_at, prods, 1, kk, kk - 1, Y, d_ct_out, s);
 }
 
 }  // extern "C"
