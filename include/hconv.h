@@ -98,15 +98,17 @@ hc_status hc_selftest_wait_timeout(const hc_ctx *ctx, uint32_t limit, void *cuda
  * ciphertexts, 5 inverse NTT of whole ciphertexts, 6 blocked convolution MAC,
  * 7 convolution launch form.  variant (0..2) selects, for kinds 0-5, the radix
  * per register round, the polynomials per CTA and the CTAs per SM for the
- * context's N; variant 2 of the inverse kinds is a persistent kernel (TMA-fed
- * at N = 4096, prefetching into its exchange buffer at N >= 8192; with fewer
- * limbs than resident CTAs there, one cluster of two CTAs per limb) and
- * variant 2 of the forward kinds at N >= 8192 transforms each limb with a
- * cluster of two CTAs.  For kind 6 variants 0..2 select the weight rows per pipeline
- * stage (about 8, 16 or 32) of the integer MAC, and variant 3 the tensor-core MAC
+ * context's N.  Variant 2 of the inverse kinds at N = 4096 and 16384, and
+ * variant 1 at N = 8192, are persistent kernels (TMA-fed at N = 4096,
+ * prefetching into their exchange buffer above); variant 1 of the forward
+ * kinds at N >= 8192 transforms each limb with a cluster of two CTAs.  In the
+ * default variants of kinds 0, 1, 3, 4 and 5, launches of few limbs run each
+ * limb split over a cluster of eight CTAs.  For kind 6 variants 0..2 select the weight rows per pipeline
+ * stage (about 16, 32 or 64; of layers with one or two spatial blocks, which do
+ * not stage their weights, the CTAs per SM) of the integer MAC, and variant 3 the tensor-core MAC
  * (residues split into 8-bit limbs, exact f16 products summed in fp32 by
  * tcgen05 MMAs, recombined and reduced mod q; layers with G <= 8 channel groups
- * and 2B <= 8 rows per group, the others keep the integer MAC with 16-row
+ * and 2B <= 8 rows per group, the others keep the integer MAC with 32-row
  * stages).  For kind 7: three launches per ring degree (forward NTTs,
  * MACs, inverse NTTs: variant 0), one persistent launch whose CTAs take the
  * layers' NTT, MAC and INTT tasks in order and wait on per-limb completion

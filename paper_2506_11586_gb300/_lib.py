@@ -475,7 +475,8 @@ def hc_conv_server_step_sparse(ctx, w, ct_in, share, mask, c1_out, c0_slots, str
 def hc_ctpt_mac(ctx, ct, pt_ntt, slots, out, stream=None):
     sl = np.ascontiguousarray(slots, dtype=np.uint32)
     n_out = _npolys(ctx, out) // 2
-    _check(lib().hc_ctpt_mac(ctx.ptr, _dptr(ct), _dptr(pt_ntt), C.c_void_p(sl.ctypes.data), sl.size,
+    # (sl.ctypes builds a view object, as long as the call's other marshalling together)
+    _check(lib().hc_ctpt_mac(ctx.ptr, _dptr(ct), _dptr(pt_ntt), C.c_void_p(sl.__array_interface__["data"][0]), sl.size,
                              _dptr(out), n_out, _stream(stream)))
 
 

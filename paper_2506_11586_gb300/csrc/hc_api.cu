@@ -1063,6 +1063,7 @@ hc_status hc_ctpt_mac(const hc_ctx *ctx, const uint64_t *d_ct, const uint64_t *d
     if (single) {
         // every slot has at most one product: fused NTT -> product -> INTT per product
         if (n < n_out) HC_CUDA_TRY(cudaMemsetAsync(d_out, 0, n_out * ct_words * sizeof(uint64_t), s));
+        if (product_split(ctx, n)) return launch_product_split(ctx, d_ct, d_pt_ntt, h_slot, d_out, n, false, s);
         ScratchGuard idx(s);
         idx.p = dev_alloc(n * sizeof(uint32_t), s);
         if (!idx.p) return set_error(HC_ERR_OOM, "slot list allocation failed");

@@ -134,6 +134,40 @@ __device__ __forceinline__ void pdl_wait()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// first statement of a kernel that is launched as a programmatic dependent and may have
+// dependents of its own
+__device__ __forceinline__ void pdl_begin()
+{
+    pdl_launch_dependents();
+    pdl_wait();
+}
+
+// loads of what an earlier launch, or another CTA of this one, may have written: through
+// L2, and never on the read-only path, whose loads the compiler may move above the wait
+__device__ __forceinline__ uint64_t ld_data(const uint64_t *p)
+{
+    return __ldcg((const unsigned long long *)p);
+}
+__device__ __forceinline__ ulonglong2 ld_data(const ulonglong2 *p) { return __ldcg(p); }
+
+// host: launch kern, as the programmatic dependent of the launch before it if asked to
+template <class... P, class... A>
+cudaError_t launch_programmatic(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool dependent,
+                                A &&...args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 // per-thread asynchronous 8-byte global -> shared copy (completes with cp_async_wait_all)
 __device__ __forceinline__ void cp_async8(void *dst, const void *src)
 {

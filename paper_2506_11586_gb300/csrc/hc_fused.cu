@@ -137,7 +137,7 @@ k_conv_fused(const __grid_constant__ FusedLayersT<NS> P, uint32_t *cnt, int *err
                 break;
             }
             uint64_t *y = sg.Y + ((size_t)poly * L + limb) * N;
-            inv_task<Cfg, SP, true>(dsm, y, y, 0, sg.limbs[limb], tid);
+            inv_task<Cfg, SP>(dsm, y, y, 0, sg.limbs[limb], tid);
         }
     }
 }

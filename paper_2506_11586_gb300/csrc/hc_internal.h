@@ -140,6 +140,13 @@ struct KsArgs {
     const LimbConst *lqp;  // [L+1]
     uint32_t L;
 };
+// standalone products over clusters (hc_split.cuh): at most kSplitMaxProducts of them, few
+// enough for its shapes; slots: each product's output, on the host (null: j)
+constexpr uint32_t kSplitMaxProducts = 256;
+bool product_split(const hc_ctx *ctx, size_t n);
+hc_status launch_product_split(const hc_ctx *ctx, const uint64_t *ct, const uint64_t *pt_ntt, const uint32_t *slots,
+                               uint64_t *out, size_t n, bool accumulate, cudaStream_t s);
+
 template <int LOGN, bool SP>
 hc_status launch_ks_n(const KsArgs &a, size_t n, uint32_t sms, cudaStream_t s);
 
@@ -384,6 +391,20 @@ hc_status launch_product_mixed(const MixItem *items, const uint32_t *units, uint
 // transform kinds that take a segment table (pseudo-kinds, variant of FWDCT / INVCT),
 // and the inverse transform with the server step's output epilogue (variant of INV)
 constexpr int KK_FWDCT_SEGS = 100, KK_INVCT_SEGS = 101, KK_INV_EXTRACT = 102;
+// and the standalone products over clusters (one shape)
+constexpr int KK_PROD_SPLIT = 103;
+// Most units (polynomial limbs; limbs of a product) that run split over clusters of eight.
+// Measured on GB300, us, split / one CTA (pair) per unit, both as programmatic dependents:
+//   forward  N = 4096:  32 limbs 4.9 / 6.3   76: 7.1 / 6.3
+//            N = 8192:  24: 6.7 / 11   96: 9.7 / 18   153: 15.9 / 18   240: 21 / 20
+//            N = 16384: 32: 10 / 21    64: 16 / 21    96: 19 / 21
+//   inverse  N = 8192:  24: 7.6 / 11   96: 11 / 18    192: 18.9 / 18.8
+//            N = 16384: 32: 12 / 21    64: 18 / 21    96: 22 / 21
+//   product  N = 4096:  16 limbs 8.3 / 23   48: 10.5 / 23   64: 17 / 16
+//            N = 8192:  12: 11.5 / 41  72: 29 / 41    96: 37 / 41
+//            N = 16384: 4: 14.7 / 45   32: 43 / 46    64: 72 / 46
+constexpr uint32_t split_units_ntt(uint32_t logn, uint32_t sms) { return sms * (logn == 12 ? 3 : logn == 13 ? 8 : 4) / 8; }
+constexpr uint32_t split_units_product(uint32_t logn, uint32_t sms) { return sms * (logn == 12 ? 3 : logn == 13 ? 4 : 2) / 8; }
 
 
 // arguments of one launch of a kernel family (unused fields ignored)
@@ -397,6 +418,7 @@ struct LaunchArgs {
     size_t n;
     bool accumulate;
     const ExtractArgs *ex;
+    const uint32_t *h_slots;  // split products: output of each, host memory, or null
 };
 template <int LOGN, bool SP>
 hc_status launch_n(const hc_ctx *ctx, int kind, int variant, const LaunchArgs &a, cudaStream_t s);

@@ -18,6 +18,7 @@
 
 #include "hc_async.cuh"
 #include "hc_ntt.cuh"
+#include "hc_split.cuh"
 
 namespace hc {
 
@@ -27,18 +28,25 @@ namespace hc {
 // sized for MINB resident CTAs.  Single-polynomial kernels (KK_FWD, KK_INV)
 // use NP = 1 with the same C and MINB.
 template <int LOGN, int V> struct Variant;
-template <> struct Variant<12, 0> { static constexpr int LOGC = 3, NP = 2, MINB = 1; };   // T 512, 128 regs
-template <> struct Variant<12, 1> { static constexpr int LOGC = 4, NP = 2, MINB = 2; };   // T 256, 128 regs
+template <> struct Variant<12, 0> { static constexpr int LOGC = 4, NP = 1, MINB = 3; };   // T 256, 80 regs
+template <> struct Variant<12, 1> { static constexpr int LOGC = 3, NP = 2, MINB = 1; };   // T 512, 128 regs
 template <> struct Variant<12, 2> { static constexpr int LOGC = 3, NP = 1, MINB = 2; };   // T 512, 64 regs
 template <> struct Variant<13, 0> { static constexpr int LOGC = 4, NP = 2, MINB = 1; };   // T 512, 128 regs
-template <> struct Variant<13, 1> { static constexpr int LOGC = 5, NP = 1, MINB = 2; };   // T 256, 128 regs
-template <> struct Variant<13, 2> { static constexpr int LOGC = 3, NP = 1, MINB = 1; };   // T 1024, 64 regs
+template <> struct Variant<13, 1> { static constexpr int LOGC = 3, NP = 1, MINB = 1; };   // T 1024, 64 regs
+template <> struct Variant<13, 2> { static constexpr int LOGC = 5, NP = 1, MINB = 2; };   // T 256, 128 regs
 template <> struct Variant<14, 0> { static constexpr int LOGC = 5, NP = 1, MINB = 1; };   // T 512, 128 regs
 template <> struct Variant<14, 1> { static constexpr int LOGC = 4, NP = 1, MINB = 1; };   // T 1024, 64 regs
 template <> struct Variant<14, 2> { static constexpr int LOGC = 5, NP = 1, MINB = 1; };   // (same as 0)
+// The transforms of a new context (variant 0 at N = 4096, 2 above) take the shapes with the
+// most independent CTAs an SM can hold, launched as programmatic dependents.  Measured on
+// GB300 with such launches, us, forward / inverse of that many limbs:
+//   N = 4096:  4096 limbs  109 / 112 (variant 0), 154 / 171 (1), 115 / 117 (2)
+//   N = 8192:  1536 limbs  98 / 93 (2), 112 / 120 (0), 104 / 101 (1: clusters / persistent)
+//              300 limbs   20 / 19 (2), 21 / 22 (0), 23 / 26 (1)
+//   N = 16384: 2048 limbs  295 / 275 (2: one CTA / persistent), 311 (clusters) / 288 (0)
 
-// shapes of the persistent inverse NTTs (inverse kinds, variant 2): TMA-fed
-// double buffer at N = 4096, prefetching into the exchange buffer above
+// shapes of the persistent inverse NTTs: TMA-fed double buffer at N = 4096 (inverse kinds,
+// variant 2), prefetching into the exchange buffer at N = 8192 (variant 1) and 16384 (2)
 template <int LOGN> struct InvTma;
 template <> struct InvTma<12> { using Cfg = NttCfg<12, 4, 1, 2>; };  // T 256, 2 x 32 KB
 template <int LOGN> struct InvPf;
@@ -47,14 +55,14 @@ template <> struct InvPf<14> { using Cfg = NttCfg<14, 5, 1, 1>; };   // T 512, 1
 template <int LOGN, int V>
 constexpr bool use_inv_tma = V == 2 && LOGN == 12;
 template <int LOGN, int V>
-constexpr bool use_inv_pf = V == 2 && LOGN >= 13;
-// the forward kinds' variant 2 at N >= 8192: one limb per cluster of two CTAs,
+constexpr bool use_inv_pf = (V == 1 && LOGN == 13) || (V == 2 && LOGN == 14);
+// the forward kinds' variant 1 at N >= 8192: one limb per cluster of two CTAs,
 // each running a half transform of this shape
 template <int LOGN> struct FwdPair;
 template <> struct FwdPair<13> { using Cfg = NttCfg<12, 4, 1, 3>; };  // T 256, 32 KB, three clusters' CTAs per SM
 template <> struct FwdPair<14> { using Cfg = NttCfg<13, 5, 1, 2>; };  // T 256, 64 KB
 template <int LOGN, int V>
-constexpr bool use_fwd_pair = V == 2 && LOGN >= 13;
+constexpr bool use_fwd_pair = V == 1 && LOGN >= 13;
 
 
 template <int LOGN, int V, bool SINGLE>
@@ -94,7 +102,7 @@ __device__ __forceinline__ void fwd_task(uint64_t *sm, const uint64_t *src, uint
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
 #pragma unroll
-        for (int r = 0; r < C; ++r) x[p][r] = __ldg(src + p * pstride + tid + r * T);
+        for (int r = 0; r < C; ++r) x[p][r] = ld_data(src + p * pstride + tid + r * T);
     }
     const TwArith<SP> ar = tw_arith<SP>(lc);
     fwd_transform<Cfg>(x, sm, lc, ar, tid);
@@ -119,10 +127,8 @@ __device__ __forceinline__ void fwd_task(uint64_t *sm, const uint64_t *src, uint
     }
 }
 
-// Inverse NTT of NP polynomials (src + p*pstride) into dst (may equal src).
-// COHERENT loads bypass the non-coherent read-only path, for inputs written
-// earlier by other CTAs of the same launch.  One CTA task.
-template <class Cfg, bool SP, bool COHERENT = false>
+// Inverse NTT of NP polynomials (src + p*pstride) into dst (may equal src).  One CTA task.
+template <class Cfg, bool SP>
 __device__ __forceinline__ void inv_core(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_t *sm, const uint64_t *src,
                                          size_t pstride, const LimbConst &lc, int tid)
 {
@@ -135,7 +141,7 @@ __device__ __forceinline__ void inv_core(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_
 #pragma unroll
         for (int r = 0; r < C / 2; ++r) {
             const int e = 2 * (tid + r * Cfg::T);
-            const ulonglong2 v = COHERENT ? __ldcg(s2 + tid + r * Cfg::T) : __ldg(s2 + tid + r * Cfg::T);
+            const ulonglong2 v = ld_data(s2 + tid + r * Cfg::T);
             sm[p * N + spos<Cfg>(e)] = v.x;
             sm[p * N + spos<Cfg>(e + 1)] = v.y;
         }
@@ -144,13 +150,13 @@ __device__ __forceinline__ void inv_core(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_
     inv_transform<Cfg>(x, sm, lc, tw_arith<SP>(lc), tid);
 }
 
-template <class Cfg, bool SP, bool COHERENT = false>
+template <class Cfg, bool SP>
 __device__ __forceinline__ void inv_task(uint64_t *sm, const uint64_t *src, uint64_t *dst, size_t pstride,
                                          const LimbConst &lc, int tid)
 {
     constexpr int NP = Cfg::NP, C = Cfg::C;
     uint64_t x[NP][C];
-    inv_core<Cfg, SP, COHERENT>(x, sm, src, pstride, lc, tid);
+    inv_core<Cfg, SP>(x, sm, src, pstride, lc, tid);
     // the transform's results are read by no later kernel of the layer: streaming
     // stores (evict first), so that L2 keeps what the next kernels read
 #pragma unroll
@@ -166,6 +172,7 @@ __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
 k_ntt_fwd(const __grid_constant__ NttSegsT<NS> segs)
 {
     extern __shared__ uint64_t sm[];
+    pdl_begin();
     const NttSeg &sg = find_seg(segs);
     const uint32_t local = blockIdx.x - sg.cta_begin;
     const uint32_t limb = sg.limb0 + local / sg.n_groups, grp = local % sg.n_groups;
@@ -178,6 +185,7 @@ __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
 k_ntt_inv(const __grid_constant__ NttSegsT<NS> segs)
 {
     extern __shared__ uint64_t sm[];
+    pdl_begin();
     const NttSeg &sg = find_seg(segs);
     const uint32_t local = blockIdx.x - sg.cta_begin;
     const uint32_t limb = sg.limb0 + local / sg.n_groups, grp = local % sg.n_groups;
@@ -195,6 +203,7 @@ k_ntt_inv_extract(const __grid_constant__ ExtractArgs ex, const LimbConst *__res
 {
     static_assert(Cfg::NP == 1, "one polynomial per CTA");
     extern __shared__ uint64_t sm[];
+    pdl_begin();
     const int tid = threadIdx.x;
     const uint32_t per_limb = ex.O * 2;
     const uint32_t limb = ex.limb0 + blockIdx.x / per_limb, pi = blockIdx.x % per_limb;
@@ -243,6 +252,7 @@ k_mac_intt(const uint64_t *__restrict__ ct_ntt, const uint64_t *__restrict__ pt_
            uint32_t n_groups)
 {
     extern __shared__ uint64_t sm[];
+    pdl_begin();
     constexpr int NP = Cfg::NP, C = Cfg::C, N = Cfg::N;
     constexpr int CPG = 2 / NP;  // component groups per output
     const int tid = threadIdx.x;
@@ -252,7 +262,7 @@ k_mac_intt(const uint64_t *__restrict__ ct_ntt, const uint64_t *__restrict__ pt_
     const LimbConst &lc = limbs[limb];
     const uint64_t q = lc.q, nq = 0ull - q, r64 = lc.r64, r64_s = lc.r64_s;
     const uint32_t ones = (uint32_t)lc.one_s;
-    const uint32_t t0 = __ldg(term_ptr + o), t1 = __ldg(term_ptr + o + 1);
+    const uint32_t t0 = __ldcg(term_ptr + o), t1 = __ldcg(term_ptr + o + 1);
 
     // MAC in the coalesced pair layout: thread tid owns residue pairs
     // e = 2*(tid + r*T), so each warp-wide 16-byte load covers 512 contiguous
@@ -269,11 +279,11 @@ k_mac_intt(const uint64_t *__restrict__ ct_ntt, const uint64_t *__restrict__ pt_
         }
 #pragma unroll 4
         for (uint32_t t = t0; t < t1; ++t) {
-            const uint32_t ci = __ldg(terms + 2 * t), pi = __ldg(terms + 2 * t + 1);
-            const ulonglong2 w = __ldg(reinterpret_cast<const ulonglong2 *>(pt_ntt + (size_t)pi * L * N + limb_off + e));
+            const uint32_t ci = __ldcg(terms + 2 * t), pi = __ldcg(terms + 2 * t + 1);
+            const ulonglong2 w = ld_data(reinterpret_cast<const ulonglong2 *>(pt_ntt + (size_t)pi * L * N + limb_off + e));
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
-                const ulonglong2 xv = __ldg(reinterpret_cast<const ulonglong2 *>(
+                const ulonglong2 xv = ld_data(reinterpret_cast<const ulonglong2 *>(
                     ct_ntt + ((size_t)ci * 2 + comp0 + p) * L * N + limb_off + e));
                 mac_add(acc[p][0], xv.x, w.x);
                 mac_add(acc[p][1], xv.y, w.y);
@@ -331,6 +341,7 @@ k_ntt_inv_tma(const __grid_constant__ NttSegsT<NS> segs, uint32_t total, int *er
 {
     static_assert(Cfg::NP == 1, "one polynomial per unit");
     extern __shared__ __align__(16) uint64_t sm[];  // [2][N]
+    pdl_begin();
     __shared__ __align__(8) uint64_t bars[2];
     constexpr int C = Cfg::C, N = Cfg::N, V = C / 2;
     constexpr uint32_t BYTES = N * sizeof(uint64_t);
@@ -416,6 +427,7 @@ k_ntt_inv_pf(const __grid_constant__ NttSegsT<NS> segs, uint32_t total)
 {
     static_assert(Cfg::NP == 1, "one polynomial per unit");
     extern __shared__ __align__(16) uint64_t sm[];  // [N], swizzled
+    pdl_begin();
     constexpr int C = Cfg::C, N = Cfg::N, T = Cfg::T;
     const int tid = threadIdx.x;
     const uint32_t G = gridDim.x;
@@ -482,6 +494,7 @@ k_ntt_fwd_pair(const __grid_constant__ NttSegsT<NS> segs)
 {
     static_assert(HCfg::NP == 1, "one polynomial per cluster");
     extern __shared__ __align__(16) uint64_t sm[];  // [N/2]: the half, then the exchanges
+    pdl_begin();
     constexpr int C = HCfg::C, T = HCfg::T, NH = HCfg::N;
     const int tid = threadIdx.x;
     const uint32_t rank = cluster_rank();
@@ -496,18 +509,23 @@ k_ntt_fwd_pair(const __grid_constant__ NttSegsT<NS> segs)
     const LimbConst &lc = sg.limbs[limb];
     const ulonglong2 w = __ldg(lc.tw_f + 1);
     const uint32_t to0 = cluster_map(sm, 0), to1 = cluster_map(sm, 1);
-    cluster_sync();  // both CTAs are running before either writes into the other
     const TwArith<SP> ar = tw_arith<SP>(lc);
+    uint64_t x[1][C];  // pairs r: residues r and r + C/2; every load before the first store
 #pragma unroll
     for (int r = 0; r < C / 2; ++r) {
         const uint32_t j = rank * (NH / 2) + tid + r * T;  // < NH
-        const uint64_t X = __ldg(src + j), Y = __ldg(src + j + NH);
-        const uint64_t t = ar.mul(Y, w);
+        x[0][r] = ld_data(src + j);
+        x[0][r + C / 2] = ld_data(src + j + NH);
+    }
+    cluster_sync();  // both CTAs are running before either writes into the other
+#pragma unroll
+    for (int r = 0; r < C / 2; ++r) {
+        const uint32_t j = rank * (NH / 2) + tid + r * T;
+        const uint64_t X = x[0][r], t = ar.mul(x[0][r + C / 2], w);
         st_cluster_u64(to0 + j * 8, X + t);
         st_cluster_u64(to1 + j * 8, ar.sub(X, t));
     }
     cluster_sync();  // the halves are complete; no remote access after this point
-    uint64_t x[1][C];
 #pragma unroll
     for (int r = 0; r < C; ++r) x[0][r] = sm[tid + r * T];
     fwd_rounds<HCfg, 0, 1>(x, sm, lc.tw_f, nullptr, ar, tid, 2 + (int)rank);
@@ -524,62 +542,6 @@ k_ntt_fwd_pair(const __grid_constant__ NttSegsT<NS> segs)
         v.y = sm[spos<HCfg>(e + 1)];
         d[tid + r * T] = v;
     }
-}
-
-// Inverse NTT of one polynomial limb by a cluster of two CTAs: CTA c runs
-// stages 0 .. log2 N - 2 on half c (positions [c N/2, (c+1) N/2)) as a
-// transform of N/2 residues with the full table's twiddles (the engine's
-// PART mode) and leaves the half in its shared memory in natural order; after a
-// cluster barrier it computes the last stage (pairs j, j + N/2, N^-1 merged)
-// for j in [c N/4, (c+1) N/4), reading both halves through distributed shared
-// memory, and stores both outputs; a last cluster barrier keeps each CTA's
-// shared memory alive until its peer has read it.
-template <class HCfg, int NS, bool SP>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(HCfg::T, HCfg::MINB)
-k_ntt_inv_pair(const __grid_constant__ NttSegsT<NS> segs)
-{
-    static_assert(HCfg::NP == 1, "one polynomial per cluster");
-    extern __shared__ __align__(16) uint64_t sm[];  // [N/2]
-    constexpr int C = HCfg::C, T = HCfg::T, NH = HCfg::N;
-    const int tid = threadIdx.x;
-    const uint32_t rank = cluster_rank();
-    const uint32_t unit = blockIdx.x >> 1;
-    uint32_t si = 0;
-    while (si + 1 < segs.n && unit >= segs.s[si + 1].cta_begin) ++si;
-    const NttSeg &sg = segs.s[si];
-    const uint32_t local = unit - sg.cta_begin;
-    const uint32_t limb = sg.limb0 + local / sg.n_groups, poly = local % sg.n_groups;
-    const size_t off = ((size_t)poly * sg.L + limb) * (2 * (size_t)NH);
-    const LimbConst &lc = sg.limbs[limb];
-    // half c: coalesced 16-byte loads into shared memory, then the round-0 layout
-    const ulonglong2 *s2 = reinterpret_cast<const ulonglong2 *>(sg.in + off + (size_t)rank * NH);
-#pragma unroll
-    for (int r = 0; r < C / 2; ++r) {
-        const int e = 2 * (tid + r * T);
-        const ulonglong2 v = __ldg(s2 + tid + r * T);
-        sm[spos<HCfg>(e)] = v.x;
-        sm[spos<HCfg>(e + 1)] = v.y;
-    }
-    uint64_t x[1][C];
-    load_round0<HCfg>(x, sm, tid);
-    const TwArith<SP> ar = tw_arith<SP>(lc);
-    inv_transform<HCfg, 1>(x, sm, lc, ar, tid, NoHook{}, 2 + (int)rank);
-    __syncthreads();  // the transform's last exchange has been read
-#pragma unroll
-    for (int r = 0; r < C; ++r) sm[inv_out_elem<HCfg>(tid, r)] = x[0][r];
-    const uint32_t from0 = cluster_map(sm, 0), from1 = cluster_map(sm, 1);
-    cluster_sync();  // both halves are in shared memory
-    const uint64_t qs = ar.q * HCfg::N;  // bound of the last stage's inputs (Shoup)
-    const ulonglong2 wn = make_ulonglong2(lc.ninv, lc.ninv_s), wnw = make_ulonglong2(lc.ninvw, lc.ninvw_s);
-    uint64_t *out = sg.out + off;
-#pragma unroll
-    for (int r = 0; r < C / 2; ++r) {
-        const uint32_t j = rank * (NH / 2) + tid + r * T;  // < NH
-        const uint64_t X = ld_cluster_u64(from0 + j * 8), Y = ld_cluster_u64(from1 + j * 8);
-        out[j] = ar.mul_canon(X + Y, wn);
-        out[j + NH] = ar.mul_canon(ar.sub(X, Y, qs), wnw);
-    }
-    cluster_sync();  // the peer has read this CTA's half
 }
 
 // ---------------------------------------------------------------------------
@@ -601,14 +563,14 @@ __device__ __forceinline__ void product_task(uint64_t *sm, const uint64_t *__res
     for (int p = 0; p < NP; ++p) {
         const uint64_t *src = ct + ((size_t)(comp0 + p) * L + limb) * N;
 #pragma unroll
-        for (int r = 0; r < C; ++r) x[p][r] = __ldg(src + tid + r * T);
+        for (int r = 0; r < C; ++r) x[p][r] = ld_data(src + tid + r * T);
     }
     const TwArith<SP> ar = tw_arith<SP>(lc);
     fwd_transform<Cfg>(x, sm, lc, ar, tid);  // lazy values, contiguous layout
     const ulonglong2 *wp = reinterpret_cast<const ulonglong2 *>(pt + (size_t)limb * N + tid * C);
 #pragma unroll
     for (int r = 0; r < C / 2; ++r) {
-        const ulonglong2 w = __ldg(wp + r);
+        const ulonglong2 w = ld_data(wp + r);
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
             x[p][2 * r] = mul_slot(ar, x[p][2 * r], w.x, lc.r64, lc.r64_s);
@@ -640,12 +602,13 @@ k_product(const uint64_t *__restrict__ ct, const uint64_t *__restrict__ pt_ntt,
           uint32_t L, uint32_t n_groups, int accumulate)
 {
     extern __shared__ uint64_t sm[];
+    pdl_begin();
     constexpr int CPG = 2 / Cfg::NP;
     constexpr size_t N = Cfg::N;
     const uint32_t limb = blockIdx.x / n_groups, grp = blockIdx.x % n_groups;
     const uint32_t j = grp / CPG;
     const uint32_t comp0 = (grp % CPG) * Cfg::NP;
-    const uint32_t oj = out_index ? __ldg(out_index + j) : j;
+    const uint32_t oj = out_index ? __ldcg(out_index + j) : j;
     product_task<Cfg, SP>(sm, ct + (size_t)j * 2 * L * N, pt_ntt + (size_t)j * L * N, out + (size_t)oj * 2 * L * N,
                       limbs[limb], L, limb, comp0, accumulate != 0);
 }
@@ -690,9 +653,13 @@ const char *kname(int kind)
     return kname_of(kind, Cfg::LOGN);
 }
 
-inline hc_status after_launch(const char *what)
+// every kernel of this file starts by waiting for the launches before it (pdl_begin), so
+// each is launched as their programmatic dependent: its launch overlaps their last CTAs
+template <class... P, class... A>
+hc_status launch(const char *what, void (*kern)(P...), uint32_t grid, uint32_t block, size_t smem, cudaStream_t s,
+                 const A &...args)
 {
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_programmatic(kern, dim3(grid), dim3(block), smem, s, true, args...);
     return e == cudaSuccess ? HC_OK : cuda_error(e, what);
 }
 
@@ -707,15 +674,13 @@ hc_status run_ntt_segs(const NttSegsT<NS> &segs, cudaStream_t s, bool inverse)
         hc_status st = prepare<Cfg, SP, KIND * 1000 + NS>(kern, Cfg::SMEM_BYTES);
         if (st != HC_OK) return st;
         ProfileScope ps(kname<Cfg>(KK_INV), s);
-        kern<<<items, Cfg::T, Cfg::SMEM_BYTES, s>>>(segs);
-        return after_launch("k_ntt_inv");
+        return launch("k_ntt_inv", kern, items, Cfg::T, Cfg::SMEM_BYTES, s, segs);
     }
     auto kern = k_ntt_fwd<Cfg, NS, SP>;
     hc_status st = prepare<Cfg, SP, KIND * 1000 + NS>(kern, Cfg::SMEM_BYTES);
     if (st != HC_OK) return st;
     ProfileScope ps(kname<Cfg>(KK_FWD), s);
-    kern<<<items, Cfg::T, Cfg::SMEM_BYTES, s>>>(segs);
-    return after_launch("k_ntt_fwd");
+    return launch("k_ntt_fwd", kern, items, Cfg::T, Cfg::SMEM_BYTES, s, segs);
 }
 
 // persistent TMA-fed inverse NTT: segs' cta_begin are unit offsets (n_groups
@@ -744,19 +709,12 @@ hc_status run_ntt_inv_tma(const NttSegsT<NS> &segs, int *err, cudaStream_t s)
     }
     const uint32_t grid = total < (uint32_t)r ? total : (uint32_t)r;
     ProfileScope ps(kname<Cfg>(KK_INV), s);
-    kern<<<grid, Cfg::T, smem, s>>>(segs, total, err);
-    return after_launch("k_ntt_inv_tma");
+    return launch("k_ntt_inv_tma", kern, grid, Cfg::T, smem, s, segs, total, err);
 }
 
-template <class HCfg, bool SP, int NS>
-hc_status run_ntt_inv_pair(const NttSegsT<NS> &segs, cudaStream_t s);
-
 // persistent prefetching inverse NTT: segs' cta_begin are unit offsets
-// (n_groups polynomials x L limbs per segment); one launch of resident CTAs.
-// With fewer limbs than resident CTAs no CTA would prefetch, and the limbs run
-// as two-CTA clusters (k_ntt_inv_pair, halves of shape PCfg) instead: measured
-// on GB300, 7-14 % lower latency for a few limbs, 11 % higher time for 1536.
-template <class Cfg, class PCfg, bool SP, int NS>
+// (n_groups polynomials x L limbs per segment); one launch of resident CTAs
+template <class Cfg, bool SP, int NS>
 hc_status run_ntt_inv_pf(const NttSegsT<NS> &segs, cudaStream_t s)
 {
     uint32_t total = 0;
@@ -778,11 +736,9 @@ hc_status run_ntt_inv_pf(const NttSegsT<NS> &segs, cudaStream_t s)
         r = per_sm * sms;
         resident[dev & 31].store(r);
     }
-    if (total < (uint32_t)r) return run_ntt_inv_pair<PCfg, SP>(segs, s);
     const uint32_t grid = total < (uint32_t)r ? total : (uint32_t)r;
     ProfileScope ps(kname<Cfg>(KK_INV), s);
-    kern<<<grid, Cfg::T, smem, s>>>(segs, total);
-    return after_launch("k_ntt_inv_pf");
+    return launch("k_ntt_inv_pf", kern, grid, Cfg::T, smem, s, segs, total);
 }
 
 // forward NTTs by clusters of two CTAs: segs' cta_begin are unit offsets (n_groups
@@ -798,23 +754,27 @@ hc_status run_ntt_fwd_pair(const NttSegsT<NS> &segs, cudaStream_t s)
     hc_status st = prepare<HCfg, SP, 7000 + NS>(kern, HCfg::SMEM_BYTES);
     if (st != HC_OK) return st;
     ProfileScope ps(kname_of(KK_FWD, HCfg::LOGN + 1), s);
-    kern<<<2 * total, HCfg::T, HCfg::SMEM_BYTES, s>>>(segs);
-    return after_launch("k_ntt_fwd_pair");
+    return launch("k_ntt_fwd_pair", kern, 2 * total, HCfg::T, HCfg::SMEM_BYTES, s, segs);
 }
 
-template <class HCfg, bool SP, int NS>
-hc_status run_ntt_inv_pair(const NttSegsT<NS> &segs, cudaStream_t s)
+// transforms of few polynomials over clusters: segs' cta_begin are unit offsets
+template <class S, bool SP, int NS>
+hc_status run_ntt_split(const NttSegsT<NS> &segs, uint32_t total, bool inverse, cudaStream_t s)
 {
-    uint32_t total = 0;
-    for (uint32_t i = 0; i < segs.n; ++i) total = segs.s[i].cta_begin + segs.s[i].n_groups * seg_limbs(segs.s[i]);
-    if (total == 0) return HC_OK;
-    if (total > 0x3fffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
-    auto kern = k_ntt_inv_pair<HCfg, NS, SP>;
-    hc_status st = prepare<HCfg, SP, 8000 + NS>(kern, HCfg::SMEM_BYTES);
-    if (st != HC_OK) return st;
-    ProfileScope ps(kname_of(KK_INV, HCfg::LOGN + 1), s);
-    kern<<<2 * total, HCfg::T, HCfg::SMEM_BYTES, s>>>(segs);
-    return after_launch("k_ntt_inv_pair");
+    ProfileScope ps(kname_of(inverse ? KK_INV : KK_FWD, S::LOGN), s);
+    return launch("k_ntt_split", inverse ? k_ntt_inv_split<S, NS, SP> : k_ntt_fwd_split<S, NS, SP>, total * S::CS,
+                  S::THREADS, S::NL * sizeof(uint64_t), s, segs);
+}
+
+template <class S, bool SP>
+hc_status run_product_split(const hc_ctx *ctx, const LaunchArgs &a, cudaStream_t s)
+{
+    if (a.n == 0) return HC_OK;
+    SlotList slots;
+    for (uint32_t j = 0; j < kSplitMaxProducts; ++j) slots.s[j] = a.h_slots && j < a.n ? a.h_slots[j] : j;
+    ProfileScope ps(kname_of(KK_PROD, S::LOGN), s);
+    return launch("k_product_split", k_product_split<S, SP>, (unsigned)(a.n * ctx->L * S::CS), S::THREADS,
+                  2 * S::NL * sizeof(uint64_t), s, a.in, a.pt, a.out, ctx->d_limbs, ctx->L, a.accumulate ? 1 : 0, slots);
 }
 
 // one-segment launch: n_groups CTAs per limb
@@ -854,9 +814,7 @@ hc_status run_mac_intt(const hc_ctx *ctx, const uint64_t *ct_ntt, const uint64_t
     const size_t items = n_groups * ctx->L;
     if (items > 0x7fffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
     ProfileScope ps(kname<Cfg>(2), s);
-    kern<<<(unsigned)items, Cfg::T, Cfg::SMEM_BYTES, s>>>(ct_ntt, pt_ntt, terms.term_ptr, terms.terms, out,
-                                                          ctx->d_limbs, ctx->L, (uint32_t)n_groups);
-    return after_launch("k_mac_intt");
+    return launch("k_mac_intt", kern, (unsigned)items, Cfg::T, Cfg::SMEM_BYTES, s, ct_ntt, pt_ntt, terms.term_ptr, terms.terms, out, ctx->d_limbs, ctx->L, (uint32_t)n_groups);
 }
 
 template <class Cfg, bool SP>
@@ -871,8 +829,7 @@ hc_status run_inv_extract(const hc_ctx *ctx, const ExtractArgs &ex, cudaStream_t
     const size_t items = (size_t)ex.O * 2 * Lc;
     if (items > 0x7fffffffu) return set_error(HC_ERR_INVALID_ARG, "layer too large");
     ProfileScope ps("k_ntt_inv_extract", s);
-    kern<<<(unsigned)items, Cfg::T, Cfg::SMEM_BYTES, s>>>(ex, ctx->d_limbs, ctx->L);
-    return after_launch("k_ntt_inv_extract");
+    return launch("k_ntt_inv_extract", kern, (unsigned)items, Cfg::T, Cfg::SMEM_BYTES, s, ex, ctx->d_limbs, ctx->L);
 }
 
 template <class Cfg, bool SP>
@@ -887,24 +844,54 @@ hc_status run_product(const hc_ctx *ctx, const uint64_t *ct, const uint64_t *pt_
     const size_t items = n_groups * ctx->L;
     if (items > 0x7fffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
     ProfileScope ps(kname<Cfg>(3), s);
-    kern<<<(unsigned)items, Cfg::T, Cfg::SMEM_BYTES, s>>>(ct, pt_ntt, out_index, out, ctx->d_limbs, ctx->L,
-                                                          (uint32_t)n_groups, accumulate ? 1 : 0);
-    return after_launch("k_product");
+    return launch("k_product", kern, (unsigned)items, Cfg::T, Cfg::SMEM_BYTES, s, ct, pt_ntt, out_index, out, ctx->d_limbs, ctx->L, (uint32_t)n_groups, accumulate ? 1 : 0);
 }
 
 }  // namespace detail
+
+// Transforms of so few polynomials that clusters of eight CTAs leave SMs idle run split
+// over such clusters, in the launch shapes a context starts with.
+template <int LOGN, bool SP>
+bool try_ntt_split(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaStream_t s, hc_status *st)
+{
+    using S = SplitShape<LOGN, 3, 1, 1>;
+    const bool inverse = kind == KK_INV || kind == KK_INVCT || kind == KK_INVCT_SEGS;
+    auto few = [&](uint64_t units) { return units > 0 && units <= split_units_ntt(LOGN, ctx->sms); };
+    if (kind == KK_FWDCT_SEGS || kind == KK_INVCT_SEGS) {
+        NttSegs segs = *a.segs;
+        uint64_t total = 0;
+        for (uint32_t i = 0; i < segs.n; ++i) {
+            segs.s[i].n_groups *= 2;  // polynomials
+            segs.s[i].cta_begin = (uint32_t)total;
+            total += (uint64_t)segs.s[i].n_groups * seg_limbs(segs.s[i]);
+        }
+        if (!few(total)) return false;
+        *st = detail::run_ntt_split<S, SP>(segs, (uint32_t)total, inverse, s);
+        return true;
+    }
+    if (kind != KK_FWD && kind != KK_INV && kind != KK_FWDCT && kind != KK_INVCT) return false;
+    const size_t polys = kind == KK_FWD || kind == KK_INV ? a.n : 2 * a.n;
+    if (polys > 0x7fffffffu / kMaxLimbs || !few((uint64_t)polys * ctx->L)) return false;
+    *st = detail::run_ntt_split<S, SP>(detail::one_seg(ctx, a.in, a.out, polys), (uint32_t)(polys * ctx->L), inverse, s);
+    return true;
+}
 
 template <int LOGN, int V, bool SP>
 hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaStream_t s)
 {
     using Fused = VCfg<LOGN, V, false>;
     using Single = VCfg<LOGN, V, true>;
+    const int base = kind == KK_FWDCT_SEGS ? KK_FWDCT : kind == KK_INVCT_SEGS ? KK_INVCT : kind;
+    if (V == default_variant(base, LOGN)) {
+        hc_status st = HC_OK;
+        if (try_ntt_split<LOGN, SP>(ctx, kind, a, s, &st)) return st;
+    }
     if constexpr (use_inv_tma<LOGN, V> || use_inv_pf<LOGN, V>) {
         auto run = [&](const auto &segs) {
             if constexpr (use_inv_tma<LOGN, V>)
                 return detail::run_ntt_inv_tma<typename InvTma<LOGN>::Cfg, SP>(segs, timeout_flag(ctx), s);
             else
-                return detail::run_ntt_inv_pf<typename InvPf<LOGN>::Cfg, typename FwdPair<LOGN>::Cfg, SP>(segs, s);
+                return detail::run_ntt_inv_pf<typename InvPf<LOGN>::Cfg, SP>(segs, s);
         };
         if (kind == KK_INV || kind == KK_INVCT) {
             const size_t polys = kind == KK_INV ? a.n : 2 * a.n;
@@ -962,11 +949,14 @@ hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaS
     }
     case KK_MAC: return detail::run_mac_intt<Fused, SP>(ctx, a.in, a.pt, a.terms, a.out, a.n, s);
     case KK_PROD: return detail::run_product<Fused, SP>(ctx, a.in, a.pt, a.out_index, a.out, a.n, a.accumulate, s);
+    case KK_PROD_SPLIT:
+        if constexpr (V == 0) return detail::run_product_split<SplitShape<LOGN, 3, 2, 1, 3, LOGN == 12 ? 8 : 16>, SP>(ctx, a, s);
+        return set_error(HC_ERR_INVALID_ARG, "the split product has one shape");
     case KK_INV_EXTRACT:
-        // variant 2 of the inverse kinds is persistent at N >= 8192; the epilogue
+        // variant 2 of the inverse kinds is persistent at N = 16384; the epilogue
         // kernel (one output limb per CTA, shared memory busy until its last store)
-        // takes the best one-CTA shape there, variant 1's
-        if constexpr (V == 2 && LOGN >= 13)
+        // takes variant 1's shape there
+        if constexpr (V == 2 && LOGN == 14)
             return detail::run_inv_extract<VCfg<LOGN, 1, true>, SP>(ctx, *a.ex, s);
         else
             return detail::run_inv_extract<Single, SP>(ctx, *a.ex, s);

@@ -28,74 +28,9 @@
 
 #include <atomic>
 
-#include "hc_async.cuh"
-#include "hc_ntt.cuh"
+#include "hc_split.cuh"
 
 namespace hc {
-
-// NG groups of T threads, NP polynomials at a time: group g transforms the digits
-// g*NP .., (g + NG)*NP .., then components g*NP ...  8 residues of each per thread.
-//   latency (NG = 4, NP = 1): with few units in flight a CTA has an SM to itself, and the
-//     time is the instructions of one warp times their latency, so the digits and the
-//     components run side by side.
-//   throughput (NG = 1, NP = 2): one set of twiddle loads for two polynomials, more CTAs
-//     per SM.
-template <int LOGN_, int LOGP_, int NG_, int NP_>
-struct KsShape {
-    static constexpr int LOGN = LOGN_, LOGP = LOGP_, CS = 1 << LOGP, NG = NG_, NP = NP_;
-    template <int P>
-    using CfgP = NttCfg<LOGN - LOGP, 3, P, 1, NG>;
-    using Cfg = CfgP<1>;
-    static constexpr int NL = Cfg::N, T = Cfg::T, C = Cfg::C, ITEMS = C / CS, THREADS = T * NG;
-    static constexpr int MINB = NG > 1 ? 1 : 768 / THREADS;
-    static_assert(ITEMS >= 1 && NL / CS == ITEMS * T, "whole slices of the cross stages");
-    static_assert(NG * NP >= 2 && NP <= 2, "both components at once");
-    static size_t smem(uint32_t L) { return (size_t)(L < 2 ? 2 : L) * NL * sizeof(uint64_t); }
-};
-
-// first LOGP stages of digits j .. j + NP - 1 for this thread's slice, results into their
-// owners' buffers
-template <class S, int NP, bool SP>
-__device__ __forceinline__ void ks_fwd_cross(const uint64_t *c1, uint32_t j, const uint64_t *sm, uint32_t slice,
-                                             const LimbConst &lc, const TwArith<SP> &ar)
-{
-    constexpr int CS = S::CS, ITEMS = S::ITEMS, T = S::T, NL = S::NL;
-    uint64_t v[NP][ITEMS][CS];
-    const unsigned long long *a = (const unsigned long long *)c1 + ((size_t)j << S::LOGN) + slice;
-#pragma unroll
-    for (int p = 0; p < NP; ++p)
-#pragma unroll
-        for (int it = 0; it < ITEMS; ++it)
-#pragma unroll
-            for (int c = 0; c < CS; ++c) v[p][it][c] = __ldcg(a + ((size_t)p << S::LOGN) + it * T + c * NL);
-    static_for<0, S::LOGP>([&](auto sc) {
-        constexpr int s = decltype(sc)::value, half = CS >> (s + 1);
-#pragma unroll
-        for (int lam = 0; lam < (1 << s); ++lam) {
-            const ulonglong2 w = __ldg(lc.tw_f + (1 << s) + lam);
-#pragma unroll
-            for (int jj = 0; jj < half; ++jj) {
-                const int k = lam * 2 * half + jj;
-#pragma unroll
-                for (int p = 0; p < NP; ++p)
-#pragma unroll
-                    for (int it = 0; it < ITEMS; ++it) {
-                        const uint64_t X = v[p][it][k], t = ar.mul(v[p][it][k + half], w);
-                        v[p][it][k] = X + t;
-                        v[p][it][k + half] = ar.sub(X, t);
-                    }
-            }
-        }
-    });
-#pragma unroll
-    for (int c = 0; c < CS; ++c) {
-        const uint32_t to = cluster_map(sm, c) + (j * NL + slice) * 8;
-#pragma unroll
-        for (int p = 0; p < NP; ++p)
-#pragma unroll
-            for (int it = 0; it < ITEMS; ++it) st_cluster_u64(to + (p * NL + it * T) * 8, v[p][it][c]);
-    }
-}
 
 // the other stages of NP digits in the buffers b, b + NL; a thread's residues (elements
 // tid*C + r) end up in its own swizzled positions
@@ -124,6 +59,13 @@ __device__ __forceinline__ void ks_fwd_local(uint64_t *b, const LimbConst &lc, c
         }
 }
 
+// a buffer per digit, or per component
+template <class S>
+size_t ks_smem(uint32_t L)
+{
+    return (size_t)(L < 2 ? 2 : L) * S::NL * sizeof(uint64_t);
+}
+
 template <class S, bool SP>
 __global__ void __cluster_dims__(S::CS, 1, 1) __launch_bounds__(S::THREADS, S::MINB)
 k_ks_switch(const KsArgs args)
@@ -131,6 +73,7 @@ k_ks_switch(const KsArgs args)
     using Cfg = typename S::template CfgP<S::NP>;
     constexpr int LOGP = S::LOGP, CS = S::CS, C = S::C, T = S::T, NL = S::NL, ITEMS = S::ITEMS, NG = S::NG, NP = S::NP;
     constexpr size_t N = (size_t)1 << S::LOGN;
+    static_assert(S::NG * S::NP >= 2, "both components at once");
     extern __shared__ __align__(16) uint64_t sm[];  // [max(L, 2)][NL]
     const int tid = threadIdx.x % T;
     const uint32_t first = threadIdx.x / T * NP;  // the group's first digit and component
@@ -141,15 +84,14 @@ k_ks_switch(const KsArgs args)
     const int tmul = CS + (int)rank;
     const uint32_t slice = rank * (NL / CS) + tid;  // this thread's first pair of the cross stages
     cluster_sync();  // every CTA of the cluster is running before one writes into another
-    pdl_launch_dependents();
-    pdl_wait();
+    pdl_begin();
 
     const uint64_t *c1 = args.a + (size_t)(2 * ct + 1) * L * N;
     for (uint32_t j = first; j < L; j += NG * NP) {
         if (j + NP <= L)
-            ks_fwd_cross<S, NP, SP>(c1, j, sm, slice, lc, ar);
+            split_fwd_cross<S, NP, SP>(c1 + j * N, N, sm, j * NL, slice, lc, ar);
         else
-            ks_fwd_cross<S, 1, SP>(c1, j, sm, slice, lc, ar);
+            split_fwd_cross<S, 1, SP>(c1 + j * N, N, sm, j * NL, slice, lc, ar);
     }
     cluster_sync();  // this CTA's parts of the digits are complete
     for (uint32_t j = first; j < L; j += NG * NP) {
@@ -208,41 +150,8 @@ k_ks_switch(const KsArgs args)
     }
     cluster_sync();  // every part is in shared memory
     if (first < 2) {
-        const ulonglong2 wn = make_ulonglong2(lc.ninv, lc.ninv_s), wnw = make_ulonglong2(lc.ninvw, lc.ninvw_s);
         uint64_t v[NP][ITEMS][CS];
-#pragma unroll
-        for (int c = 0; c < CS; ++c) {
-            const uint32_t from = cluster_map(sm, c) + (first * NL + slice) * 8;
-#pragma unroll
-            for (int p = 0; p < NP; ++p)
-#pragma unroll
-                for (int it = 0; it < ITEMS; ++it) v[p][it][c] = ld_cluster_u64(from + (p * NL + it * T) * 8);
-        }
-        static_for<0, LOGP>([&](auto sc) {
-            constexpr int s = decltype(sc)::value, dist = 1 << s, ngrp = CS >> (s + 1);
-            const uint64_t qs = ar.q << (S::LOGN - LOGP + s);  // bound of the stage's inputs (Shoup)
-#pragma unroll
-            for (int g = 0; g < ngrp; ++g) {
-                const ulonglong2 w = __ldg(lc.tw_i + ngrp + g);
-#pragma unroll
-                for (int jj = 0; jj < dist; ++jj) {
-                    const int k = g * 2 * dist + jj;
-#pragma unroll
-                    for (int p = 0; p < NP; ++p)
-#pragma unroll
-                        for (int it = 0; it < ITEMS; ++it) {
-                            const uint64_t X = v[p][it][k], Y = v[p][it][k + dist];
-                            if constexpr (s == LOGP - 1) {
-                                v[p][it][k] = ar.mul_canon(X + Y, wn);
-                                v[p][it][k + dist] = ar.mul_canon(ar.sub(X, Y, qs), wnw);
-                            } else {
-                                v[p][it][k] = X + Y;
-                                v[p][it][k + dist] = ar.mul(ar.sub(X, Y, qs), w);
-                            }
-                        }
-                }
-            }
-        });
+        split_inv_cross<S, NP, SP>(v, sm, first * NL, slice, lc, ar);
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
             uint64_t *u = args.u + ((size_t)(2 * ct + first + p) * L1 + i) * N + slice;
@@ -266,24 +175,14 @@ hc_status run_ks_switch(const KsArgs &a, size_t n, cudaStream_t s)
     const uint32_t bit = 1u << (dev & 31);
     if (!(done.load(std::memory_order_relaxed) & bit)) {
         const cudaError_t e =
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem(kMaxLimbs - 1));
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ks_smem<S>(kMaxLimbs - 1));
         if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute(k_ks_switch)");
         done.fetch_or(bit);
     }
     const size_t ctas = n * (a.L + 1) * S::CS;
     if (ctas > 0x7fffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
     ProfileScope ps("k_ks_switch", s);
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)ctas);
-    cfg.blockDim = dim3(S::THREADS);
-    cfg.dynamicSmemBytes = S::smem(a.L);
-    cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a);
+    const cudaError_t e = launch_programmatic(kern, dim3((unsigned)ctas), dim3(S::THREADS), ks_smem<S>(a.L), s, true, a);
     return e == cudaSuccess ? HC_OK : cuda_error(e, "launch k_ks_switch");
 }
 
@@ -298,11 +197,11 @@ hc_status launch_ks_n(const KsArgs &a, size_t n, uint32_t sms, cudaStream_t s)
 {
     const bool few = 8 * n * (a.L + 1) <= 2 * (size_t)sms;
     if constexpr (LOGN < 14) {
-        if (few) return run_ks_switch<KsShape<LOGN, 3, 4, 1>, SP>(a, n, s);
+        if (few) return run_ks_switch<SplitShape<LOGN, 3, 4, 1, 3, 8>, SP>(a, n, s);
     } else {
-        if (few) return run_ks_switch<KsShape<LOGN, 3, 2, 1>, SP>(a, n, s);
+        if (few) return run_ks_switch<SplitShape<LOGN, 3, 2, 1, 3, 16>, SP>(a, n, s);
     }
-    return run_ks_switch<KsShape<LOGN, LOGN - 11, 1, 2>, SP>(a, n, s);
+    return run_ks_switch<SplitShape<LOGN, LOGN - 11, 1, 2>, SP>(a, n, s);
 }
 
 }  // namespace hc

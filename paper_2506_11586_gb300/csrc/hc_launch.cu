@@ -49,10 +49,9 @@ __global__ void k_range_check(const uint64_t *__restrict__ p, const LimbConst *_
 }
 
 
-// Launch shapes a context starts with (the autotuner may change them).  Measured
-// on GB300: at N >= 8192 the forward transforms run fastest as two-CTA clusters
-// and the inverse ones as the persistent prefetching kernel (variant 2 of both),
-// for a few polynomials (latency) and for a layer's hundreds (throughput) alike.
+// Launch shapes a context starts with (the autotuner may change them); figures at
+// Variant in hc_kernels.cuh.  In these shapes launches of few limbs run split over
+// clusters (split_units_ntt).
 int default_variant(int kind, uint32_t logn)
 {
     if (logn >= 13 && (kind == KK_FWD || kind == KK_FWDCT || kind == KK_INV || kind == KK_INVCT)) return 2;
@@ -74,6 +73,7 @@ k_mac_conv(const __grid_constant__ MacSegsT<NS> segs, int *err)
 {
     __shared__ __align__(8) uint64_t bars[kMacBars];
     extern __shared__ __align__(16) uint64_t dsm[];
+    pdl_begin();
     uint32_t si = 0;
     while (si + 1 < segs.n && blockIdx.x >= segs.s[si + 1].cta_begin) ++si;
     const MacSeg &sg = segs.s[si];
@@ -170,8 +170,8 @@ static hc_status run_mac_segs(MacSegsT<NS> &segs, size_t smem, int *err, cudaStr
     }
     if (begin == 0) return HC_OK;
     ProfileScope ps("k_mac_conv", s);
-    k_mac_conv<NS><<<begin, kMacThreads, smem, s>>>(segs, err);
-    return after_launch_status("k_mac_conv");
+    const cudaError_t e = launch_programmatic(k_mac_conv<NS>, dim3(begin), dim3(kMacThreads), smem, s, true, segs, err);
+    return e == cudaSuccess ? HC_OK : cuda_error(e, "launch k_mac_conv");
 }
 
 size_t mac_seg_smem(const MacSeg &sg)
@@ -272,6 +272,7 @@ hc_status dispatch(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaStream_
     const int v = kind == KK_FWDCT_SEGS    ? ctx->variant[KK_FWDCT]
                   : kind == KK_INVCT_SEGS  ? ctx->variant[KK_INVCT]
                   : kind == KK_INV_EXTRACT ? ctx->variant[KK_INVCT]
+                  : kind == KK_PROD_SPLIT  ? 0
                                            : ctx->variant[kind];
     const bool fold = a.segs ? a.segs->s[0].fold != 0 : ctx->fold;
     switch (ctx->logN) {
@@ -365,6 +366,25 @@ hc_status launch_product(const hc_ctx *ctx, const uint64_t *ct, const uint64_t *
     a.n = n;
     a.accumulate = accumulate;
     return dispatch(ctx, KK_PROD, a, s);
+}
+
+bool product_split(const hc_ctx *ctx, size_t n)
+{
+    return ctx->variant[KK_PROD] == default_variant(KK_PROD, ctx->logN) && n <= kSplitMaxProducts &&
+           n * ctx->L <= split_units_product(ctx->logN, ctx->sms);
+}
+
+hc_status launch_product_split(const hc_ctx *ctx, const uint64_t *ct, const uint64_t *pt_ntt, const uint32_t *slots,
+                               uint64_t *out, size_t n, bool accumulate, cudaStream_t s)
+{
+    LaunchArgs a{};
+    a.in = ct;
+    a.pt = pt_ntt;
+    a.h_slots = slots;
+    a.out = out;
+    a.n = n;
+    a.accumulate = accumulate;
+    return dispatch(ctx, KK_PROD_SPLIT, a, s);
 }
 
 hc_status launch_lift_int8(const hc_ctx *ctx, const int8_t *packed, uint64_t *out, size_t n_polys, cudaStream_t s)

@@ -225,7 +225,7 @@ __device__ __forceinline__ void mac_stream_task(const MacSeg &sg, uint32_t chunk
     const size_t LN = (size_t)sg.L * sg.N, off = (size_t)limb * sg.N + chunk * KC;
     const uint32_t k = threadIdx.x % KC, h = threadIdx.x / KC;
     const uint64_t *xg = sg.X + off + k;
-    for (uint32_t r = h; r < rows; r += H) xs[r * KC + k] = split25(__ldg(xg + r * LN));
+    for (uint32_t r = h; r < rows; r += H) xs[r * KC + k] = split25(ld_data(xg + r * LN));
     const LimbConst &lc = sg.limbs[limb];
     const uint64_t q = lc.q;
     const uint32_t sc = (uint32_t)lc.special_c;

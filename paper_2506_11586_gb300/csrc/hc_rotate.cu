@@ -66,8 +66,7 @@ k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *
            const LimbConst *__restrict__ lq, const ModDown *__restrict__ md, uint64_t special, uint32_t L, uint32_t N,
            uint32_t g, uint32_t rows, uint32_t a_ct, uint32_t add_ct)
 {
-    pdl_launch_dependents();
-    pdl_wait();
+    pdl_begin();
     const uint32_t k = 2 * (blockIdx.x * kKsBlock + threadIdx.x);
     const uint32_t mask2 = 2 * N - 1, L1 = L + 1;
     const uint64_t half = (special - 1) / 2;
@@ -77,7 +76,7 @@ k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *
         const LimbConst &lc = lq[i];
         const uint64_t q = lc.q;
         auto strided = [&](uint32_t by) { return ((size_t)(cc >> 1) * by * 2 * L + (cc & 1) * L + i) * N + k; };
-        auto ld2 = [](const uint64_t *p) { return __ldcg(reinterpret_cast<const ulonglong2 *>(p)); };
+        auto ld2 = [](const uint64_t *p) { return ld_data(reinterpret_cast<const ulonglong2 *>(p)); };
         ulonglong2 v;
         if constexpr (DIVIDE) {
             const ulonglong2 ui = ld2(u + ((size_t)cc * L1 + i) * N + k), us = ld2(u + ((size_t)cc * L1 + L) * N + k);
@@ -105,8 +104,8 @@ k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *
         } else if (((uintptr_t)a & 15) == 0) {
             v = ld2(a + strided(a_ct));
         } else {  // the caller's input on an odd word
-            const unsigned long long *p = (const unsigned long long *)a + strided(a_ct);
-            v = make_ulonglong2(__ldcg(p), __ldcg(p + 1));
+            const uint64_t *p = a + strided(a_ct);
+            v = make_ulonglong2(ld_data(p), ld_data(p + 1));
         }
         uint64_t *o = out + (size_t)r * N;
         if (g == 1 && ((uintptr_t)out & 15) == 0) {
@@ -191,19 +190,11 @@ hc_status ks_apply(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *
                    uint32_t add_ct = 1)
 {
     const uint32_t rows = (uint32_t)(n * 2 * ctx->L);
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(ctx->N / 2 / kKsBlock, rows < 65535 ? rows : 65535);
-    cfg.blockDim = dim3(kKsBlock);
-    cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = u ? 1 : 0;  // the first kernel of a chain follows other launches as usual
     ProfileScope ps("k_ks_apply", s);
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, u ? k_ks_apply<true> : k_ks_apply<false>, a, u, add, out,
-                                             (const LimbConst *)ctx->d_limbs, (const ModDown *)key->d_md, key->special,
-                                             ctx->L, ctx->N, g, rows, a_ct, add_ct);
+    const cudaError_t e = launch_programmatic(
+        u ? k_ks_apply<true> : k_ks_apply<false>, dim3(ctx->N / 2 / kKsBlock, rows < 65535 ? rows : 65535),
+        dim3(kKsBlock), 0, s, true, a, u, add, out, ctx->d_limbs, key->d_md, key->special, ctx->L, ctx->N, g,
+        rows, a_ct, add_ct);
     return e == cudaSuccess ? HC_OK : cuda_error(e, "launch k_ks_apply");
 }
 
