@@ -245,7 +245,7 @@ __device__ __forceinline__ void inv_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const 
 #pragma unroll
                 for (int p = 0; p < Cfg::NP; ++p) {
                     const uint64_t X = x[p][j], Y = x[p][j + dist];
-                    x[p][j] = ar.mul_canon(X + Y, wn);
+                    x[p][j] = ar.template div_canon<Cfg::LOGN>(X + Y, wn);
                     x[p][j + dist] = ar.mul_canon(ar.sub(X, Y, qs), wnw);
                 }
             }

@@ -114,7 +114,7 @@ __device__ __forceinline__ void split_inv_cross(uint64_t (&v)[NP][S::ITEMS][S::C
                     for (int it = 0; it < ITEMS; ++it) {
                         const uint64_t X = v[p][it][k], Y = v[p][it][k + dist];
                         if constexpr (s == LOGP - 1) {
-                            v[p][it][k] = ar.mul_canon(X + Y, wn);
+                            v[p][it][k] = ar.template div_canon<S::LOGN>(X + Y, wn);
                             v[p][it][k + dist] = ar.mul_canon(ar.sub(X, Y, qs), wnw);
                         } else {
                             v[p][it][k] = X + Y;

@@ -62,3 +62,22 @@ def test_inverse_bounds(rounds, half):
         assert folds <= 4
         b = max(5 if m > limit else m for m in model)
         assert b <= 4096
+
+
+@pytest.mark.parametrize("logn", [12, 13, 14])
+@pytest.mark.parametrize("q", CANONICAL_PRIMES)
+def test_division_by_the_degree(q, logn):
+    """y / 2^logn mod q by one product: exact shifts, a non-negative value below 2^53 that
+    one fold at 2^50 and one subtraction make canonical."""
+    c, ninv = (1 << 50) - q, pow(1 << logn, -1, q)
+    ys = [0, 1, -1, 8192 * q, -8192 * q, 8192 * q - 1, 1 - 8192 * q, q, -q, (1 << logn) - 1, -(1 << logn)]
+    ys += [(int(x) - (1 << 63)) // (1 << 63) * 8192 * q + int(x) % (8192 * q) for x in Stream(5, logn).u64(200)]
+    for y in ys:
+        assert abs(y) <= 8192 * q
+        k = -y % (1 << logn)
+        t = y - k * c
+        assert -(1 << 63) <= t < 1 << 63 and t % (1 << logn) == 0
+        r = (t >> logn) + (k << (50 - logn)) + 4 * q
+        assert 0 <= r < 1 << 53
+        r = (r & ((1 << 50) - 1)) + (r >> 50) * c
+        assert r < 2 * q and (r - q if r >= q else r) == y * ninv % q
