@@ -999,15 +999,19 @@ hc_status hc_conv_ct_pt_host(const hc_ctx *ctx, const hc_weights *w, const uint6
     dout.p = dev_alloc(w->O * ct_bytes, s);
     if (!din.p || !dout.p) return set_error(HC_ERR_OOM, "device buffer allocation failed");
     HC_CUDA_TRY(cudaMemcpyAsync(din.p, h_ct_in, w->I * ct_bytes, cudaMemcpyHostToDevice, s));
-    const uint32_t K = std::min<uint32_t>(kHostChunks, w->Mp);
-    if (w->mode != HC_WEIGHTS_NTT_OFFLINE || !conv_job_blocked(ctx, w) || K < 2) {
+    if (w->mode != HC_WEIGHTS_NTT_OFFLINE || !conv_job_blocked(ctx, w) || w->Mp < 2) {
         hc_status st = hc_conv_ct_pt(ctx, w, (const uint64_t *)din.p, (uint64_t *)dout.p, cuda_stream);
         if (st != HC_OK) return st;
         HC_CUDA_TRY(cudaMemcpyAsync(h_ct_out, dout.p, w->O * ct_bytes, cudaMemcpyDeviceToHost, s));
         return hc_ctx_device_status(ctx, cuda_stream);
     }
     // Pipelined: the outputs of a block of output channels (contiguous in the output
-    // and in the weights) go back to the host while the next block is computed.
+    // and in the weights) go back to the host while the next block is computed.  The copies
+    // bound the call (188 GB/s measured to pinned memory, several times slower than the
+    // kernels), so the first blocks are small, a sixteenth of the channels, to start them
+    // early, and each later one is as large as those before it together, which hides its
+    // kernels behind their copies and keeps the copies few.  128 output ciphertexts at
+    // N = 8192, L = 3, of a 27x27 layer on GB300: 345 -> 336 us.
     hc_status st = check_inputs(ctx, (const uint64_t *)din.p, (size_t)2 * w->I, s);
     if (st != HC_OK) return st;
     CopyLane *lane = nullptr;
@@ -1019,11 +1023,9 @@ hc_status hc_conv_ct_pt_host(const hc_ctx *ctx, const hc_weights *w, const uint6
     st = launch_ntt_fwd_ct(ctx, (const uint64_t *)din.p, x, w->I, s);
     if (st != HC_OK) return st;
     const size_t LN = (size_t)ctx->L * ctx->N;
-    const uint32_t per = (w->Mp + K - 1) / K;
     uint32_t used = 0;
-    for (uint32_t j = 0; j < K; ++j) {
-        const uint32_t m0 = j * per, m1 = std::min(w->Mp, m0 + per);
-        if (m0 >= m1) break;
+    for (uint32_t m0 = 0, m1, j = 0; m0 < w->Mp; m0 = m1, ++j) {
+        m1 = j + 1 == kHostChunks ? w->Mp : std::min(w->Mp, m0 ? 2 * m0 : std::max(1u, w->Mp / 16));
         const size_t o0 = (size_t)m0 * w->B, no = (size_t)(m1 - m0) * w->B;
         st = launch_mac_conv(ctx, x, w->d_pt + (size_t)m0 * w->G * LN, y + o0 * ct_words, w->G, w->B, m1 - m0, s);
         if (st == HC_OK) st = launch_ntt_inv_ct(ctx, y + o0 * ct_words, y + o0 * ct_words, no, s);
