@@ -86,7 +86,7 @@ __device__ __forceinline__ void load_round0(uint64_t (&x)[Cfg::NP][Cfg::C], cons
 #pragma unroll
     for (int r = 0; r < Cfg::C; ++r)
 #pragma unroll
-        for (int p = 0; p < Cfg::NP; ++p) x[p][r] = sm[p * Cfg::N + spos<Cfg>(tid * Cfg::C + r)];
+        for (int p = 0; p < Cfg::NP; ++p) x[p][r] = sm[p * Cfg::SW + spos_at<Cfg>(tid * Cfg::C, r)];
 }
 
 // ---------------------------------------------------------------------------
@@ -110,7 +110,7 @@ __device__ __forceinline__ void fwd_task(uint64_t *sm, const uint64_t *src, uint
 #pragma unroll
     for (int r = 0; r < C; ++r) {
 #pragma unroll
-        for (int p = 0; p < NP; ++p) sm[p * N + spos<Cfg>(tid * C + r)] = ar.canon(x[p][r]);
+        for (int p = 0; p < NP; ++p) sm[p * Cfg::SW + spos_at<Cfg>(tid * C, r)] = ar.canon(x[p][r]);
     }
     __syncthreads();
 #pragma unroll
@@ -118,10 +118,9 @@ __device__ __forceinline__ void fwd_task(uint64_t *sm, const uint64_t *src, uint
         ulonglong2 *d = reinterpret_cast<ulonglong2 *>(dst + p * pstride);
 #pragma unroll
         for (int r = 0; r < C / 2; ++r) {
-            const int e = 2 * (tid + r * T);
             ulonglong2 v;
-            v.x = sm[p * N + spos<Cfg>(e)];
-            v.y = sm[p * N + spos<Cfg>(e + 1)];
+            v.x = sm[p * Cfg::SW + spos_at<Cfg>(2 * tid, 2 * r * T)];
+            v.y = sm[p * Cfg::SW + spos_at<Cfg>(2 * tid, 2 * r * T + 1)];
             d[tid + r * T] = v;
         }
     }
@@ -140,10 +139,9 @@ __device__ __forceinline__ void inv_core(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_
         const ulonglong2 *s2 = reinterpret_cast<const ulonglong2 *>(src + p * pstride);
 #pragma unroll
         for (int r = 0; r < C / 2; ++r) {
-            const int e = 2 * (tid + r * Cfg::T);
             const ulonglong2 v = ld_data(s2 + tid + r * Cfg::T);
-            sm[p * N + spos<Cfg>(e)] = v.x;
-            sm[p * N + spos<Cfg>(e + 1)] = v.y;
+            sm[p * Cfg::SW + spos_at<Cfg>(2 * tid, 2 * r * Cfg::T)] = v.x;
+            sm[p * Cfg::SW + spos_at<Cfg>(2 * tid, 2 * r * Cfg::T + 1)] = v.y;
         }
     }
     load_round0<Cfg>(x, sm, tid);
@@ -291,8 +289,8 @@ k_mac_intt(const uint64_t *__restrict__ ct_ntt, const uint64_t *__restrict__ pt_
         }
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-            sm[p * N + spos<Cfg>(e)] = mac_reduce(acc[p][0], q, nq, r64, r64_s, ones);
-            sm[p * N + spos<Cfg>(e + 1)] = mac_reduce(acc[p][1], q, nq, r64, r64_s, ones);
+            sm[p * Cfg::SW + spos<Cfg>(e)] = mac_reduce(acc[p][0], q, nq, r64, r64_s, ones);
+            sm[p * Cfg::SW + spos<Cfg>(e + 1)] = mac_reduce(acc[p][1], q, nq, r64, r64_s, ones);
         }
     }
     uint64_t x[NP][C];
@@ -339,8 +337,8 @@ template <class Cfg, int NS, bool SP>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
 k_ntt_inv_tma(const __grid_constant__ NttSegsT<NS> segs, uint32_t total, int *err)
 {
-    static_assert(Cfg::NP == 1, "one polynomial per unit");
-    extern __shared__ __align__(16) uint64_t sm[];  // [2][N]
+    static_assert(Cfg::NP == 1 && !Cfg::PADDED, "one polynomial per unit, copied as it lies");
+    extern __shared__ __align__(16) uint64_t sm[];  // [2][SW]
     pdl_begin();
     __shared__ __align__(8) uint64_t bars[2];
     constexpr int C = Cfg::C, N = Cfg::N, V = C / 2;
@@ -361,7 +359,7 @@ k_ntt_inv_tma(const __grid_constant__ NttSegsT<NS> segs, uint32_t total, int *er
         locate(u, si, limb, poly);
         const NttSeg &sg = segs.s[si];
         mbar_arrive_expect_tx(&bars[b], BYTES);
-        bulk_g2s(sm + (size_t)b * N, sg.in + ((size_t)poly * sg.L + limb) * N, BYTES, &bars[b]);
+        bulk_g2s(sm + (size_t)b * Cfg::SW, sg.in + ((size_t)poly * sg.L + limb) * N, BYTES, &bars[b]);
     };
     if (tid == 0) {
         mbar_init(&bars[0], 1);
@@ -388,7 +386,7 @@ k_ntt_inv_tma(const __grid_constant__ NttSegsT<NS> segs, uint32_t total, int *er
         locate(u, si, limb, poly);
         const NttSeg &sg = segs.s[si];
         const LimbConst &lc = sg.limbs[limb];
-        uint64_t *buf = sm + (size_t)b * N;
+        uint64_t *buf = sm + (size_t)b * Cfg::SW;
         const uint32_t rho = V >= 8 ? (uint32_t)tid : (uint32_t)tid >> 1;
         const ulonglong2 *vec = reinterpret_cast<const ulonglong2 *>(buf) + (size_t)tid * V;
         ulonglong2 t[V];
@@ -449,8 +447,7 @@ k_ntt_inv_pf(const __grid_constant__ NttSegsT<NS> segs, uint32_t total)
         const int base = (tid & ~31) * C + (tid & 31);
 #pragma unroll
         for (int r = 0; r < C; ++r) {
-            const int e = base + 32 * r;
-            cp_async8(sm + spos<Cfg>(e), src + e);
+            cp_async8(sm + spos_at<Cfg>(base, 32 * r), src + base + 32 * r);
         }
         cp_async_commit();
     };
@@ -466,7 +463,7 @@ k_ntt_inv_pf(const __grid_constant__ NttSegsT<NS> segs, uint32_t total)
         const LimbConst &lc = sg.limbs[limb];
         uint64_t x[1][C];
 #pragma unroll
-        for (int r = 0; r < C; ++r) x[0][r] = sm[spos<Cfg>(tid * C + r)];
+        for (int r = 0; r < C; ++r) x[0][r] = sm[spos_at<Cfg>(tid * C, r)];
         const uint32_t next = u + G;
         const TwArith<SP> ar = tw_arith<SP>(lc);
         inv_transform<Cfg>(x, sm, lc, ar, tid, [&] {
@@ -531,15 +528,14 @@ k_ntt_fwd_pair(const __grid_constant__ NttSegsT<NS> segs)
     fwd_rounds<HCfg, 0, 1>(x, sm, lc.tw_f, nullptr, ar, tid, 2 + (int)rank);
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < C; ++r) sm[spos<HCfg>(tid * C + r)] = ar.canon(x[0][r]);
+    for (int r = 0; r < C; ++r) sm[spos_at<HCfg>(tid * C, r)] = ar.canon(x[0][r]);
     __syncthreads();
     ulonglong2 *d = reinterpret_cast<ulonglong2 *>(sg.out + off + (size_t)rank * NH);
 #pragma unroll
     for (int r = 0; r < C / 2; ++r) {
-        const int e = 2 * (tid + r * T);
         ulonglong2 v;
-        v.x = sm[spos<HCfg>(e)];
-        v.y = sm[spos<HCfg>(e + 1)];
+        v.x = sm[spos_at<HCfg>(2 * tid, 2 * r * T)];
+        v.y = sm[spos_at<HCfg>(2 * tid, 2 * r * T + 1)];
         d[tid + r * T] = v;
     }
 }

@@ -53,9 +53,9 @@ __device__ __forceinline__ void ks_fwd_local(uint64_t *b, const LimbConst &lc, c
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
             if constexpr (SP)  // [0, 2^53), as the sums want it
-                b[p * NL + spos<Cfg>(tid * C + r)] = ar.fold(x[p][r] + 2048 * ar.q);
+                b[p * NL + spos_at<Cfg>(tid * C, r)] = ar.fold(x[p][r] + 2048 * ar.q);
             else
-                b[p * NL + spos<Cfg>(tid * C + r)] = x[p][r];
+                b[p * NL + spos_at<Cfg>(tid * C, r)] = x[p][r];
         }
 }
 
@@ -122,8 +122,8 @@ k_ks_switch(const KsArgs args)
                     for (int e = 0; e < E; e += 2) {
                         const ulonglong2 k = __ldg(
                             reinterpret_cast<const ulonglong2 *>(key + (size_t)(2 * j + p) * L1 * N + h + e));
-                        mac_add(acc[p][e], b[spos<Cfg>(tid * C + h + e)], k.x);
-                        mac_add(acc[p][e + 1], b[spos<Cfg>(tid * C + h + e + 1)], k.y);
+                        mac_add(acc[p][e], b[spos_at<Cfg>(tid * C, h + e)], k.x);
+                        mac_add(acc[p][e + 1], b[spos_at<Cfg>(tid * C, h + e + 1)], k.y);
                     }
             }
 #pragma unroll
