@@ -201,11 +201,13 @@ struct TwArith<true> {
     // in both terms: one wide product in place of the six of a product with N^-1.
     // |(y - k c) / 2^LOGN| <= 2^51 + 2^23 for LOGN >= 12, hence 4 q to make it positive.
     // Inverse transforms on GB300: 2048 limbs at N = 16384 275 -> 268 us, 4096 limbs at
-    // N = 4096 171 -> 167 us.
+    // N = 4096 98.6 -> 97.4; at N = 8192, in 128 registers with 32 residues, 1536 limbs
+    // 93.3 -> 96.1, so there the product with N^-1 stays.
     template <int LOGN>
-    __device__ __forceinline__ uint64_t div_canon(uint64_t y, ulonglong2) const
+    __device__ __forceinline__ uint64_t div_canon(uint64_t y, ulonglong2 wn) const
     {
         static_assert(LOGN >= 12 && LOGN <= 15, "ring degrees");
+        if constexpr (LOGN == 13) return mul_canon(y, wn);
         const uint32_t k = (0u - (uint32_t)y) & ((1u << LOGN) - 1);
         uint64_t t;
         asm("{\n\t"
