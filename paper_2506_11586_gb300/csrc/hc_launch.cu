@@ -61,11 +61,10 @@ int default_variant(int kind, uint32_t logn)
 // ---------------------------------------------------------------------------
 // Blocked convolution MAC (the tasks in hc_mac.cuh): one task per CTA; the
 // CTAs of a launch cover the (chunk, limb, channel group) tasks of every
-// segment (layer) of the table.  Layers of one or two blocks stream their weights
-// (chunks of kMacStreamKC slots; figures at mac_stream_task), the others, whose rows share
-// a weight four times and more, take them through the shared-memory ring.
+// segment (layer) of the table.  Layers whose input chunk is small stream their weights
+// (MS = 0; figures at mac_stream_task): chunks of 128 slots while four CTAs' fit an SM, else
+// of 64; the others take them through the shared-memory ring.
 constexpr int kMacThreads = 256;
-constexpr uint32_t kMacStreamKC = 128;
 
 template <int NS>
 __global__ void __launch_bounds__(kMacThreads, 4)
@@ -82,11 +81,18 @@ k_mac_conv(const __grid_constant__ MacSegsT<NS> segs, int *err)
     const uint32_t lc = seg_limbs(sg);
     const uint32_t limb = sg.limb0 + rest % lc;
     const uint32_t m0 = (rest / lc) * sg.MB, m1 = min(sg.M, m0 + sg.MB);
-    if (sg.KC == kMacStreamKC) {
-        if (sg.B == 1)
-            mac_stream_task<kMacStreamKC, kMacThreads, 2, 2>(sg, chunk, limb, m0, m1, dsm);
-        else
-            mac_stream_task<kMacStreamKC, kMacThreads, 1, 4>(sg, chunk, limb, m0, m1, dsm);
+    if (sg.MS == 0) {
+        if (sg.B & 1) {
+            if (sg.KC == 128)
+                mac_stream_task<128, kMacThreads, 2, 2>(sg, chunk, limb, m0, m1, dsm);
+            else
+                mac_stream_task<64, kMacThreads, 2, 2>(sg, chunk, limb, m0, m1, dsm);
+        } else {
+            if (sg.KC == 128)
+                mac_stream_task<128, kMacThreads, 1, 4>(sg, chunk, limb, m0, m1, dsm);
+            else
+                mac_stream_task<64, kMacThreads, 1, 4>(sg, chunk, limb, m0, m1, dsm);
+        }
         return;
     }
     if (threadIdx.x == 0) mac_bars_init<kMacThreads>(bars);
@@ -135,8 +141,9 @@ MacSeg make_mac_seg(const hc_ctx *ctx, const uint64_t *x, const uint64_t *w, uin
     sg.B = B;
     sg.M = M;
     // streamed: the input chunk alone, at least four CTAs per SM
-    const bool stream = !ring && B <= 2 && mac_smem(G, B, 0, kMacStreamKC) <= kMacSmemCap / 4;
-    const uint32_t kc = sg.KC = stream ? kMacStreamKC : kMacKC;
+    const uint32_t skc = mac_smem(G, B, 0, 128) <= kMacSmemCap / 4 ? 128 : 64;
+    const bool stream = !ring && mac_smem(G, B, 0, skc) <= kMacSmemCap / 4;
+    const uint32_t kc = sg.KC = stream ? skc : kMacKC;
     sg.MS = stream ? 0 : mac_stage_channels(G, B, M, v, kc);
     const size_t smem = mac_smem(G, B, sg.MS, kc);
     const uint32_t per_sm = (uint32_t)(kMacSmemCap / smem) < 4 ? (uint32_t)(kMacSmemCap / smem) : 4;
@@ -145,7 +152,8 @@ MacSeg make_mac_seg(const hc_ctx *ctx, const uint64_t *x, const uint64_t *w, uin
     const uint32_t want = (target + sg.chunks * ctx->L - 1) / (sg.chunks * ctx->L);
     const uint32_t groups = want < 1 ? 1 : (want > M ? M : want);
     sg.MB = (M + groups - 1) / groups;
-    const uint32_t unit = stream ? kMacThreads / kMacStreamKC * (B == 1 ? 2 : 1) : sg.MS;
+    const uint32_t rgroups = kMacThreads / kc, tiles = B & 1 ? B : B / 2;
+    const uint32_t unit = stream ? (B & 1 ? 2 : 1) * (rgroups > tiles ? rgroups / tiles : 1) : sg.MS;
     sg.MB = (sg.MB + unit - 1) / unit * unit;  // whole stages, or whole passes of the row groups, per CTA
     sg.groups = (M + sg.MB - 1) / sg.MB;
     return sg;

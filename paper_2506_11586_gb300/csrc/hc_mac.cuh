@@ -203,25 +203,25 @@ __device__ __forceinline__ bool mac_task(const MacSeg &sg, uint32_t chunk, uint3
     return true;
 }
 
-// The same sums for few blocks (RR = 2B rows a channel, B = 1 or 2) as one CTA task of NT
-// threads: the input chunk in shared memory, cut at 2^25, and the weights straight from
-// memory into registers, each once, coalesced (32 slots of a row per warp and load), four
-// terms of a tile's loads in flight.  With so few rows per weight nothing is gained by
-// staging the weights, and the layer is bound by memory once a row group waits for nobody:
-// thread (k, h) owns slot k0 + k and takes the channels m0 + h*CR ... in steps of H*CR,
-// without barriers.  Tiles of CR channels x RR rows, CR*RR = 4 sums (24 registers, so that
-// 32 warps fit an SM).  Measured on GB300, the whole layer with its transforms: 256 -> 256
-// channels at N = 16384 (G = 4, 802 MB in and out of this task) 545 us through the ring,
-// 459 streamed, of which this task is 165 us, 72 % of measured copy bandwidth; 2048 -> 1000
-// classifier (G = 24) 88 -> 76 us; 16 -> 64 channels 55x55 (B = 2) 112 -> 103 us.  Chunks of
-// 256 slots: 464, 82 and 106 us.
+// The same sums as one CTA task of NT threads without staging: the input chunk in shared
+// memory, cut at 2^25, and the weights straight from memory into registers, coalesced (32
+// slots of a row per warp and load), four terms of a tile's loads in flight.  A row group
+// waits for nobody, so a layer with few terms a sum is bound by memory.  Thread (k, h) owns
+// slot k0 + k; the H row groups take tiles of CR channels x RR of the P = 2B rows in turn
+// (RR divides P, rows fastest), CR*RR = 4 sums (24 registers, so that 32 warps fit an SM).
+// Each weight is loaded once per RR rows, from memory once and then from the caches.
+// Measured on GB300, the whole layer with its transforms: 256 -> 256 channels at N = 16384
+// (G = 4, B = 1, 802 MB in and out of this task) 545 us through the ring, 459 streamed, of
+// which this task is 165 us, 72 % of measured copy bandwidth; 2048 -> 1000 classifier
+// (G = 24, B = 1) 88 -> 76 us; 16 -> 64 channels 55x55 (B = 2) 112 -> 103 us;
+// 64 -> 64 channels 56x56 (G = 8, B = 4, through the ring 107 us for this task) 227 -> 207 us.
 template <int KC, int NT, int CR, int RR>
 __device__ __forceinline__ void mac_stream_task(const MacSeg &sg, uint32_t chunk, uint32_t limb, uint32_t m0,
                                                 uint32_t m1, uint64_t *xs)
 {
     constexpr uint32_t H = NT / KC;
     static_assert(NT % KC == 0 && KC % 32 == 0, "whole warps per row group");
-    const uint32_t G = sg.G, rows = G * RR;
+    const uint32_t G = sg.G, P = 2 * sg.B, rows = G * P;
     const size_t LN = (size_t)sg.L * sg.N, off = (size_t)limb * sg.N + chunk * KC;
     const uint32_t k = threadIdx.x % KC, h = threadIdx.x / KC;
     const uint64_t *xg = sg.X + off + k;
@@ -237,9 +237,9 @@ __device__ __forceinline__ void mac_stream_task(const MacSeg &sg, uint32_t chunk
     const size_t GLN = G * LN;
     const uint64_t *wk = sg.W + off + k;
     uint64_t *yk = sg.Y + off + k;
-    auto tile = [&](auto cr, uint32_t m) {
+    auto tile = [&](auto cr, uint32_t m, uint32_t r0) {
         constexpr int CN = decltype(cr)::value;
-        const uint64_t *w = wk + m * GLN, *xp = xs + k;
+        const uint64_t *w = wk + m * GLN, *xp = xs + r0 * KC + k;
         MacAcc25 acc[CN][RR];
 #pragma unroll
         for (int c = 0; c < CN; ++c)
@@ -251,9 +251,9 @@ __device__ __forceinline__ void mac_stream_task(const MacSeg &sg, uint32_t chunk
 #pragma unroll
             for (int g = 0; g < NG; ++g, w += LN)
 #pragma unroll
-                for (int c = 0; c < CN; ++c) wv[g][c] = __ldcs((const unsigned long long *)w + c * GLN);
+                for (int c = 0; c < CN; ++c) wv[g][c] = __ldca((const unsigned long long *)w + c * GLN);
 #pragma unroll
-            for (int g = 0; g < NG; ++g, xp += RR * KC) {
+            for (int g = 0; g < NG; ++g, xp += P * KC) {
                 uint32_t wt[CN];
 #pragma unroll
                 for (int c = 0; c < CN; ++c) {
@@ -276,15 +276,18 @@ __device__ __forceinline__ void mac_stream_task(const MacSeg &sg, uint32_t chunk
         for (int c = 0; c < CN; ++c)
 #pragma unroll
             for (int r = 0; r < RR; ++r)
-                yk[((size_t)(m + c) * RR + r) * LN] =
+                yk[((size_t)(m + c) * P + r0 + r) * LN] =
                     special ? mac25_reduce_special(acc[c][r], q, sc, p25, p28)
                             : mac25_reduce(acc[c][r], q, 0ull - q, lc.r64, lc.r64_s, (uint32_t)lc.one_s);
     };
-    for (uint32_t m = m0 + h * CR; m < m1; m += H * CR) {
+    const uint32_t tiles = P / RR;  // of a channel
+    uint32_t m = m0 + h / tiles * CR, t = h % tiles;
+    while (m < m1) {
         if (CR == 1 || m + CR <= m1)
-            tile(std::integral_constant<int, CR>{}, m);
+            tile(std::integral_constant<int, CR>{}, m, t * RR);
         else
-            tile(std::integral_constant<int, 1>{}, m);
+            tile(std::integral_constant<int, 1>{}, m, t * RR);
+        for (t += H; t >= tiles; t -= tiles) m += CR;
     }
 }
 
