@@ -212,15 +212,17 @@ hc_status ks_switch(const hc_galois_key *key, const uint64_t *a, uint64_t *u, si
 }
 
 // acc = P_steps;  acc = rot_{key(i)}(acc) + P_i, i = steps-1 .. 0;  out = acc.  Ciphertext j
-// of P_i is prods[i*by_i + j*by_j].  Each step is two launches: the key switch, then the
+// of P_i is prods[i*by_i + j*by_j]; spare: n_spare ciphertexts of memory free by now.  Each step is two launches: the key switch, then the
 // division and the addition, whose stores are already permuted for the next step.
 template <class KeyAt>
 hc_status rotate_chain(const hc_ctx *ctx, const KeyAt &key_at, const uint64_t *prods, uint32_t by_i,
-                       uint32_t by_j, uint32_t steps, size_t n, uint64_t *out, cudaStream_t s)
+                       uint32_t by_j, uint32_t steps, size_t n, uint64_t *out, uint64_t *spare,
+                       size_t n_spare, cudaStream_t s)
 {
     RotateScratch sc(s);
-    hc_status st = sc.alloc(ctx, n, steps > 1, s);
+    hc_status st = sc.alloc(ctx, n, steps > 1 && n_spare < n, s);
     if (st != HC_OK) return st;
+    if (n_spare >= n) sc.a[1] = spare;
     const size_t step = (size_t)by_i * 2 * ctx->L * ctx->N;
     const hc_galois_key *key = key_at(steps - 1);
     st = ks_apply(ctx, key, prods + steps * step, nullptr, nullptr, sc.a[0], key->g, n, s, by_j);
@@ -366,7 +368,7 @@ hc_status hc_mac_rotate_many(const hc_ctx *ctx, const hc_galois_key *key, const 
     uint64_t *first = n == 1 ? d_out : prods;  // P_0 of a one-term iteration is the result
     st = products(ctx, ctn, d_w_ntt, 1, m, n, first, s);
     if (st != HC_OK || n == 1) return st;
-    return rotate_chain(ctx, [&](uint32_t) { return key; }, prods, m, 1, n - 1, m, d_out, s);
+    return rotate_chain(ctx, [&](uint32_t) { return key; }, prods, m, 1, n - 1, m, d_out, ctn, m, s);
 }
 
 hc_status hc_mac_rotate(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *d_ct, const uint64_t *d_w_ntt,
@@ -445,7 +447,7 @@ hc_status hc_zp_conv(const hc_ctx *ctx, const hc_conv_desc *desc, const hc_galoi
     if (st != HC_OK || kk == 1) return st;
     // offsets i and i + 1 lie in one kernel row unless i + 1 starts a new one
     auto key_at = [&](uint32_t i) { return (i + 1) % desc->kw == 0 ? key_row : key_1; };
-    return rotate_chain(ctx, key_at, prods, 1, kk, kk - 1, Y, d_ct_out, s);
+    return rotate_chain(ctx, key_at, prods, 1, kk, kk - 1, Y, d_ct_out, ctn, C, s);
 }
 
 }  // extern "C"
