@@ -7,7 +7,7 @@
 // by the key and summed in registers, and the two sums are transformed back; digits and
 // products never go to memory (L (L+1) + 2 (L+1) polynomials of a ciphertext written and
 // read again by separate transform and multiply kernels).  A transform of N residues
-// is split as in k_ntt_fwd_pair: the first LOGP forward stages pair residues N / 2^LOGP
+// is split as in hc_split.cuh: the first LOGP forward stages pair residues N / 2^LOGP
 // apart, each CTA computes them for its slice of the pairs and writes the results into
 // the CTA that owns them (distributed shared memory), the rest is local to the CTA;
 // the inverse runs the other way round.  2^LOGP CTAs per unit are for latency: the

@@ -163,7 +163,7 @@ __device__ __forceinline__ void static_for(F &&f)
 
 // ---- one forward round: K Cooley-Tukey stages in registers ---------------------
 // PART > 0: the transform is one of the 2^PART parts of a larger transform after that
-// transform's first PART stages (see k_ntt_fwd_pair, k_ks_switch): local stage s,
+// transform's first PART stages (see k_ntt_fwd_pair, hc_split.cuh): local stage s,
 // group i uses the full table's entry tmul*2^s + i, tmul = 2^PART + the part's
 // index; every round reads the natural table.
 template <class Cfg, int R, int SIG, int PART, bool SP>
@@ -214,7 +214,7 @@ __device__ __forceinline__ void fwd_round(uint64_t (&x)[Cfg::NP][Cfg::C], const 
 
 // ---- one inverse round: K Gentleman-Sande stages in registers ------------------
 // PART > 0: the transform is one of the 2^PART parts of a larger transform, before
-// that transform's last PART stages (see k_ntt_inv_pair, k_ks_switch): stage s, group
+// that transform's last PART stages (see hc_split.cuh): stage s, group
 // i uses the full table's entry tmul*(N >> (s+1)) + i (N this transform's size, tmul =
 // 2^PART + the part's index); every round reads the natural table and no stage is the
 // last.
