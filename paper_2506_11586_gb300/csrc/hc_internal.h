@@ -395,7 +395,7 @@ constexpr int KK_FWDCT_SEGS = 100, KK_INVCT_SEGS = 101, KK_INV_EXTRACT = 102;
 constexpr int KK_PROD_SPLIT = 103;
 // Most units (polynomial limbs; limbs of a product) that run split over clusters of eight.
 // Measured on GB300, us, split / one CTA (pair) per unit, both as programmatic dependents:
-//   forward  N = 4096:  32 limbs 4.9 / 6.3   76: 7.1 / 6.3
+//   forward  N = 4096:  32 limbs 4.9 / 6.3   76: 7.1 / 6.3   128: 7.5 / 8.3 (12.3 launched early)
 //            N = 8192:  24: 6.7 / 11   96: 9.7 / 18   153: 15.9 / 18   240: 21 / 20
 //            N = 16384: 32: 10 / 21    64: 16 / 21    96: 19 / 21
 //   inverse  N = 8192:  24: 7.6 / 11   96: 11 / 18    192: 18.9 / 18.8
@@ -403,7 +403,7 @@ constexpr int KK_PROD_SPLIT = 103;
 //   product  N = 4096:  16 limbs 8.3 / 23   48: 10.5 / 23   64: 17 / 16
 //            N = 8192:  12: 11.5 / 41  72: 29 / 41    96: 37 / 41
 //            N = 16384: 4: 14.7 / 45   32: 43 / 46    64: 72 / 46
-constexpr uint32_t split_units_ntt(uint32_t logn, uint32_t sms) { return sms * (logn == 12 ? 3 : logn == 13 ? 8 : 4) / 8; }
+constexpr uint32_t split_units_ntt(uint32_t logn, uint32_t sms) { return sms * (logn == 12 ? 7 : logn == 13 ? 8 : 4) / 8; }
 constexpr uint32_t split_units_product(uint32_t logn, uint32_t sms) { return sms * (logn == 12 ? 3 : logn == 13 ? 4 : 2) / 8; }
 
 

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 P45 = 35184371138561  # prime, 1 mod 2^15: no folded twiddles
-NTT_LIMBS = {4096: 3, 8192: 8, 16384: 4}      # eighths of the SM count
+NTT_LIMBS = {4096: 7, 8192: 8, 16384: 4}      # eighths of the SM count
 PRODUCT_LIMBS = {4096: 3, 8192: 4, 16384: 2}
 
 
