@@ -407,6 +407,10 @@ constexpr uint32_t split_units_ntt(uint32_t logn, uint32_t sms) { return sms * (
 constexpr uint32_t split_units_product(uint32_t logn, uint32_t sms) { return sms * (logn == 12 ? 3 : logn == 13 ? 4 : 2) / 8; }
 
 
+// What kernels read or store as pairs of residues must lie on 16 bytes; callers' buffers need
+// not (inputs are read, and most outputs stored, word by word).
+inline bool odd_word(const void *p) { return ((uintptr_t)p & 15) != 0; }
+
 // arguments of one launch of a kernel family (unused fields ignored)
 struct LaunchArgs {
     const NttSegs *segs;

@@ -885,6 +885,26 @@ bool try_ntt_split(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaStream_
     return true;
 }
 
+// Inverse transforms at N >= 8192 whose input lies on an odd word, in any variant: the
+// prefetching kernel copies it word by word, the others load pairs.
+template <int LOGN, bool SP>
+hc_status launch_inv_odd(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaStream_t s)
+{
+    if (kind == KK_INVCT_SEGS) {
+        NttSegs segs = *a.segs;
+        uint32_t begin = 0;
+        for (uint32_t i = 0; i < segs.n; ++i) {
+            segs.s[i].n_groups *= 2;  // polynomials
+            segs.s[i].cta_begin = begin;
+            begin += segs.s[i].n_groups * seg_limbs(segs.s[i]);
+        }
+        return detail::run_ntt_inv_pf<typename InvPf<LOGN>::Cfg, SP>(segs, s);
+    }
+    const size_t polys = kind == KK_INV ? a.n : 2 * a.n;
+    if (polys * ctx->L > 0x7fffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
+    return detail::run_ntt_inv_pf<typename InvPf<LOGN>::Cfg, SP>(detail::one_seg(ctx, a.in, a.out, polys), s);
+}
+
 template <int LOGN, int V, bool SP>
 hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaStream_t s)
 {
@@ -976,6 +996,11 @@ hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaS
 template <int LOGN, bool SP>
 hc_status launch_n(const hc_ctx *ctx, int kind, int variant, const LaunchArgs &a, cudaStream_t s)
 {
+    if constexpr (LOGN >= 13) {
+        bool odd = (kind == KK_INV || kind == KK_INVCT) && odd_word(a.in);
+        for (uint32_t i = 0; kind == KK_INVCT_SEGS && i < a.segs->n; ++i) odd = odd || odd_word(a.segs->s[i].in);
+        if (odd) return launch_inv_odd<LOGN, SP>(ctx, kind, a, s);
+    }
     switch (variant) {
     case 0: return launch_variant<LOGN, 0, SP>(ctx, kind, a, s);
     case 1: return launch_variant<LOGN, 1, SP>(ctx, kind, a, s);

@@ -195,7 +195,7 @@ bool mac_conv_fits(uint32_t G, uint32_t B)
 hc_status launch_mac_conv(const hc_ctx *ctx, const uint64_t *x_ntt, const uint64_t *w_ntt, uint64_t *y, uint32_t G,
                           uint32_t B, uint32_t M, cudaStream_t s)
 {
-    if (ctx->variant[KK_MACB] == kMacTcVariant && mac_tc_fits(G, B))
+    if (ctx->variant[KK_MACB] == kMacTcVariant && mac_tc_fits(G, B) && !odd_word(y))
         return launch_mac_tc(ctx, x_ntt, w_ntt, y, G, B, M, 0, 0, s);
     if (!mac_conv_fits(G, B) || ctx->N % 64) return set_error(HC_ERR_UNSUPPORTED, "blocked MAC does not fit");
     MacSegs1 segs{};
@@ -206,7 +206,7 @@ hc_status launch_mac_conv(const hc_ctx *ctx, const uint64_t *x_ntt, const uint64
 
 static bool use_tc(const hc_ctx *ctx, const MacLayer &ly)
 {
-    return ctx->variant[KK_MACB] == kMacTcVariant && mac_tc_fits(ly.G, ly.B);
+    return ctx->variant[KK_MACB] == kMacTcVariant && mac_tc_fits(ly.G, ly.B) && !odd_word(ly.y);
 }
 
 hc_status launch_mac_conv_layers(const hc_ctx *const *ctxs, const MacLayer *layers, size_t n, cudaStream_t s)

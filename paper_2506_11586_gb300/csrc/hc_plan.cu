@@ -153,10 +153,11 @@ uint32_t count_launches(const hc_plan *p)
     for (uint32_t d = 0; d < 3; ++d) {
         uint32_t cnt = 0, maxl = 0;
         const PlanConv *first = nullptr;
-        bool form[2] = {false, false};
+        bool form[2] = {false, false}, odd = false;
         for (const PlanConv &c : p->convs)
             if (c.ctx->logN == 12 + d && c.blocked) {
                 if (!first) first = &c;
+                odd = odd || odd_word(c.out);
                 form[c.ctx->fold ? 1 : 0] = true;
                 if (c.ctx->L > maxl) maxl = c.ctx->L;
                 ++cnt;
@@ -167,7 +168,7 @@ uint32_t count_launches(const hc_plan *p)
                 n += count_groups(p, [&](const PlanConv &c) { return c.ctx->logN == 12 + d && c.blocked && c.ctx->L > l; },
                                   2, true);
             fused[d] = true;
-        } else if (first->ctx->variant[KK_CONV] == 1 && cnt <= (uint32_t)kFusedMaxLayers && p->d_ctr) {
+        } else if (first->ctx->variant[KK_CONV] == 1 && cnt <= (uint32_t)kFusedMaxLayers && p->d_ctr && !odd) {
             n += (uint32_t)form[0] + (uint32_t)form[1];
             fused[d] = true;
         }
@@ -444,9 +445,11 @@ hc_status launch_conv_jobs(const ConvJob *jobs, size_t n, cudaStream_t s, uint32
     for (uint32_t logN = 12; logN <= 14; ++logN) {
         const ConvJob *first = nullptr;
         size_t count = 0;
+        bool odd = false;
         for (size_t i = 0; i < n; ++i)
             if (jobs[i].ctx->logN == logN && jobs[i].blocked) {
                 if (!first) first = &jobs[i];
+                odd = odd || odd_word(jobs[i].out);
                 ++count;
             }
         if (!first) continue;
@@ -456,7 +459,7 @@ hc_status launch_conv_jobs(const ConvJob *jobs, size_t n, cudaStream_t s, uint32
             fused[logN - 12] = true;
             continue;
         }
-        if (first->ctx->variant[KK_CONV] != 1 || count > (size_t)kFusedMaxLayers || !ctr) continue;
+        if (first->ctx->variant[KK_CONV] != 1 || count > (size_t)kFusedMaxLayers || !ctr || odd) continue;
         const size_t words = fused_counter_words(jobs, n, logN);
         if (words > ctr_words) continue;
         hc_status st = launch_conv_fused(jobs, n, logN, ctr, s);
