@@ -16,6 +16,12 @@
  *     Coefficient-domain arrays are in natural order.  NTT-domain arrays hold
  *     slot k = a(psi_i^(2*rev(k)+1)) mod q_i, where rev reverses log2(N) bits
  *     and psi_i is the smallest primitive 2N-th root of unity mod q_i.
+ *   - Alignment: device buffers lie on 8 bytes (an input or output ciphertext
+ *     may start at any word).  On 16 bytes must lie: NTT-domain operands
+ *     (d_pt_ntt, d_w_ntt), the polynomials of hc_ntt_fwd, the d_out of the Z_P
+ *     preprocessing calls, and at N = 4096 also the polynomials of hc_ntt_inv,
+ *     the d_poly of hc_zp_encode and the outputs of convolutions with a blocked
+ *     MAC.  What is not, is refused with HC_ERR_INVALID_ARG.
  *   - Ranges: inputs must be canonical residues in [0, q_i); outputs are
  *     canonical.  Inputs are not range-checked unless the context was created
  *     with HC_CTX_CHECKED, in which case an out-of-range input makes the call

@@ -1048,6 +1048,7 @@ hc_status hc_ctpt_mac(const hc_ctx *ctx, const uint64_t *d_ct, const uint64_t *d
     if (n_out == 0) return HC_OK;
     if (!d_out) return set_error(HC_ERR_INVALID_ARG, "d_out is NULL");
     if (n > 0 && (!d_ct || !d_pt_ntt || !h_slot)) return set_error(HC_ERR_INVALID_ARG, "null input");
+    if (n > 0 && odd_word(d_pt_ntt)) return set_error(HC_ERR_INVALID_ARG, "d_pt_ntt is not aligned to 16 bytes");
     if (n > 0xffffffffull || n_out > 0xffffffffull) return set_error(HC_ERR_INVALID_ARG, "batch too large");
     std::vector<uint32_t> count(n_out, 0);
     for (size_t j = 0; j < n; ++j) {

@@ -275,6 +275,22 @@ hc_status after(const char *what)
     return e == cudaSuccess ? HC_OK : cuda_error(e, what);
 }
 
+// an operand that the kind's kernels take in pairs lies on an odd word (segment tables: checked
+// by launch_conv_jobs)
+bool odd_operand(const hc_ctx *ctx, int kind, const LaunchArgs &a)
+{
+    switch (kind) {
+    case KK_FWD:
+    case KK_FWDCT: return odd_word(a.out);
+    case KK_INV:
+    case KK_INVCT: return ctx->logN < 13 && odd_word(a.in);  // above: launch_inv_odd
+    case KK_MAC: return odd_word(a.in) || odd_word(a.pt);
+    case KK_PROD:
+    case KK_PROD_SPLIT: return odd_word(a.pt);
+    default: return false;
+    }
+}
+
 hc_status dispatch(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaStream_t s)
 {
     const int v = kind == KK_FWDCT_SEGS    ? ctx->variant[KK_FWDCT]
@@ -282,6 +298,7 @@ hc_status dispatch(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaStream_
                   : kind == KK_INV_EXTRACT ? ctx->variant[KK_INVCT]
                   : kind == KK_PROD_SPLIT  ? 0
                                            : ctx->variant[kind];
+    if (a.n && odd_operand(ctx, kind, a)) return set_error(HC_ERR_INVALID_ARG, "buffer not aligned to 16 bytes");
     const bool fold = a.segs ? a.segs->s[0].fold != 0 : ctx->fold;
     switch (ctx->logN) {
     case 12: return fold ? launch_n<12, true>(ctx, kind, v, a, s) : launch_n<12, false>(ctx, kind, v, a, s);

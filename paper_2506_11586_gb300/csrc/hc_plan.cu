@@ -440,6 +440,10 @@ size_t conv_jobs_counter_words(const ConvJob *jobs, size_t n)
 // the batched launch sequence of n conv jobs (all degrees), in stream order on s
 hc_status launch_conv_jobs(const ConvJob *jobs, size_t n, cudaStream_t s, uint32_t *ctr, size_t ctr_words)
 {
+    // outputs on odd words: the inverse transforms at N >= 8192 take them (launch_inv_odd)
+    for (size_t i = 0; i < n; ++i)
+        if (jobs[i].ctx->logN == 12 && jobs[i].blocked && odd_word(jobs[i].out))
+            return set_error(HC_ERR_INVALID_ARG, "output ciphertexts not aligned to 16 bytes");
     // degrees whose blocked jobs run as one fused persistent launch
     bool fused[3] = {false, false, false};
     for (uint32_t logN = 12; logN <= 14; ++logN) {
@@ -577,6 +581,7 @@ hc_status hc_plan_create(const hc_work_item *items, size_t n, hc_plan **out)
                 return set_error(HC_ERR_UNSUPPORTED, "item %zu: plans need NTT-preprocessed (offline) weights", i);
         } else if (it.kind == HC_WORK_PRODUCTS) {
             if (it.n == 0 || !it.d_pt_ntt) return set_error(HC_ERR_INVALID_ARG, "item %zu: empty product list", i);
+            if (odd_word(it.d_pt_ntt)) return set_error(HC_ERR_INVALID_ARG, "item %zu: d_pt_ntt not aligned to 16 bytes", i);
         } else {
             return set_error(HC_ERR_INVALID_ARG, "item %zu: unknown kind %u", i, it.kind);
         }

@@ -163,15 +163,16 @@ struct RotateScratch {
 
 // out[m*B + b] = INTT(sum_g x[g*B + b] . w[m*G + g]), x forward transformed.  The blocked
 // MAC reads each weight once and sums at the multiply pipe's rate, and the inverse
-// transforms run as a launch of their own; k_mac_intt, which reads its terms word by word
-// from each output's CTA, stays for what does not fit or is not aligned.  Measured on GB300,
+// transforms run as a launch of their own; k_mac_intt, which reads its terms pair by pair
+// from each output's CTA and stores word by word, stays for what does not fit and for an
+// output on an odd word.  Measured on GB300,
 // N = 8192, L = 3: a layer of 288 outputs of 16 terms and its rotations 1011 us with
 // k_mac_intt (376 us of it), 929 so; an iteration of 16 products 281 and 271 us.
 hc_status products(const hc_ctx *ctx, const uint64_t *x, const uint64_t *w, uint32_t G, uint32_t B, uint32_t M,
                    uint64_t *out, cudaStream_t s)
 {
     const uint32_t n_out = M * B;
-    if (mac_conv_fits(G, B) && (((uintptr_t)w | (uintptr_t)out) & 15) == 0) {
+    if (mac_conv_fits(G, B) && !odd_word(out)) {
         const hc_status st = launch_mac_conv(ctx, x, w, out, G, B, M, s);
         return st == HC_OK ? launch_ntt_inv_ct(ctx, out, out, n_out, s) : st;
     }
@@ -347,6 +348,7 @@ hc_status hc_mac_rotate_many(const hc_ctx *ctx, const hc_galois_key *key, const 
     if (key->ctx != ctx) return set_error(HC_ERR_INVALID_ARG, "key was made for another context");
     if (!d_ct || !d_w_ntt || !d_out || n == 0 || m == 0) return set_error(HC_ERR_INVALID_ARG, "null buffer or empty batch");
     if ((uint64_t)n * m > 0x3fffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
+    if (odd_word(d_w_ntt)) return set_error(HC_ERR_INVALID_ARG, "d_w_ntt is not aligned to 16 bytes");
     DeviceGuard dg(ctx->device);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
     hc_status st = check_inputs(ctx, d_ct, (size_t)2 * m, s);
@@ -425,6 +427,7 @@ hc_status hc_zp_conv(const hc_ctx *ctx, const hc_conv_desc *desc, const hc_galoi
                          grow);
     const uint64_t n_out64 = (uint64_t)kk * Y;
     if (n_out64 * C > 0x3fffffffu) return set_error(HC_ERR_INVALID_ARG, "layer too large");
+    if (odd_word(d_w_ntt)) return set_error(HC_ERR_INVALID_ARG, "d_w_ntt is not aligned to 16 bytes");
     const uint32_t n_out = (uint32_t)n_out64;
     DeviceGuard dg(ctx->device);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);

@@ -69,3 +69,46 @@ def test_layer_on_odd_words(L, N, nl, M):
             L.hc_ctx_device_status(ctx)
             assert torch.equal(out, ref), (form, mac)
             assert t[0] == -1 and t[-1] == -1
+
+
+def test_operands_taken_in_pairs_are_refused(L):
+    """Odd words where the kernels take pairs: an error before the launch, and the context goes on."""
+    N, moduli = 4096, CANONICAL_PRIMES[:2]
+    ctx = L.hc_ctx_create(N, moduli, T_PLAIN)
+    s = Stream(33, 1)
+    ct = to_dev(uniform_residues(s, moduli, (2, 2), N))
+    pt = to_dev(uniform_residues(s, moduli, (2,), N))
+    _, pt_odd = _odd(pt.numel(), pt)
+    _, ct_odd = _odd(ct.numel(), ct)
+    out = torch.full((ct.numel(),), 7, dtype=torch.int64, device="cuda")
+    gk = np.stack([np.stack([np.stack([s.below(q, N) for q in CANONICAL_PRIMES[:3]]) for _ in range(2)]) for _ in range(2)])
+    key = L.hc_galois_key_create(ctx, CANONICAL_PRIMES[2], 5, gk)
+    desc = L.make_desc(1, 4, 4, 2, 1, 2)
+    w = L.hc_weights_preprocess(ctx, L.make_desc(2, 6, 6, 3, 3, 3), s.int8(54).reshape(3, 2, 3, 3))
+    wi = to_dev(uniform_residues(s, moduli, (w.I, 2), N))
+    _, w_out = _odd(w.O * 4 * N)
+    calls = {
+        "fwd": lambda: L.hc_ntt_fwd(ctx, pt_odd),
+        "inv": lambda: L.hc_ntt_inv(ctx, pt_odd),
+        "products": lambda: L.hc_ctpt_mac(ctx, ct, pt_odd, np.array([0, 1]), out),
+        "sums": lambda: L.hc_ctpt_mac(ctx, ct, pt_odd, np.array([0, 0]), out),
+        "iteration": lambda: L.hc_mac_rotate(ctx, key, ct[0], pt_odd, out[:4 * N]),
+        "zp conv": lambda: L.hc_zp_conv(ctx, desc, key, None, pt_odd, ct[0], out[:4 * N]),
+        "plan": lambda: L.hc_plan_create([L.work_products(ctx, ct, pt_odd, out)]),
+        "layer": lambda: L.hc_conv_ct_pt(ctx, w, wi, w_out),
+    }
+    for name, call in calls.items():
+        with pytest.raises(L.HcError) as e:
+            call()
+        assert e.value.status == L.HC_ERR_INVALID_ARG, name
+    torch.cuda.synchronize()
+    assert torch.all(out == 7) and torch.all(w_out == -1)
+    # ciphertexts may lie anywhere
+    ref = torch.empty_like(out)
+    L.hc_ctpt_mac(ctx, ct, pt, np.array([0, 1]), ref)
+    t, out_odd = _odd(ct.numel())
+    L.hc_ctpt_mac(ctx, ct_odd, pt, np.array([0, 1]), out_odd)
+    assert torch.equal(out_odd, ref) and t[0] == -1 and t[-1] == -1
+    L.hc_mac_rotate(ctx, key, ct[0], pt, ref[:4 * N])
+    L.hc_mac_rotate(ctx, key, ct_odd[:4 * N], pt, out_odd[:4 * N])
+    assert torch.equal(out_odd[:4 * N], ref[:4 * N])
