@@ -150,6 +150,16 @@ __device__ __forceinline__ uint64_t ld_data(const uint64_t *p)
 }
 __device__ __forceinline__ ulonglong2 ld_data(const ulonglong2 *p) { return __ldcg(p); }
 
+// an ordinary load, through L1, for what several warps or CTAs of an SM read (the sums' term
+// lists and operands, weights).  p must not come from a __restrict__ parameter, which would
+// make it a read-only one.  Sums of four products through L2 instead, 64 of them at
+// N = 16384, L = 4, into 16: 131 -> 169 us.
+template <class T>
+__device__ __forceinline__ T ld_near(const T *p)
+{
+    return *p;
+}
+
 // host: launch kern, as the programmatic dependent of the launch before it if asked to
 template <class... P, class... A>
 cudaError_t launch_programmatic(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool dependent,

@@ -244,9 +244,8 @@ k_ntt_inv_extract(const __grid_constant__ ExtractArgs ex, const LimbConst *__res
 // consecutive CTAs (consecutive outputs) share weight polynomials in L2.
 template <class Cfg, bool SP>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
-k_mac_intt(const uint64_t *__restrict__ ct_ntt, const uint64_t *__restrict__ pt_ntt,
-           const uint32_t *__restrict__ term_ptr, const uint32_t *__restrict__ terms,
-           uint64_t *__restrict__ out, const LimbConst *__restrict__ limbs, uint32_t L,
+k_mac_intt(const uint64_t *ct_ntt, const uint64_t *pt_ntt, const uint32_t *term_ptr, const uint32_t *terms,
+           uint64_t *out, const LimbConst *__restrict__ limbs, uint32_t L,
            uint32_t n_groups)
 {
     extern __shared__ uint64_t sm[];
@@ -260,7 +259,7 @@ k_mac_intt(const uint64_t *__restrict__ ct_ntt, const uint64_t *__restrict__ pt_
     const LimbConst &lc = limbs[limb];
     const uint64_t q = lc.q, nq = 0ull - q, r64 = lc.r64, r64_s = lc.r64_s;
     const uint32_t ones = (uint32_t)lc.one_s;
-    const uint32_t t0 = __ldcg(term_ptr + o), t1 = __ldcg(term_ptr + o + 1);
+    const uint32_t t0 = ld_near(term_ptr + o), t1 = ld_near(term_ptr + o + 1);
 
     // MAC in the coalesced pair layout: thread tid owns residue pairs
     // e = 2*(tid + r*T), so each warp-wide 16-byte load covers 512 contiguous
@@ -275,18 +274,34 @@ k_mac_intt(const uint64_t *__restrict__ ct_ntt, const uint64_t *__restrict__ pt_
             mac_zero(acc[p][0]);
             mac_zero(acc[p][1]);
         }
-#pragma unroll 4
-        for (uint32_t t = t0; t < t1; ++t) {
-            const uint32_t ci = __ldcg(terms + 2 * t), pi = __ldcg(terms + 2 * t + 1);
-            const ulonglong2 w = ld_data(reinterpret_cast<const ulonglong2 *>(pt_ntt + (size_t)pi * L * N + limb_off + e));
+        auto terms_of = [&](uint32_t t, auto ng) {  // ng terms, their loads first
+            constexpr int NG = decltype(ng)::value;
+            uint32_t ci[NG], pi[NG];
 #pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                const ulonglong2 xv = ld_data(reinterpret_cast<const ulonglong2 *>(
-                    ct_ntt + ((size_t)ci * 2 + comp0 + p) * L * N + limb_off + e));
-                mac_add(acc[p][0], xv.x, w.x);
-                mac_add(acc[p][1], xv.y, w.y);
+            for (int k = 0; k < NG; ++k) {
+                ci[k] = ld_near(terms + 2 * (t + k));
+                pi[k] = ld_near(terms + 2 * (t + k) + 1);
             }
-        }
+            ulonglong2 w[NG], xv[NG][NP];
+#pragma unroll
+            for (int k = 0; k < NG; ++k) {
+                w[k] = ld_near(reinterpret_cast<const ulonglong2 *>(pt_ntt + (size_t)pi[k] * L * N + limb_off + e));
+#pragma unroll
+                for (int p = 0; p < NP; ++p)
+                    xv[k][p] = ld_near(reinterpret_cast<const ulonglong2 *>(
+                        ct_ntt + ((size_t)ci[k] * 2 + comp0 + p) * L * N + limb_off + e));
+            }
+#pragma unroll
+            for (int k = 0; k < NG; ++k)
+#pragma unroll
+                for (int p = 0; p < NP; ++p) {
+                    mac_add(acc[p][0], xv[k][p].x, w[k].x);
+                    mac_add(acc[p][1], xv[k][p].y, w[k].y);
+                }
+        };
+        uint32_t t = t0;
+        for (; t + 4 <= t1; t += 4) terms_of(t, std::integral_constant<int, 4>{});
+        for (; t < t1; ++t) terms_of(t, std::integral_constant<int, 1>{});
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
             sm[p * Cfg::SW + spos<Cfg>(e)] = mac_reduce(acc[p][0], q, nq, r64, r64_s, ones);
@@ -546,9 +561,8 @@ k_ntt_fwd_pair(const __grid_constant__ NttSegsT<NS> segs)
 // plaintext [L][N], out its output ciphertext [2][L][N]:
 //   out[c][limb] (+)= INTT(NTT(ct[c][limb]) . pt[limb])                  (App. C.1)
 template <class Cfg, bool SP>
-__device__ __forceinline__ void product_task(uint64_t *sm, const uint64_t *__restrict__ ct,
-                                             const uint64_t *__restrict__ pt, uint64_t *out, const LimbConst &lc,
-                                             uint32_t L, uint32_t limb, uint32_t comp0, bool accumulate)
+__device__ __forceinline__ void product_task(uint64_t *sm, const uint64_t *ct, const uint64_t *pt,
+                                             uint64_t *out, const LimbConst &lc, uint32_t L, uint32_t limb, uint32_t comp0, bool accumulate)
 {
     constexpr int NP = Cfg::NP, C = Cfg::C, T = Cfg::T, N = Cfg::N;
     const int tid = threadIdx.x;
@@ -566,7 +580,7 @@ __device__ __forceinline__ void product_task(uint64_t *sm, const uint64_t *__res
     const ulonglong2 *wp = reinterpret_cast<const ulonglong2 *>(pt + (size_t)limb * N + tid * C);
 #pragma unroll
     for (int r = 0; r < C / 2; ++r) {
-        const ulonglong2 w = ld_data(wp + r);
+        const ulonglong2 w = ld_near(wp + r);
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
             x[p][2 * r] = mul_slot(ar, x[p][2 * r], w.x, lc.r64, lc.r64_s);
@@ -593,8 +607,8 @@ __device__ __forceinline__ void product_task(uint64_t *sm, const uint64_t *__res
 
 template <class Cfg, bool SP>
 __global__ void __launch_bounds__(Cfg::T, Cfg::MINB)
-k_product(const uint64_t *__restrict__ ct, const uint64_t *__restrict__ pt_ntt,
-          const uint32_t *__restrict__ out_index, uint64_t *out, const LimbConst *__restrict__ limbs,
+k_product(const uint64_t *ct, const uint64_t *pt_ntt, const uint32_t *out_index, uint64_t *out,
+          const LimbConst *__restrict__ limbs,
           uint32_t L, uint32_t n_groups, int accumulate)
 {
     extern __shared__ uint64_t sm[];
@@ -604,7 +618,7 @@ k_product(const uint64_t *__restrict__ ct, const uint64_t *__restrict__ pt_ntt,
     const uint32_t limb = blockIdx.x / n_groups, grp = blockIdx.x % n_groups;
     const uint32_t j = grp / CPG;
     const uint32_t comp0 = (grp % CPG) * Cfg::NP;
-    const uint32_t oj = out_index ? __ldcg(out_index + j) : j;
+    const uint32_t oj = out_index ? ld_near(out_index + j) : j;
     product_task<Cfg, SP>(sm, ct + (size_t)j * 2 * L * N, pt_ntt + (size_t)j * L * N, out + (size_t)oj * 2 * L * N,
                       limbs[limb], L, limb, comp0, accumulate != 0);
 }
