@@ -142,14 +142,21 @@ __device__ __forceinline__ void pdl_begin()
     pdl_wait();
 }
 
-// loads of what an earlier launch, or another CTA of this one, may have written: through
-// L2, and never on the read-only path, whose loads the compiler may move above the wait
+// Loads of what an earlier launch, or another CTA of this one, may have written: through L2,
+// and never on the read-only path, whose loads the compiler may move above the wait.  It may
+// move the load intrinsic too, which it does not see touching memory, unless the address
+// comes from after_wait.
+template <class T>
+__device__ __forceinline__ const T *after_wait(const T *p)
+{
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
 __device__ __forceinline__ uint64_t ld_data(const uint64_t *p)
 {
     return __ldcg((const unsigned long long *)p);
 }
 __device__ __forceinline__ ulonglong2 ld_data(const ulonglong2 *p) { return __ldcg(p); }
-
 // an ordinary load, through L1, for what several warps or CTAs of an SM read (the sums' term
 // lists and operands, weights).  p must not come from a __restrict__ parameter, which would
 // make it a read-only one.  Sums of four products through L2 instead, 64 of them at

@@ -98,6 +98,7 @@ __device__ __forceinline__ void fwd_task(uint64_t *sm, const uint64_t *src, uint
                                          const LimbConst &lc, int tid)
 {
     constexpr int NP = Cfg::NP, C = Cfg::C, T = Cfg::T, N = Cfg::N;
+    src = after_wait(src);
     uint64_t x[NP][C];
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
@@ -132,6 +133,7 @@ __device__ __forceinline__ void inv_core(uint64_t (&x)[Cfg::NP][Cfg::C], uint64_
                                          size_t pstride, const LimbConst &lc, int tid)
 {
     constexpr int NP = Cfg::NP, C = Cfg::C, N = Cfg::N;
+    src = after_wait(src);
     // coalesced 16-byte loads into shared memory, then the round-0 layout
     // (element tid*C + r) out of it
 #pragma unroll
@@ -517,7 +519,7 @@ k_ntt_fwd_pair(const __grid_constant__ NttSegsT<NS> segs)
     const uint32_t local = unit - sg.cta_begin;
     const uint32_t limb = sg.limb0 + local / sg.n_groups, poly = local % sg.n_groups;
     const size_t off = ((size_t)poly * sg.L + limb) * (2 * (size_t)NH);
-    const uint64_t *src = sg.in + off;
+    const uint64_t *src = after_wait(sg.in + off);
     const LimbConst &lc = sg.limbs[limb];
     const ulonglong2 w = __ldg(lc.tw_f + 1);
     const uint32_t to0 = cluster_map(sm, 0), to1 = cluster_map(sm, 1);
@@ -567,7 +569,7 @@ __device__ __forceinline__ void product_task(uint64_t *sm, const uint64_t *ct, c
     constexpr int NP = Cfg::NP, C = Cfg::C, T = Cfg::T, N = Cfg::N;
     const int tid = threadIdx.x;
     const uint64_t q = lc.q;
-
+    ct = after_wait(ct);
     uint64_t x[NP][C];
 #pragma unroll
     for (int p = 0; p < NP; ++p) {

@@ -86,7 +86,7 @@ k_ks_switch(const KsArgs args)
     cluster_sync();  // every CTA of the cluster is running before one writes into another
     pdl_begin();
 
-    const uint64_t *c1 = args.a + (size_t)(2 * ct + 1) * L * N;
+    const uint64_t *c1 = after_wait(args.a) + (size_t)(2 * ct + 1) * L * N;
     for (uint32_t j = first; j < L; j += NG * NP) {
         if (j + NP <= L)
             split_fwd_cross<S, NP, SP>(c1 + j * N, N, sm, j * NL, slice, lc, ar);

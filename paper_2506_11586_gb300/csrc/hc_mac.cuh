@@ -224,7 +224,7 @@ __device__ __forceinline__ void mac_stream_task(const MacSeg &sg, uint32_t chunk
     const uint32_t G = sg.G, P = 2 * sg.B, rows = G * P;
     const size_t LN = (size_t)sg.L * sg.N, off = (size_t)limb * sg.N + chunk * KC;
     const uint32_t k = threadIdx.x % KC, h = threadIdx.x / KC;
-    const uint64_t *xg = sg.X + off + k;
+    const uint64_t *xg = after_wait(sg.X + off + k);
     for (uint32_t r = h; r < rows; r += H) xs[r * KC + k] = split25(ld_data(xg + r * LN));
     const LimbConst &lc = sg.limbs[limb];
     const uint64_t q = lc.q;
@@ -251,7 +251,7 @@ __device__ __forceinline__ void mac_stream_task(const MacSeg &sg, uint32_t chunk
 #pragma unroll
             for (int g = 0; g < NG; ++g, w += LN)
 #pragma unroll
-                for (int c = 0; c < CN; ++c) wv[g][c] = __ldca((const unsigned long long *)w + c * GLN);
+                for (int c = 0; c < CN; ++c) wv[g][c] = ld_near(w + c * GLN);
 #pragma unroll
             for (int g = 0; g < NG; ++g, xp += P * KC) {
                 uint32_t wt[CN];

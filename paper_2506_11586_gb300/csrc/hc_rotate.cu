@@ -67,6 +67,9 @@ k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *
            uint32_t g, uint32_t rows, uint32_t a_ct, uint32_t add_ct)
 {
     pdl_begin();
+    a = after_wait(a);
+    u = after_wait(u);
+    add = after_wait(add);
     const uint32_t k = 2 * (blockIdx.x * kKsBlock + threadIdx.x);
     const uint32_t mask2 = 2 * N - 1, L1 = L + 1;
     const uint64_t half = (special - 1) / 2;

@@ -158,7 +158,7 @@ k_ntt_fwd_split(const __grid_constant__ NttSegsT<NS> segs)
     const TwArith<SP> ar = tw_arith<SP>(lc);
     cluster_sync();  // every CTA of the cluster is running before one writes into another
     pdl_begin();
-    split_fwd_cross<S, 1, SP>(sg.in + off, 0, sm, 0, rank * (NL / S::CS) + tid, lc, ar);
+    split_fwd_cross<S, 1, SP>(after_wait(sg.in) + off, 0, sm, 0, rank * (NL / S::CS) + tid, lc, ar);
     cluster_sync();  // this CTA's part is complete, and every load of an in-place transform done
     uint64_t x[1][C];
 #pragma unroll
@@ -186,7 +186,7 @@ k_ntt_inv_split(const __grid_constant__ NttSegsT<NS> segs)
     const LimbConst &lc = sg.limbs[limb];
     const TwArith<SP> ar = tw_arith<SP>(lc);
     pdl_begin();
-    const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(sg.in + off + rank * NL + tid * C);
+    const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(after_wait(sg.in + off + rank * NL + tid * C));
     uint64_t x[1][C];
 #pragma unroll
     for (int r = 0; r < C; r += 2) {
@@ -219,7 +219,7 @@ struct SlotList {
 //   out[slot][c] (+)= INTT(NTT(ct[j][c]) . pt[j])                              (App. C.1)
 template <class S, bool SP>
 __global__ void __cluster_dims__(S::CS, 1, 1) __launch_bounds__(S::THREADS, S::MINB)
-k_product_split(const uint64_t *__restrict__ ct, const uint64_t *__restrict__ pt, uint64_t *out,
+k_product_split(const uint64_t *ct, const uint64_t *pt, uint64_t *out,
                 const LimbConst *__restrict__ limbs, uint32_t L, int accumulate,
                 const __grid_constant__ SlotList slots)
 {
@@ -238,13 +238,14 @@ k_product_split(const uint64_t *__restrict__ ct, const uint64_t *__restrict__ pt
     uint64_t *b = sm + comp * NL;
     cluster_sync();  // every CTA of the cluster is running before one writes into another
     pdl_begin();
-    split_fwd_cross<S, 1, SP>(ct + ((size_t)(2 * j + comp) * L + limb) * N, 0, sm, comp * NL, slice, lc, ar);
+    split_fwd_cross<S, 1, SP>(after_wait(ct) + ((size_t)(2 * j + comp) * L + limb) * N, 0, sm, comp * NL, slice, lc, ar);
     cluster_sync();  // this CTA's parts are complete
     uint64_t x[1][C];
 #pragma unroll
     for (int r = 0; r < C; ++r) x[0][r] = b[tid + r * T];
     fwd_rounds<Cfg, 0, S::LOGP, SP>(x, b, lc.tw_f, nullptr, ar, tid, tmul);
-    const ulonglong2 *w = reinterpret_cast<const ulonglong2 *>(pt + ((size_t)j * L + limb) * N + rank * NL + tid * C);
+    const ulonglong2 *w =
+        reinterpret_cast<const ulonglong2 *>(after_wait(pt + ((size_t)j * L + limb) * N + rank * NL + tid * C));
 #pragma unroll
     for (int r = 0; r < C; r += 2) {
         const ulonglong2 a = ld_data(w + r / 2);
