@@ -109,7 +109,9 @@ hc_status hc_selftest_wait_timeout(const hc_ctx *ctx, uint32_t limit, void *cuda
  * prefetching into their exchange buffer above); variant 1 of the forward
  * kinds at N >= 8192 transforms each limb with a cluster of two CTAs.  In the
  * default variants of kinds 0, 1, 3, 4 and 5, launches of few limbs run each
- * limb split over a cluster of eight CTAs.  For kind 6 variants 0..2 select the weight rows per pipeline
+ * limb split over a cluster of eight CTAs, and contexts with a modulus that is
+ * not 2^50 - c, c < 2^22, take other shapes in those of kinds 0, 2, 3 and 4 at
+ * sizes where these are quicker.  For kind 6 variants 0..2 select the weight rows per pipeline
  * stage (about 16, 32 or 64; of layers with one or two spatial blocks, which do
  * not stage their weights, the CTAs per SM) of the integer MAC, and variant 3 the tensor-core MAC
  * (residues split into 8-bit limbs, exact f16 products summed in fp32 by

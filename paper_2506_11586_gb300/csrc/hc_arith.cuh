@@ -141,11 +141,9 @@ struct TwArith<false> {
     // canonical y / 2^LOGN, wn = 2^-LOGN
     template <int LOGN>
     __device__ __forceinline__ uint64_t div_canon(uint64_t y, ulonglong2 wn) const { return mul_canon(y, wn); }
-    // x - y for y <= b (b = 0: y is a product)
-    __device__ __forceinline__ uint64_t sub(uint64_t x, uint64_t y, uint64_t b = 0) const
-    {
-        return x - y + (b ? b : 4 * q);
-    }
+    // x - y for a product y, and for y <= b
+    __device__ __forceinline__ uint64_t sub(uint64_t x, uint64_t y) const { return x - y + 4 * q; }
+    __device__ __forceinline__ uint64_t sub(uint64_t x, uint64_t y, uint64_t b) const { return x - y + b; }
     // canonical residue of any x < 2^64
     __device__ __forceinline__ uint64_t canon(uint64_t x) const { return canon3(reduce_lazy(x, ones, nq), q); }
 };

@@ -874,31 +874,58 @@ hc_status run_product(const hc_ctx *ctx, const uint64_t *ct, const uint64_t *pt_
 
 }  // namespace detail
 
-// Transforms of so few polynomials that clusters of eight CTAs leave SMs idle run split
-// over such clusters, in the launch shapes a context starts with.
-template <int LOGN, bool SP>
-bool try_ntt_split(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaStream_t s, hc_status *st)
+// f(segments counted in polynomials, their number of limbs) of a transform launch
+template <class F>
+hc_status with_polys(const hc_ctx *ctx, int kind, const LaunchArgs &a, F &&f)
 {
-    using S = SplitShape<LOGN, 3, 1, 1>;
-    const bool inverse = kind == KK_INV || kind == KK_INVCT || kind == KK_INVCT_SEGS;
-    auto few = [&](uint64_t units) { return units > 0 && units <= split_units_ntt(LOGN, ctx->sms); };
     if (kind == KK_FWDCT_SEGS || kind == KK_INVCT_SEGS) {
         NttSegs segs = *a.segs;
         uint64_t total = 0;
         for (uint32_t i = 0; i < segs.n; ++i) {
-            segs.s[i].n_groups *= 2;  // polynomials
+            segs.s[i].n_groups *= 2;
             segs.s[i].cta_begin = (uint32_t)total;
             total += (uint64_t)segs.s[i].n_groups * seg_limbs(segs.s[i]);
         }
-        if (!few(total)) return false;
-        *st = detail::run_ntt_split<S, SP>(segs, (uint32_t)total, inverse, s);
-        return true;
+        return f(segs, total);
     }
-    if (kind != KK_FWD && kind != KK_INV && kind != KK_FWDCT && kind != KK_INVCT) return false;
     const size_t polys = kind == KK_FWD || kind == KK_INV ? a.n : 2 * a.n;
-    if (polys > 0x7fffffffu / kMaxLimbs || !few((uint64_t)polys * ctx->L)) return false;
-    *st = detail::run_ntt_split<S, SP>(detail::one_seg(ctx, a.in, a.out, polys), (uint32_t)(polys * ctx->L), inverse, s);
-    return true;
+    if (polys * ctx->L > 0x7fffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
+    return f(detail::one_seg(ctx, a.in, a.out, polys), (uint64_t)polys * ctx->L);
+}
+
+// Transforms in the shapes a context starts with, where those of its default variants are not
+// the quickest; *taken: launched here.
+//   Split over clusters: so few limbs that clusters of eight CTAs leave SMs idle.
+//   Shoup products take a fifth longer than folded ones, so that one wave of a shape with many
+//   CTAs an SM can cost more than two of a quicker one.  Measured on GB300, us, the default
+//   variant's shape / here / the library's before there were folded products:
+//     forward  N = 4096:  153 limbs 15.3 / 11.6 / 14.4   280: 16.4 / 11.7 / 14.4  (340: 16.7 / - / 20)
+//              N = 8192:  133 limbs 17.5 (split) / 12.6 / 16.5   153: 25.1 / 19.3 / 20.5
+//                         305: 35.3 / 29.7 / 31.3   608: 45.8 / 45.8 / 49.2   1216: 88.9 / 88.6 / 93.4
+//   and, in launch_variant,
+//     products N = 4096:  114 limbs 28.2 / 25.5 / 25.5   300: 49.9 / 46.2 / 46.1  (228: 38 / - / 46)
+//              N = 8192:  160 limbs 91 / 84 / 90   456: 142 / 143 / 153   600: 196 / 192 / 189
+//     sums     N = 4096:  16 of 16 terms 36.8 / 26.2 / 36.6   N = 8192: 76 of 4 terms 46 / 42 / 41
+//   Elsewhere, at N = 16384 and inverse, the default variants' shapes are the quickest.
+template <int LOGN, bool SP, class Segs>
+hc_status launch_few(const Segs &segs, uint64_t limbs, bool inverse, uint32_t sms, cudaStream_t s, bool *taken)
+{
+    using S = SplitShape<LOGN, 3, 1, 1>;
+    const bool shoup = !SP && !inverse;
+    *taken = limbs > 0;
+    if (limbs <= (shoup && LOGN == 13 ? sms * 3 / 4 : split_units_ntt(LOGN, sms)))
+        return *taken ? detail::run_ntt_split<S, SP>(segs, (uint32_t)limbs, inverse, s) : HC_OK;
+    if constexpr (!SP && LOGN == 12)
+        if (shoup && limbs <= 2 * sms)  // C = 8, one wave of two CTAs an SM
+            return detail::run_ntt_segs<VCfg<LOGN, 2, true>, SP, KK_FWD>(segs, sms, s, false);
+    if constexpr (!SP && LOGN == 13) {
+        if (shoup && limbs <= sms)  // C = 16, one wave of one CTA an SM
+            return detail::run_ntt_segs<VCfg<LOGN, 0, true>, SP, KK_FWD>(segs, sms, s, false);
+        if (shoup && limbs <= 0x3fffffffu)
+            return detail::run_ntt_fwd_pair<typename FwdPair<LOGN>::Cfg, SP>(segs, s);
+    }
+    *taken = false;
+    return HC_OK;
 }
 
 // Inverse transforms at N >= 8192 whose input lies on an odd word, in any variant: the
@@ -906,19 +933,9 @@ bool try_ntt_split(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaStream_
 template <int LOGN, bool SP>
 hc_status launch_inv_odd(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaStream_t s)
 {
-    if (kind == KK_INVCT_SEGS) {
-        NttSegs segs = *a.segs;
-        uint32_t begin = 0;
-        for (uint32_t i = 0; i < segs.n; ++i) {
-            segs.s[i].n_groups *= 2;  // polynomials
-            segs.s[i].cta_begin = begin;
-            begin += segs.s[i].n_groups * seg_limbs(segs.s[i]);
-        }
+    return with_polys(ctx, kind, a, [&](const auto &segs, uint64_t) {
         return detail::run_ntt_inv_pf<typename InvPf<LOGN>::Cfg, SP>(segs, s);
-    }
-    const size_t polys = kind == KK_INV ? a.n : 2 * a.n;
-    if (polys * ctx->L > 0x7fffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
-    return detail::run_ntt_inv_pf<typename InvPf<LOGN>::Cfg, SP>(detail::one_seg(ctx, a.in, a.out, polys), s);
+    });
 }
 
 template <int LOGN, int V, bool SP>
@@ -927,9 +944,13 @@ hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaS
     using Fused = VCfg<LOGN, V, false>;
     using Single = VCfg<LOGN, V, true>;
     const int base = kind == KK_FWDCT_SEGS ? KK_FWDCT : kind == KK_INVCT_SEGS ? KK_INVCT : kind;
-    if (V == default_variant(base, LOGN)) {
-        hc_status st = HC_OK;
-        if (try_ntt_split<LOGN, SP>(ctx, kind, a, s, &st)) return st;
+    const bool inverse = base == KK_INV || base == KK_INVCT;
+    if (V == default_variant(base, LOGN) && (inverse || base == KK_FWD || base == KK_FWDCT)) {
+        bool taken = false;
+        const hc_status st = with_polys(ctx, kind, a, [&](const auto &segs, uint64_t limbs) {
+            return launch_few<LOGN, SP>(segs, limbs, inverse, ctx->sms, s, &taken);
+        });
+        if (st != HC_OK || taken) return st;
     }
     if constexpr (use_inv_tma<LOGN, V> || use_inv_pf<LOGN, V>) {
         auto run = [&](const auto &segs) {
@@ -992,8 +1013,23 @@ hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaS
         return kind == KK_FWDCT_SEGS ? detail::run_ntt_segs<Fused, SP, KK_FWDCT>(segs, ctx->sms, s, false)
                                      : detail::run_ntt_segs<Fused, SP, KK_INVCT>(segs, ctx->sms, s, true);
     }
-    case KK_MAC: return detail::run_mac_intt<Fused, SP>(ctx, a.in, a.pt, a.terms, a.out, a.n, s);
-    case KK_PROD: return detail::run_product<Fused, SP>(ctx, a.in, a.pt, a.out_index, a.out, a.n, a.accumulate, s);
+    case KK_MAC:
+        // by Shoup products (figures at launch_few)
+        if constexpr (!SP && LOGN == 12 && V == 0)
+            return detail::run_mac_intt<VCfg<LOGN, 2, false>, SP>(ctx, a.in, a.pt, a.terms, a.out, a.n, s);
+        if constexpr (!SP && LOGN == 13 && V == 0)
+            if ((uint64_t)a.n * ctx->L <= 2 * ctx->sms)
+                return detail::run_mac_intt<VCfg<LOGN, 1, false>, SP>(ctx, a.in, a.pt, a.terms, a.out, a.n, s);
+        return detail::run_mac_intt<Fused, SP>(ctx, a.in, a.pt, a.terms, a.out, a.n, s);
+    case KK_PROD:
+        // by Shoup products (figures at launch_few)
+        if constexpr (!SP && LOGN < 14 && V == 0) {
+            const uint64_t limbs = (uint64_t)a.n * ctx->L, sms = ctx->sms;
+            if (LOGN == 12 ? limbs <= sms || (limbs > sms * 3 / 2 && limbs <= 3 * sms) : limbs > sms)
+                return detail::run_product<VCfg<LOGN, LOGN == 12 ? 1 : 2, false>, SP>(
+                    ctx, a.in, a.pt, a.out_index, a.out, a.n, a.accumulate, s);
+        }
+        return detail::run_product<Fused, SP>(ctx, a.in, a.pt, a.out_index, a.out, a.n, a.accumulate, s);
     case KK_PROD_SPLIT:
         if constexpr (V == 0) return detail::run_product_split<SplitShape<LOGN, 3, 2, 1, 3, LOGN == 12 ? 8 : 16>, SP>(ctx, a, s);
         return set_error(HC_ERR_INVALID_ARG, "the split product has one shape");

@@ -51,7 +51,8 @@ __global__ void k_range_check(const uint64_t *__restrict__ p, const LimbConst *_
 
 // Launch shapes a context starts with (the autotuner may change them); figures at
 // Variant in hc_kernels.cuh.  In these shapes launches of few limbs run split over
-// clusters (split_units_ntt).
+// clusters (split_units_ntt), and contexts without folded twiddles take other shapes at
+// some sizes (launch_few, launch_variant).
 int default_variant(int kind, uint32_t logn)
 {
     if (logn >= 13 && (kind == KK_FWD || kind == KK_FWDCT || kind == KK_INV || kind == KK_INVCT)) return 2;
