@@ -1006,12 +1006,17 @@ hc_status hc_conv_ct_pt_host(const hc_ctx *ctx, const hc_weights *w, const uint6
         return hc_ctx_device_status(ctx, cuda_stream);
     }
     // Pipelined: the outputs of a block of output channels (contiguous in the output
-    // and in the weights) go back to the host while the next block is computed.  The copies
-    // bound the call (188 GB/s measured to pinned memory, several times slower than the
-    // kernels), so the first blocks are small, a sixteenth of the channels, to start them
-    // early, and each later one is as large as those before it together, which hides its
-    // kernels behind their copies and keeps the copies few.  128 output ciphertexts at
-    // N = 8192, L = 3, of a 27x27 layer on GB300: 345 -> 336 us.
+    // and in the weights) go back to the host while the next block is computed.  Mostly the
+    // copies bound the call (188 GB/s measured to pinned memory), so the first blocks are
+    // small, a sixteenth of the channels, to start them early, and each later one is as large
+    // as those before it together, which hides its kernels behind their copies and keeps the
+    // copies few.  In layers of many channel groups the kernels bound it, and the last block's
+    // copy comes after all of them: hence no block above a quarter of the channels.  Measured
+    // on GB300, us, eight equal blocks / doubling to the end / so:
+    //   128 output ciphertexts, N = 8192, L = 3, 27x27, G = 4:  342 / 334 / 337
+    //   1152, N = 4096, L = 2, 27x27, G = 16, B = 9:  1045 / 1185 / 1130
+    //   256, N = 8192, L = 3, 56x56, G = 13, B = 8:   1018 / 1028 / 971
+    // At most seven blocks (kHostChunks events).
     hc_status st = check_inputs(ctx, (const uint64_t *)din.p, (size_t)2 * w->I, s);
     if (st != HC_OK) return st;
     CopyLane *lane = nullptr;
@@ -1025,7 +1030,7 @@ hc_status hc_conv_ct_pt_host(const hc_ctx *ctx, const hc_weights *w, const uint6
     const size_t LN = (size_t)ctx->L * ctx->N;
     uint32_t used = 0;
     for (uint32_t m0 = 0, m1, j = 0; m0 < w->Mp; m0 = m1, ++j) {
-        m1 = j + 1 == kHostChunks ? w->Mp : std::min(w->Mp, m0 ? 2 * m0 : std::max(1u, w->Mp / 16));
+        m1 = std::min(w->Mp, m0 + (m0 ? std::min(m0, (w->Mp + 3) / 4) : std::max(1u, w->Mp / 16)));
         const size_t o0 = (size_t)m0 * w->B, no = (size_t)(m1 - m0) * w->B;
         st = launch_mac_conv(ctx, x, w->d_pt + (size_t)m0 * w->G * LN, y + o0 * ct_words, w->G, w->B, m1 - m0, s);
         if (st == HC_OK) st = launch_ntt_inv_ct(ctx, y + o0 * ct_words, y + o0 * ct_words, no, s);
