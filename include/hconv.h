@@ -440,7 +440,7 @@ hc_status hc_galois_key_create(const hc_ctx *ctx, uint64_t special_prime, uint32
 
 /* Rotate n_ct ciphertexts d_ct_in [n][2][L][N] (coefficient domain, residues
  * < q_i) into d_ct_out (same layout, must not overlap the input).  Scratch of
- * n*(L+1)*(L+2)*N*8 bytes comes from the allocator.  Errors: HC_ERR_INVALID_ARG,
+ * n*(4*L+2)*N*8 bytes comes from the allocator.  Errors: HC_ERR_INVALID_ARG,
  * HC_ERR_RANGE (checked mode), HC_ERR_OOM, HC_ERR_CUDA. */
 hc_status hc_ct_rotate(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *d_ct_in,
                        uint64_t *d_ct_out, size_t n_ct, void *cuda_stream);
@@ -450,14 +450,14 @@ hc_status hc_ct_rotate(const hc_ctx *ctx, const hc_galois_key *key, const uint64
  *   acc = d_ct * w_{n-1};  for i = n-2 .. 0: acc = rotate(acc) + d_ct * w_i;
  * d_out [2][L][N] = acc (coefficient domain; must not overlap d_ct).  Decrypts
  * to sum_i rot^i(m * w_i) slot-wise mod P.  The n products run first, in one
- * launch; scratch of (n + 1) ciphertexts plus one rotation's comes from the
- * allocator.  Errors as hc_ct_rotate. */
+ * batch (forward transforms, sums of products, inverse transforms); scratch of
+ * (n + 1) ciphertexts plus one rotation's comes from the allocator.  Errors as hc_ct_rotate. */
 hc_status hc_mac_rotate(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *d_ct,
                         const uint64_t *d_w_ntt, uint32_t n, uint64_t *d_out, void *cuda_stream);
 
 /* The same iteration for m ciphertexts d_ct [m][2][L][N] that share the n
  * plaintexts (e.g. m client vectors through one matrix-vector layer), run in
- * lockstep: the m*n products in one launch, then n - 1 rotations of all m
+ * lockstep: the m*n products in one batch, then n - 1 rotations of all m
  * accumulators at once.  d_out [m][2][L][N] (must not overlap d_ct); scratch
  * of (m*n + m) ciphertexts plus one rotation of m.  hc_mac_rotate is m = 1.
  * Errors as hc_ct_rotate. */

@@ -80,6 +80,9 @@ k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *
         const uint64_t q = lc.q;
         auto strided = [&](uint32_t by) { return ((size_t)(cc >> 1) * by * 2 * L + (cc & 1) * L + i) * N + k; };
         auto ld2 = [](const uint64_t *p) { return ld_data(reinterpret_cast<const ulonglong2 *>(p)); };
+        auto ld_a = [&](const uint64_t *p) {  // a may be a caller's buffer, on an odd word
+            return ((uintptr_t)a & 15) == 0 ? ld2(p) : make_ulonglong2(ld_data(p), ld_data(p + 1));
+        };
         ulonglong2 v;
         if constexpr (DIVIDE) {
             const ulonglong2 ui = ld2(u + ((size_t)cc * L1 + i) * N + k), us = ld2(u + ((size_t)cc * L1 + L) * N + k);
@@ -100,15 +103,12 @@ k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *
                 v.y = div(ui.y, us.y);
             }
             if (!(cc & 1)) {
-                const ulonglong2 b = ld2(a + (size_t)r * N + k);
+                const ulonglong2 b = ld_a(a + (size_t)r * N + k);
                 v.x = csub(v.x + b.x, q);
                 v.y = csub(v.y + b.y, q);
             }
-        } else if (((uintptr_t)a & 15) == 0) {
-            v = ld2(a + strided(a_ct));
-        } else {  // the caller's input on an odd word
-            const uint64_t *p = a + strided(a_ct);
-            v = make_ulonglong2(ld_data(p), ld_data(p + 1));
+        } else {
+            v = ld_a(a + strided(a_ct));
         }
         uint64_t *o = out + (size_t)r * N;
         if (g == 1 && ((uintptr_t)out & 15) == 0) {
@@ -145,21 +145,20 @@ struct Buf {
 
 bool key_ok(const hc_galois_key *k) { return k && k->magic == kMagicGaloisKey; }
 
-// Device scratch of a chain of rotations of n ciphertexts: two permuted ciphertext buffers
-// (one read while the other is written) and the key switch's result.
+// Device scratch of the rotations of n ciphertexts: one permuted ciphertext buffer and the key
+// switch's result.
 struct RotateScratch {
     Buf mem;
-    uint64_t *a[2], *u;
+    uint64_t *a, *u;
     explicit RotateScratch(cudaStream_t s) : mem(s) {}
-    hc_status alloc(const hc_ctx *ctx, size_t n, bool chain, cudaStream_t s)
+    hc_status alloc(const hc_ctx *ctx, size_t n, cudaStream_t s)
     {
         const size_t ct = n * 2 * ctx->L * (size_t)ctx->N, ks = n * 2 * (ctx->L + 1) * (size_t)ctx->N;
         if (n * 2 * (ctx->L + 1) > 0xffffffffu) return set_error(HC_ERR_INVALID_ARG, "batch too large");
-        mem.p = dev_alloc(((chain ? 2 : 1) * ct + ks) * 8, s);
+        mem.p = dev_alloc((ct + ks) * 8, s);
         if (!mem.p) return set_error(HC_ERR_OOM, "scratch allocation failed");
-        a[0] = (uint64_t *)mem.p;
-        a[1] = chain ? a[0] + ct : nullptr;
-        u = a[0] + (chain ? 2 : 1) * ct;
+        a = (uint64_t *)mem.p;
+        u = a + ct;
         return HC_OK;
     }
 };
@@ -216,25 +215,26 @@ hc_status ks_switch(const hc_galois_key *key, const uint64_t *a, uint64_t *u, si
 }
 
 // acc = P_steps;  acc = rot_{key(i)}(acc) + P_i, i = steps-1 .. 0;  out = acc.  Ciphertext j
-// of P_i is prods[i*by_i + j*by_j]; spare: n_spare ciphertexts of memory free by now.  Each step is two launches: the key switch, then the
-// division and the addition, whose stores are already permuted for the next step.
+// of P_i is prods[i*by_i + j*by_j].  Each step is two launches: the key switch, then the
+// division and the addition, whose stores are already permuted for the next step.  The
+// accumulators a step reads lie in the scratch and in out in turn, the last step's in the
+// scratch, so that a chain needs no more memory than one rotation.
 template <class KeyAt>
 hc_status rotate_chain(const hc_ctx *ctx, const KeyAt &key_at, const uint64_t *prods, uint32_t by_i,
-                       uint32_t by_j, uint32_t steps, size_t n, uint64_t *out, uint64_t *spare,
-                       size_t n_spare, cudaStream_t s)
+                       uint32_t by_j, uint32_t steps, size_t n, uint64_t *out, cudaStream_t s)
 {
     RotateScratch sc(s);
-    hc_status st = sc.alloc(ctx, n, steps > 1 && n_spare < n, s);
+    hc_status st = sc.alloc(ctx, n, s);
     if (st != HC_OK) return st;
-    if (n_spare >= n) sc.a[1] = spare;
+    auto acc = [&](uint32_t i) { return i & 1 ? out : sc.a; };
     const size_t step = (size_t)by_i * 2 * ctx->L * ctx->N;
     const hc_galois_key *key = key_at(steps - 1);
-    st = ks_apply(ctx, key, prods + steps * step, nullptr, nullptr, sc.a[0], key->g, n, s, by_j);
-    for (uint32_t i = steps, b = 0; st == HC_OK && i-- > 0; b ^= 1) {
-        st = ks_switch(key, sc.a[b], sc.u, n, s);
+    st = ks_apply(ctx, key, prods + steps * step, nullptr, nullptr, acc(steps - 1), key->g, n, s, by_j);
+    for (uint32_t i = steps; st == HC_OK && i-- > 0;) {
+        st = ks_switch(key, acc(i), sc.u, n, s);
         if (st != HC_OK) break;
         const hc_galois_key *next = i ? key_at(i - 1) : nullptr;
-        st = ks_apply(ctx, key, sc.a[b], sc.u, prods + i * step, i ? sc.a[b ^ 1] : out, next ? next->g : 1, n, s, 1, by_j);
+        st = ks_apply(ctx, key, acc(i), sc.u, prods + i * step, i ? acc(i - 1) : out, next ? next->g : 1, n, s, 1, by_j);
         key = next;
     }
     return st;
@@ -337,10 +337,10 @@ hc_status hc_ct_rotate(const hc_ctx *ctx, const hc_galois_key *key, const uint64
     hc_status st = check_inputs(ctx, d_ct_in, 2 * n_ct, s);
     if (st != HC_OK) return st;
     RotateScratch sc(s);
-    st = sc.alloc(ctx, n_ct, false, s);
-    if (st == HC_OK) st = ks_apply(ctx, key, d_ct_in, nullptr, nullptr, sc.a[0], key->g, n_ct, s);
-    if (st == HC_OK) st = ks_switch(key, sc.a[0], sc.u, n_ct, s);
-    if (st == HC_OK) st = ks_apply(ctx, key, sc.a[0], sc.u, nullptr, d_ct_out, 1, n_ct, s);
+    st = sc.alloc(ctx, n_ct, s);
+    if (st == HC_OK) st = ks_apply(ctx, key, d_ct_in, nullptr, nullptr, sc.a, key->g, n_ct, s);
+    if (st == HC_OK) st = ks_switch(key, sc.a, sc.u, n_ct, s);
+    if (st == HC_OK) st = ks_apply(ctx, key, sc.a, sc.u, nullptr, d_ct_out, 1, n_ct, s);
     return st;
 }
 
@@ -373,7 +373,7 @@ hc_status hc_mac_rotate_many(const hc_ctx *ctx, const hc_galois_key *key, const 
     uint64_t *first = n == 1 ? d_out : prods;  // P_0 of a one-term iteration is the result
     st = products(ctx, ctn, d_w_ntt, 1, m, n, first, s);
     if (st != HC_OK || n == 1) return st;
-    return rotate_chain(ctx, [&](uint32_t) { return key; }, prods, m, 1, n - 1, m, d_out, ctn, m, s);
+    return rotate_chain(ctx, [&](uint32_t) { return key; }, prods, m, 1, n - 1, m, d_out, s);
 }
 
 hc_status hc_mac_rotate(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *d_ct, const uint64_t *d_w_ntt,
@@ -453,7 +453,7 @@ hc_status hc_zp_conv(const hc_ctx *ctx, const hc_conv_desc *desc, const hc_galoi
     if (st != HC_OK || kk == 1) return st;
     // offsets i and i + 1 lie in one kernel row unless i + 1 starts a new one
     auto key_at = [&](uint32_t i) { return (i + 1) % desc->kw == 0 ? key_row : key_1; };
-    return rotate_chain(ctx, key_at, prods, 1, kk, kk - 1, Y, d_ct_out, ctn, C, s);
+    return rotate_chain(ctx, key_at, prods, 1, kk, kk - 1, Y, d_ct_out, s);
 }
 
 }  // extern "C"
