@@ -427,6 +427,10 @@ struct LaunchArgs {
 template <int LOGN, bool SP>
 hc_status launch_n(const hc_ctx *ctx, int kind, int variant, const LaunchArgs &a, cudaStream_t s);
 
+// Meaning of the variant numbers (Variant in hc_kernels.cuh and the others that kernel kinds
+// take): counted up whenever one comes to stand for another launch shape, so that choices
+// cached by an autotuner that knew the old shapes are not applied.
+constexpr int kShapeTable = 2;
 // default launch variant of a kernel family at ring degree 2^logn
 int default_variant(int kind, uint32_t logn);
 

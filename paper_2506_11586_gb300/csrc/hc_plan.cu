@@ -269,7 +269,7 @@ std::string tune_key(const hc_ctx *c, int kind, const char *gpu, int sms, uint64
     for (char &ch : k)
         if (ch == ' ' || ch == '\t') ch = '_';
     char buf[64];
-    snprintf(buf, sizeof buf, "|sm%d|N%u|L%u", sms, c->N, c->L);
+    snprintf(buf, sizeof buf, "|shapes%d|sm%d|N%u|L%u", kShapeTable, sms, c->N, c->L);
     k += buf;
     for (uint32_t i = 0; i < c->L; ++i) {
         snprintf(buf, sizeof buf, "|%llx", (unsigned long long)c->q[i]);
