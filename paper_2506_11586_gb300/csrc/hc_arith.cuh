@@ -122,6 +122,9 @@ __device__ __forceinline__ uint64_t canon4(uint64_t x, uint64_t q)
 // sub-partition, 33.5 with unsigned values, 41.6 with Shoup products (5 wide and 4
 // narrow multiply-adds, 5 additions and moves).
 constexpr uint64_t kFoldMax = 35;
+// The most, in multiples of q, that a folded inverse stage's inputs may reach: their sums and
+// differences are below 8190 q < 2^63 - 2^50, which leaves div_canon's k c < 2^36 room.
+constexpr uint64_t kFoldStage = 4095;
 
 template <bool SP>
 struct TwArith;
@@ -194,7 +197,7 @@ struct TwArith<true> {
     {
         return canon_pos(mul(y, w, 16 * q));  // -10 * 2^50 + 16 q > 0
     }
-    // canonical y / 2^LOGN for 2^LOGN | q - 1 and |y| <= 8192 q.  Then c = -1 mod 2^LOGN, so
+    // canonical y / 2^LOGN for 2^LOGN | q - 1 and |y| <= 2 kFoldStage q.  Then c = -1 mod 2^LOGN, so
     // with k = -y mod 2^LOGN the sum y + k q = (y - k c) + 2^50 k is a multiple of 2^LOGN
     // in both terms: one wide product in place of the six of a product with N^-1.
     // |(y - k c) / 2^LOGN| <= 2^51 + 2^23 for LOGN >= 12, hence 4 q to make it positive.

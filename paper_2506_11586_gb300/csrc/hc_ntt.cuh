@@ -277,7 +277,7 @@ __device__ __forceinline__ void inv_stage(uint64_t (&x)[Cfg::NP][Cfg::C], const 
     constexpr int dist = 1 << SIG;
     constexpr int ngrp = RS::KK >> (SIG + 1);
     constexpr uint64_t bound = inv_stage_bound<Cfg, R, SIG, PART, SP>();
-    static_assert(bound <= (SP ? 4096 : 8192), "differences must fit 64 bits");
+    static_assert(bound <= (SP ? kFoldStage : 8192), "differences must fit 64 bits, and div_canon's shift");
     const uint64_t q = ar.q;
     const uint64_t qs = q * bound;    // bound of the stage's inputs
     if constexpr (s == Cfg::LOGN - 1 && PART == 0) {
