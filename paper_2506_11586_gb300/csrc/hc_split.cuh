@@ -90,6 +90,10 @@ __device__ __forceinline__ void split_inv_cross(uint64_t (&v)[NP][S::ITEMS][S::C
                                                 uint32_t slice, const LimbConst &lc, const TwArith<SP> &ar)
 {
     constexpr int LOGP = S::LOGP, CS = S::CS, ITEMS = S::ITEMS, T = S::T, NL = S::NL;
+    if constexpr (SP) {  // inputs of the last stage: sums throughout, or a product in an earlier one
+        constexpr uint64_t sums = inv_in_bound<typename S::Cfg, S::Cfg::NROUNDS, LOGP>() << (LOGP - 1);
+        static_assert(sums <= kFoldStage && (kFoldMax << LOGP) <= kFoldStage, "cross stages overflow");
+    }
     const ulonglong2 wn = make_ulonglong2(lc.ninv, lc.ninv_s), wnw = make_ulonglong2(lc.ninvw, lc.ninvw_s);
 #pragma unroll
     for (int c = 0; c < CS; ++c) {
