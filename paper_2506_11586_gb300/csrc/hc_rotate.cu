@@ -56,11 +56,12 @@ __device__ __forceinline__ uint64_t reduce_any(uint64_t v, const LimbConst &lc)
 // past N (g = 1: as it stands).  DIVIDE false: w = a, both components.  Reads are 16-byte
 // and coalesced; the permutation is on the stores, each word stored once, where gathering
 // it in the key switch would read every word L+1 times in 32-byte sectors.
-// a's ciphertexts lie a_ct ciphertexts apart, add's add_ct.
+// a's ciphertexts lie a_ct ciphertexts apart, add's add_ct.  ODD: a is a caller's buffer on an odd
+// word, read word by word (chosen on the host: a test per load takes 2 us of 15 steps' 261).
 // 2-D grid: y walks the rows (one polynomial limb each), x the N / 2 pairs of coefficients.
 constexpr uint32_t kKsBlock = 128;
 
-template <bool DIVIDE>
+template <bool DIVIDE, bool ODD>
 __global__ void __launch_bounds__(kKsBlock)
 k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *out,
            const LimbConst *__restrict__ lq, const ModDown *__restrict__ md, uint64_t special, uint32_t L, uint32_t N,
@@ -80,8 +81,8 @@ k_ks_apply(const uint64_t *a, const uint64_t *u, const uint64_t *add, uint64_t *
         const uint64_t q = lc.q;
         auto strided = [&](uint32_t by) { return ((size_t)(cc >> 1) * by * 2 * L + (cc & 1) * L + i) * N + k; };
         auto ld2 = [](const uint64_t *p) { return ld_data(reinterpret_cast<const ulonglong2 *>(p)); };
-        auto ld_a = [&](const uint64_t *p) {  // a may be a caller's buffer, on an odd word
-            return ((uintptr_t)a & 15) == 0 ? ld2(p) : make_ulonglong2(ld_data(p), ld_data(p + 1));
+        auto ld_a = [&](const uint64_t *p) {
+            return !ODD ? ld2(p) : make_ulonglong2(ld_data(p), ld_data(p + 1));
         };
         ulonglong2 v;
         if constexpr (DIVIDE) {
@@ -195,7 +196,8 @@ hc_status ks_apply(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *
     const uint32_t rows = (uint32_t)(n * 2 * ctx->L);
     ProfileScope ps("k_ks_apply", s);
     const cudaError_t e = launch_programmatic(
-        u ? k_ks_apply<true> : k_ks_apply<false>, dim3(ctx->N / 2 / kKsBlock, rows < 65535 ? rows : 65535),
+        odd_word(a) ? (u ? k_ks_apply<true, true> : k_ks_apply<false, true>)
+                    : (u ? k_ks_apply<true, false> : k_ks_apply<false, false>), dim3(ctx->N / 2 / kKsBlock, rows < 65535 ? rows : 65535),
         dim3(kKsBlock), 0, s, true, a, u, add, out, ctx->d_limbs, key->d_md, key->special, ctx->L, ctx->N, g,
         rows, a_ct, add_ct);
     return e == cudaSuccess ? HC_OK : cuda_error(e, "launch k_ks_apply");
