@@ -141,10 +141,14 @@ def alg_bytes(geo, N, L):
 
 # Integer-pipe cost model (measured on GB300 with ncu counters): the fmaheavy
 # pipe runs 64 32-bit multiply-adds per clock per SM; a 32x32->64 multiply
-# (mad.wide.u32) occupies it twice as long.  In these units a lazy Shoup
-# multiplication (5 wide + 4 narrow) costs 14, a MAC term (4 wide) 8 and the
-# final reduction of a MAC sum (one Shoup + one w=1 reduction) 19.
-IMAD_EQ_BUTTERFLY, IMAD_EQ_MAC_TERM, IMAD_EQ_REDUCE = 14, 8, 19
+# (mad.wide.u32) occupies it twice as long.  In these units, per butterfly, term
+# of a sum, reduction of a sum and slot of a standalone product:
+#   shoup   any moduli: a lazy Shoup multiplication (5 wide + 4 narrow), 4 wide, one
+#           Shoup + one w=1 reduction, and the products charged as one multiplication
+#   folded  moduli 2^50 - c, which every workload here has: 6 wide, 3 wide, 6 wide,
+#           and a sum of one term by 4 wide with 4 more to fold and reduce
+IMAD_EQ = {"shoup": (14, 8, 19, 14), "folded": (12, 6, 12, 16)}
+FORM = "folded"
 
 
 def device_sms():
@@ -184,34 +188,37 @@ def int_probe(L, ctx, stream, iters=4096):
     return out
 
 
-def kernel_work(name, geo, N, L):
+def kernel_work(name, geo, N, L, form="shoup"):
     """Algorithmic bytes and IMAD-equivalents of one launch of a kernel of the layer."""
+    butterfly, term, reduce_, _ = IMAD_EQ[form]
     logn = N.bit_length() - 1
     bfly = (N // 2) * logn
     poly = 8 * N * L
     I, P, O, prods = geo["I"], geo["P"], geo["O"], geo["products"]
-    mac = prods * 2 * L * N * IMAD_EQ_MAC_TERM + O * 2 * L * N * IMAD_EQ_REDUCE
+    mac = prods * 2 * L * N * term + O * 2 * L * N * reduce_
     if name.startswith("k_ntt_fwd"):
-        return {"bytes": 2 * poly * 2 * I, "imad_eq": 2 * I * L * bfly * IMAD_EQ_BUTTERFLY}
+        return {"bytes": 2 * poly * 2 * I, "imad_eq": 2 * I * L * bfly * butterfly}
     if name.startswith("k_ntt_inv"):
-        return {"bytes": 2 * poly * 2 * O, "imad_eq": 2 * O * L * bfly * IMAD_EQ_BUTTERFLY}
+        return {"bytes": 2 * poly * 2 * O, "imad_eq": 2 * O * L * bfly * butterfly}
     if name.startswith("k_mac_conv") or name.startswith("k_mac_tc"):
         return {"bytes": poly * (2 * I + P + 2 * O), "imad_eq": mac}
     # fused MAC + inverse NTT
-    return {"bytes": poly * (2 * I + P + 2 * O), "imad_eq": mac + 2 * O * L * bfly * IMAD_EQ_BUTTERFLY}
+    return {"bytes": poly * (2 * I + P + 2 * O), "imad_eq": mac + 2 * O * L * bfly * butterfly}
 
 
-def conv_imad_eq(I, O, products, N, L):
+def conv_imad_eq(I, O, products, N, L, form="shoup"):
     """IMAD-equivalents of one conv layer: forward NTT of 2I, MAC, inverse NTT of 2O polynomial limbs."""
+    butterfly, term, reduce_, _ = IMAD_EQ[form]
     bfly = (N // 2) * (N.bit_length() - 1)
-    return (2 * I * L * bfly * IMAD_EQ_BUTTERFLY + products * 2 * L * N * IMAD_EQ_MAC_TERM
-            + O * 2 * L * N * IMAD_EQ_REDUCE + 2 * O * L * bfly * IMAD_EQ_BUTTERFLY)
+    return (2 * I * L * bfly * butterfly + products * 2 * L * N * term
+            + O * 2 * L * N * reduce_ + 2 * O * L * bfly * butterfly)
 
 
-def product_imad_eq(N, L):
+def product_imad_eq(N, L, form="shoup"):
     """IMAD-equivalents of one standalone ct x pt product: NTT, pointwise product, INTT of 2L limbs."""
+    butterfly, _, _, slot = IMAD_EQ[form]
     bfly = (N // 2) * (N.bit_length() - 1)
-    return 2 * L * (2 * bfly * IMAD_EQ_BUTTERFLY + N * IMAD_EQ_BUTTERFLY)
+    return 2 * L * (2 * bfly * butterfly + N * slot)
 
 
 def roofline_fracs(nbytes, imad_eq, ms):
@@ -485,7 +492,7 @@ def batched_squeezenet(L, stream, reps=20, with_plain=True):
            "bit_exact_vs_per_layer": exact_layers, "bit_exact_vs_plain": exact_plain, "kernels": kern,
            "offline_weight_ntt_s": offline_s,
            "variants": {name: L.hc_ctx_get_variant(ctx, k) for name, k in KIND_NAMES.items()},
-           "roofline": roofline_fracs(nbytes, sum(conv_imad_eq(w.I, w.O, w.products, 8192, 3) for w in ws), ms)}
+           "roofline": roofline_fracs(nbytes, sum(conv_imad_eq(w.I, w.O, w.products, 8192, 3, FORM) for w in ws), ms)}
     plan.close()
     return out
 
@@ -553,7 +560,7 @@ def whole_networks(L, stream, reps=10):
                      "per_layer_ms": statistics.median(pl), "speedup_vs_per_layer": statistics.median(pl) / ms,
                      "bit_exact_vs_per_layer": exact, "offline_weight_ntt_s": offline_s, "kernels": kern,
                      "variants": {k: L.hc_ctx_get_variant(ctx, v) for k, v in KIND_NAMES.items()},
-                     "roofline": roofline_fracs(nbytes, sum(conv_imad_eq(w.I, w.O, w.products, N, nl)
+                     "roofline": roofline_fracs(nbytes, sum(conv_imad_eq(w.I, w.O, w.products, N, nl, FORM)
                                                             for w in ws), ms)}
         plan.close()
         del items, batched
@@ -608,7 +615,7 @@ def batched_uneven(L, stream, reps=20, with_plain=True):
            "speedup_vs_per_degree": statistics.median(pd) / ms,
            "speedup_vs_plain": statistics.median(pp) / ms if pp[0] is not None else None,
            "bit_exact_vs_per_degree": exact_deg, "bit_exact_vs_plain": exact_plain, "kernels": kern,
-           "roofline": roofline_fracs(nbytes, sum(n * product_imad_eq(c.N, c.L) for c, _, _, _, n in items), ms)}
+           "roofline": roofline_fracs(nbytes, sum(n * product_imad_eq(c.N, c.L, FORM) for c, _, _, _, n in items), ms)}
     plan.close()
     return out
 
@@ -684,13 +691,13 @@ def products16(L, stream, flush, reps=50):
     bfly = (N // 2) * (N.bit_length() - 1)
     ind_bytes = n * 8 * N * nl * 5
     acc_bytes = n * 8 * N * nl * 3 + 8 * N * nl * 2
-    acc_imad = (n * 2 * nl * bfly * IMAD_EQ_BUTTERFLY + n * 2 * nl * N * IMAD_EQ_MAC_TERM
-                + 2 * nl * N * IMAD_EQ_REDUCE + 2 * nl * bfly * IMAD_EQ_BUTTERFLY)
+    _, term, reduce_, _ = IMAD_EQ["shoup"]  # these sums take four wide products a term in either form
+    acc_imad = (n + 1) * 2 * nl * bfly * IMAD_EQ[FORM][0] + 2 * nl * N * (n * term + reduce_)
     mi, ma, mp = statistics.median(ti), statistics.median(ta), statistics.median(tp)
     res = {"workload": "ctpt_16_products_N4096_L2", "products": n,
            "independent": {"ms": mi, "p99_ms": sorted(ti)[int(0.99 * (len(ti) - 1))], "value": n / (mi / 1e3),
                            "unit": UNIT, "alg_bytes": ind_bytes,
-                           "roofline": roofline_fracs(ind_bytes, n * product_imad_eq(N, nl), mi),
+                           "roofline": roofline_fracs(ind_bytes, n * product_imad_eq(N, nl, FORM), mi),
                            "kernels": _kernel_trace(L, fi, "products16_independent")},
            "accumulated": {"ms": ma, "p99_ms": sorted(ta)[int(0.99 * (len(ta) - 1))], "value": n / (ma / 1e3),
                            "unit": UNIT, "alg_bytes": acc_bytes, "roofline": roofline_fracs(acc_bytes, acc_imad, ma),
@@ -772,10 +779,11 @@ def zp_rotations(L, stream, reps=20):
 def zp_rotation_imad_eq(N, nl):
     """IMAD-equivalents of one key-switched rotation of one ciphertext: forward NTT of the
     L digits over L+1 moduli, the digit-key MAC, inverse NTT of 2(L+1) limbs, mod-down."""
+    butterfly = IMAD_EQ[FORM][0]
     bfly = (N // 2) * (N.bit_length() - 1)
-    return ((nl * (nl + 1) + 2 * (nl + 1)) * bfly * IMAD_EQ_BUTTERFLY
-            + nl * 2 * (nl + 1) * N * IMAD_EQ_MAC_TERM + 2 * (nl + 1) * N * IMAD_EQ_REDUCE
-            + 2 * nl * N * IMAD_EQ_BUTTERFLY)
+    # sums of 4 wide products a term, reduced by 3; the division by p_sp is a Shoup product
+    return ((nl * (nl + 1) + 2 * (nl + 1)) * bfly * butterfly
+            + nl * 2 * (nl + 1) * N * 8 + 2 * (nl + 1) * N * 6 + 2 * nl * N * IMAD_EQ["shoup"][0])
 
 
 def zp_conv_section(L, stream, ctx, ctx_p, key_1, s, moduli, special, reps):
@@ -814,9 +822,7 @@ def zp_conv_section(L, stream, ctx, ctx_p, key_1, s, moduli, special, reps):
     poly = 8 * N * nl
     rot = Y * (kk - 1)
     nbytes = (poly * (2 * C_ + n_plain + 2 * Y) + (kk - 1) * (poly * 2 * Y * 3 + 8 * N * nl * 2 * (nl + 1)))
-    imad = (2 * C_ * nl * bfly * IMAD_EQ_BUTTERFLY + n_plain * 2 * nl * N * IMAD_EQ_MAC_TERM
-            + kk * Y * 2 * nl * N * IMAD_EQ_REDUCE + kk * Y * 2 * nl * bfly * IMAD_EQ_BUTTERFLY
-            + rot * zp_rotation_imad_eq(N, nl))
+    imad = conv_imad_eq(C_, kk * Y, n_plain, N, nl, FORM) + rot * zp_rotation_imad_eq(N, nl)
     res = {"workload": "zp_conv_fire2_expand3x3_16to64_55x55_N8192_L3", "products": n_plain, "rotations": rot,
            "input_cts": C_, "output_cts": Y, "ms": ms, "p99_ms": max(t), "value": n_plain / (ms / 1e3),
            "unit": UNIT, "rotations_per_s": rot / (ms / 1e3), "preprocess_s": pre_s,
@@ -967,7 +973,7 @@ def run_gb300(args):
     kname = max(rprof, key=lambda k: rprof[k][1])
     kl, kms = rprof[kname]
     k_avg_ms = kms / kl
-    work = kernel_work(kname, geo, N, nl)
+    work = kernel_work(kname, geo, N, nl, FORM)
     bytes_layer = alg_bytes(geo, N, nl)
     hbm_peak, peak_kind = measured_peaks()
     alu_peak = alu_peak_imad_eq()
