@@ -131,7 +131,6 @@ struct TwArith;
 
 template <>
 struct TwArith<false> {
-    static constexpr bool kFolded = false;
     uint64_t q, nq;
     uint32_t ones;  // floor(2^64 / q)
     __device__ __forceinline__ TwArith(uint64_t q_, uint64_t, uint64_t one_s)
@@ -153,7 +152,6 @@ struct TwArith<false> {
 
 template <>
 struct TwArith<true> {
-    static constexpr bool kFolded = true;
     uint64_t q;
     uint32_t c, c4, p20;
     __device__ __forceinline__ TwArith(uint64_t q_, uint64_t c_, uint64_t)
@@ -270,19 +268,6 @@ __device__ __forceinline__ void mac_add(MacAcc &a, uint64_t x, uint64_t w)
         "}"
         : "+l"(a.s0), "+l"(a.s1), "+l"(a.s2), "+r"(a.c0)
         : "l"(x), "l"(w));
-}
-
-// a += b (same representation; the s0 carry is counted in c0)
-__device__ __forceinline__ void mac_merge(MacAcc &a, const MacAcc &b)
-{
-    asm("{\n\t"
-        "add.cc.u64 %0, %0, %4;\n\t"
-        "addc.u32 %3, %3, %7;\n\t"
-        "add.u64 %1, %1, %5;\n\t"
-        "add.u64 %2, %2, %6;\n\t"
-        "}"
-        : "+l"(a.s0), "+l"(a.s1), "+l"(a.s2), "+r"(a.c0)
-        : "l"(b.s0), "l"(b.s1), "l"(b.s2), "r"(b.c0));
 }
 
 // V = lo + 2^64 hi of an accumulator: lo = s0 + 2^32 lo32(s1), hi = c0 + s2 + hi32(s1) + carry

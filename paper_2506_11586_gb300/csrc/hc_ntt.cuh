@@ -93,32 +93,10 @@ struct RoundShape {
     static constexpr int SUBS = Cfg::C >> K;  // sub-transforms per thread
 };
 
-// ---- element owned by (thread, register slot r) in each round ----------------
+// ---- element owned by (thread, register slot r = v*KK + j) in each round ------------
+// As base (of the thread) plus offset (constant after unrolling), for spos_at.
 // forward round: sub-transform u = tid*SUBS + v covers, at stride S = N >> (S0+K),
 // the KK elements (u / S) * (N >> S0) + (u % S) + j*S.
-template <class Cfg, int R>
-__device__ __forceinline__ int fwd_elem(int tid, int r)
-{
-    using RS = RoundShape<Cfg, R>;
-    constexpr int S = Cfg::N >> (RS::S0 + RS::K);
-    const int v = r >> RS::K, j = r & (RS::KK - 1);
-    const int u = tid * RS::SUBS + v;
-    return (u / S) * (Cfg::N >> RS::S0) + (u % S) + j * S;
-}
-
-// inverse round: sub-transform u = tid + v*T covers, at stride S = 2^S0, the KK
-// elements (u / S) * (S << K) + (u % S) + j*S.
-template <class Cfg, int R>
-__device__ __forceinline__ int inv_elem(int tid, int r)
-{
-    using RS = RoundShape<Cfg, R>;
-    constexpr int S = 1 << RS::S0;
-    const int v = r >> RS::K, j = r & (RS::KK - 1);
-    const int u = tid + v * Cfg::T;
-    return (u / S) * (S << RS::K) + (u % S) + j * S;
-}
-
-// the same as base (of the thread) and offset (constant after unrolling), for spos_at
 template <class Cfg, int R>
 __device__ __forceinline__ int fwd_base(int tid)
 {
@@ -134,6 +112,8 @@ __device__ __forceinline__ int fwd_off(int r)
     constexpr int S = Cfg::N >> (RS::S0 + RS::K);
     return S == 1 ? r : r * S;
 }
+// inverse round: sub-transform u = tid + v*T covers, at stride S = 2^S0, the KK
+// elements (u / S) * (S << K) + (u % S) + j*S.
 template <class Cfg, int R>
 __device__ __forceinline__ int inv_base(int tid)
 {
@@ -353,7 +333,7 @@ __device__ __forceinline__ void inv_round(uint64_t (&x)[Cfg::NP][Cfg::C], const 
 // per thread and C^R <= 32 -- rounds 0 and 1 for every shape here.  Forward
 // round R (stride N >> (RC + K) over blocks of N >> RC): local iff
 // log2 N - R log2 C <= 5 + log2 C -- the last two rounds (three for some
-// shapes).  Checked for every shape on a CPU model of fwd_elem / inv_elem.
+// shapes).  Checked for every shape on a CPU model of these layouts.
 #ifndef HC_WARP_LOCAL_XCHG
 #define HC_WARP_LOCAL_XCHG 1
 #endif
@@ -457,7 +437,7 @@ struct NoHook {
 
 // inverse: x holds element tid*C + r (contiguous) on entry, canonical values
 // < q; on exit the last-round layout (element tid + r'*T for the slot order of
-// inv_elem), canonical.  The first exchange synchronises the warp only: since
+// inv_base, inv_off), canonical.  The first exchange synchronises the warp only: since
 // the caller's last CTA barrier, no thread may have accessed shared memory
 // outside its own warp's block of 32*C elements (every caller's last accesses
 // are its reads of the round-0 layout, element tid*C + r).  hook() runs (in every thread) right before the last
