@@ -111,9 +111,10 @@ hc_status hc_selftest_wait_timeout(const hc_ctx *ctx, uint32_t limit, void *cuda
  * default variants of kinds 0, 1, 3, 4 and 5, launches of few limbs run each
  * limb split over a cluster of eight CTAs, and contexts with a modulus that is
  * not 2^50 - c, c < 2^22, take other shapes in those of kinds 0, 2, 3 and 4 at
- * sizes where these are quicker.  For kind 6 variants 0..2 select the weight rows per pipeline
- * stage (about 16, 32 or 64; of layers with one or two spatial blocks, which do
- * not stage their weights, the CTAs per SM) of the integer MAC, and variant 3 the tensor-core MAC
+ * sizes where these are quicker.  For kind 6 variants 0..2 select the weight
+ * rows per pipeline stage (about 16, 32 or 64) of the integer MAC, or in layers
+ * that do not stage their weights (G channel groups by B spatial blocks of at
+ * most 50) the waves of CTAs (4, 2 or 8), and variant 3 the tensor-core MAC
  * (residues split into 8-bit limbs, exact f16 products summed in fp32 by
  * tcgen05 MMAs, recombined and reduced mod q; layers with G <= 8 channel groups
  * and 2B <= 8 rows per group, the others keep the integer MAC with 32-row

@@ -51,7 +51,7 @@ template <int LOGN> struct InvTma;
 template <> struct InvTma<12> { using Cfg = NttCfg<12, 4, 1, 2>; };  // T 256, 2 x 32 KB
 template <int LOGN> struct InvPf;
 template <> struct InvPf<13> { using Cfg = NttCfg<13, 5, 1, 2>; };   // T 256, 64 KB, two CTAs per SM
-template <> struct InvPf<14> { using Cfg = NttCfg<14, 5, 1, 1>; };   // T 512, 128 KB
+template <> struct InvPf<14> { using Cfg = NttCfg<14, 5, 1, 1>; };   // T 512, 132 KB (padded)
 template <int LOGN, int V>
 constexpr bool use_inv_tma = V == 2 && LOGN == 12;
 template <int LOGN, int V>

@@ -4,7 +4,7 @@
 // Every product j computes out_j = INTT(NTT(ct_j) . pt_j) per component and
 // limb (App. C.1).  The batch is cut into units -- one limb of one product,
 // both components at N = 4096 and 8192, one component at N = 16384 -- so that
-// every unit is one 512-thread CTA's worth of work with at most 128 KB of
+// every unit is one 512-thread CTA's worth of work with at most 132 KB of
 // shared memory whatever its N.  One CTA per SM stays resident and pulls
 // units from a global counter in the host's order (most expensive first),
 // which balances uneven units across SMs without a tail of idle SMs per
@@ -16,7 +16,7 @@ namespace {
 
 using MixCfg12 = NttCfg<12, 3, 2, 1>;  // C 8, both components, 64 KB
 using MixCfg13 = NttCfg<13, 4, 2, 1>;  // C 16, both components, 128 KB
-using MixCfg14 = NttCfg<14, 5, 1, 1>;  // C 32, one component, 128 KB
+using MixCfg14 = NttCfg<14, 5, 1, 1>;  // C 32, one component, 132 KB (padded)
 constexpr int kMixThreads = 512;
 static_assert(MixCfg12::T == kMixThreads && MixCfg13::T == kMixThreads && MixCfg14::T == kMixThreads,
               "mixed-degree units share one CTA shape");

@@ -197,9 +197,9 @@ hc_status ks_apply(const hc_ctx *ctx, const hc_galois_key *key, const uint64_t *
     ProfileScope ps("k_ks_apply", s);
     const cudaError_t e = launch_programmatic(
         odd_word(a) ? (u ? k_ks_apply<true, true> : k_ks_apply<false, true>)
-                    : (u ? k_ks_apply<true, false> : k_ks_apply<false, false>), dim3(ctx->N / 2 / kKsBlock, rows < 65535 ? rows : 65535),
-        dim3(kKsBlock), 0, s, true, a, u, add, out, ctx->d_limbs, key->d_md, key->special, ctx->L, ctx->N, g,
-        rows, a_ct, add_ct);
+                    : (u ? k_ks_apply<true, false> : k_ks_apply<false, false>),
+        dim3(ctx->N / 2 / kKsBlock, rows < 65535 ? rows : 65535), dim3(kKsBlock), 0, s, true, a, u, add, out,
+        ctx->d_limbs, key->d_md, key->special, ctx->L, ctx->N, g, rows, a_ct, add_ct);
     return e == cudaSuccess ? HC_OK : cuda_error(e, "launch k_ks_apply");
 }
 
