@@ -579,10 +579,10 @@ __device__ __forceinline__ void product_task(uint64_t *sm, const uint64_t *ct, c
     }
     const TwArith<SP> ar = tw_arith<SP>(lc);
     fwd_transform<Cfg>(x, sm, lc, ar, tid);  // lazy values, contiguous layout
-    const ulonglong2 *wp = reinterpret_cast<const ulonglong2 *>(pt + (size_t)limb * N + tid * C);
+    const ulonglong2 *wp = reinterpret_cast<const ulonglong2 *>(after_wait(pt) + (size_t)limb * N + tid * C);
 #pragma unroll
     for (int r = 0; r < C / 2; ++r) {
-        const ulonglong2 w = ld_near(wp + r);
+        const ulonglong2 w = ld_data(wp + r);
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
             x[p][2 * r] = mul_slot(ar, x[p][2 * r], w.x, lc.r64, lc.r64_s);
