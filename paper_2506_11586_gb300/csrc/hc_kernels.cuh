@@ -901,10 +901,13 @@ hc_status with_polys(const hc_ctx *ctx, int kind, const LaunchArgs &a, F &&f)
 //   variant's shape / here / the library's before there were folded products:
 //     forward  N = 4096:  153 limbs 15.3 / 11.6 / 14.4   280: 16.4 / 11.7 / 14.4  (340: 16.7 / - / 20)
 //              N = 8192:  133 limbs 17.5 (split) / 12.6 / 16.5   153: 25.1 / 19.3 / 20.5
-//                         305: 35.3 / 29.7 / 31.3   608: 45.8 / 45.8 / 49.2   1216: 88.9 / 88.6 / 93.4
+//                         229 to 304, one wave: 24.6 / - / 28.6   305: 35.3 / 29.7 / 31.3
+//                         608: 45.7 / 47.2 / 49.2, but before another kernel 57 / 53 / 53
 //   and, in launch_variant,
-//     products N = 4096:  114 limbs 28.2 / 25.5 / 25.5   300: 49.9 / 46.2 / 46.1  (228: 38 / - / 46)
-//              N = 8192:  160 limbs 91 / 84 / 90   456: 142 / 143 / 153   600: 196 / 192 / 189
+//     products N = 4096:  114 limbs 28.2 / 25.5 / 25.5   300: 49.9 / 46.2 / 46.1  (76: 22 / - / 25,
+//                         228: 38 / - / 46)
+//              N = 8192:  228 limbs 91 / 88 / 91   400: 155 / 143 / 153   1000: 331 / 321 / 329; where
+//                         the last of one-CTA waves is full: 300: 98 / (100) / 96   600: 190 / (197) / 187
 //     sums     N = 4096:  16 of 16 terms 36.8 / 26.2 / 36.6   N = 8192: 76 of 4 terms 46 / 42 / 41
 //   Elsewhere, at N = 16384 and inverse, the default variants' shapes are the quickest.
 template <int LOGN, bool SP, class Segs>
@@ -921,7 +924,7 @@ hc_status launch_few(const Segs &segs, uint64_t limbs, bool inverse, uint32_t sm
     if constexpr (!SP && LOGN == 13) {
         if (shoup && limbs <= sms)  // C = 16, one wave of one CTA an SM
             return detail::run_ntt_segs<VCfg<LOGN, 0, true>, SP, KK_FWD>(segs, sms, s, false);
-        if (shoup && limbs <= 0x3fffffffu)
+        if (shoup && limbs <= 0x3fffffffu && !(limbs > sms * 3 / 2 && limbs <= 2 * sms))
             return detail::run_ntt_fwd_pair<typename FwdPair<LOGN>::Cfg, SP>(segs, s);
     }
     *taken = false;
@@ -1025,7 +1028,8 @@ hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaS
         // by Shoup products (figures at launch_few)
         if constexpr (!SP && LOGN < 14 && V == 0) {
             const uint64_t limbs = (uint64_t)a.n * ctx->L, sms = ctx->sms;
-            if (LOGN == 12 ? limbs <= sms || (limbs > sms * 3 / 2 && limbs <= 3 * sms) : limbs > sms)
+            if (LOGN == 12 ? (limbs > sms / 2 && limbs <= sms) || (limbs > sms * 3 / 2 && limbs <= 3 * sms)
+                           : limbs > sms && limbs % sms && limbs % sms <= sms * 3 / 4)
                 return detail::run_product<VCfg<LOGN, LOGN == 12 ? 1 : 2, false>, SP>(
                     ctx, a.in, a.pt, a.out_index, a.out, a.n, a.accumulate, s);
         }

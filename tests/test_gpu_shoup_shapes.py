@@ -39,7 +39,7 @@ def _residues(seed, moduli, before, N):
 @pytest.mark.parametrize("N", [4096, 8192, 16384])
 def test_forward(L, N, moduli):
     nl, sms = len(moduli), _sms()
-    lines = {4096: (sms * 7 // 8, sms, 2 * sms), 8192: (sms * 3 // 4, sms, 3 * sms // 2), 16384: (sms // 2, sms)}[N]
+    lines = {4096: (sms * 7 // 8, sms, 2 * sms), 8192: (sms * 3 // 4, sms, 3 * sms // 2, 2 * sms), 16384: (sms // 2, sms)}[N]
     ctx, one = (L.hc_ctx_create(N, moduli, T_PLAIN) for _ in range(2))
     for kind in (L.KIND_NTT_FWD, L.KIND_NTT_INV):
         L.hc_ctx_set_variant(one, kind, EXPLICIT[N])
@@ -56,7 +56,8 @@ def test_forward(L, N, moduli):
 @pytest.mark.parametrize("N", [4096, 8192])
 def test_products_and_sums(L, N):
     moduli, sms = (P45,), _sms()
-    for n in (1, sms // 2 + 1, sms, sms + 1, 3 * sms // 2 + 1, 2 * sms + 1, 3 * sms, 3 * sms + 1):
+    lines = {4096: (sms // 2, sms, 3 * sms // 2, 3 * sms), 8192: (sms, 7 * sms // 4, 2 * sms)}[N]
+    for n in [1] + [x + d for x in lines for d in (0, 1)]:
         ct, pt = to_dev(_residues(42, moduli, (n, 2), N)), to_dev(_residues(43, moduli, (n,), N))
         slots = (np.arange(n) * 7 + 3) % n if n % 7 else np.arange(n)[::-1]
         got = []
