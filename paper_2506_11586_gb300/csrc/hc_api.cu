@@ -1010,13 +1010,15 @@ hc_status hc_conv_ct_pt_host(const hc_ctx *ctx, const hc_weights *w, const uint6
     // copies bound the call (188 GB/s measured to pinned memory), so the first blocks are
     // small, a sixteenth of the channels, to start them early, and each later one is as large
     // as those before it together, which hides its kernels behind their copies and keeps the
-    // copies few.  In layers of many channel groups the kernels bound it, and the last block's
-    // copy comes after all of them: hence no block above a quarter of the channels.  Measured
-    // on GB300, us, eight equal blocks / doubling to the end / so:
+    // copies few.  In layers of many channel groups and blocks, whose MAC does not stream its
+    // weights, the kernels bound it, and the last block's copy comes after all of them: there
+    // no block is above a quarter of the channels.  Measured on GB300, us, eight equal blocks /
+    // doubling to the end / doubling up to a quarter:
     //   128 output ciphertexts, N = 8192, L = 3, 27x27, G = 4:  342 / 334 / 337
     //   1152, N = 4096, L = 2, 27x27, G = 16, B = 9:  1045 / 1185 / 1130
     //   256, N = 8192, L = 3, 56x56, G = 13, B = 8:   1018 / 1028 / 971
-    // At most seven blocks (kHostChunks events).
+    // streamed layers: between even and 0.8 % for doubling; nine channels, G = 13, B = 5:
+    // 212 / 167 / 176.  At most seven blocks (kHostChunks events).
     hc_status st = check_inputs(ctx, (const uint64_t *)din.p, (size_t)2 * w->I, s);
     if (st != HC_OK) return st;
     CopyLane *lane = nullptr;
@@ -1029,8 +1031,9 @@ hc_status hc_conv_ct_pt_host(const hc_ctx *ctx, const hc_weights *w, const uint6
     if (st != HC_OK) return st;
     const size_t LN = (size_t)ctx->L * ctx->N;
     uint32_t used = 0;
+    const uint32_t most = w->Mp < 16 || mac_streams(w->G, w->B) ? w->Mp : (w->Mp + 3) / 4;
     for (uint32_t m0 = 0, m1, j = 0; m0 < w->Mp; m0 = m1, ++j) {
-        m1 = std::min(w->Mp, m0 + (m0 ? std::min(m0, (w->Mp + 3) / 4) : std::max(1u, w->Mp / 16)));
+        m1 = std::min(w->Mp, m0 + (m0 ? std::min(m0, most) : std::max(1u, w->Mp / 16)));
         const size_t o0 = (size_t)m0 * w->B, no = (size_t)(m1 - m0) * w->B;
         st = launch_mac_conv(ctx, x, w->d_pt + (size_t)m0 * w->G * LN, y + o0 * ct_words, w->G, w->B, m1 - m0, s);
         if (st == HC_OK) st = launch_ntt_inv_ct(ctx, y + o0 * ct_words, y + o0 * ct_words, no, s);

@@ -316,6 +316,8 @@ hc_status launch_mac_tc(const hc_ctx *ctx, const uint64_t *x, const uint64_t *w,
 MacSeg make_mac_seg(const hc_ctx *ctx, const uint64_t *x, const uint64_t *w, uint64_t *y, uint32_t G, uint32_t B,
                     uint32_t M, bool ring = false, uint32_t waves = 4);
 size_t mac_seg_smem(const MacSeg &sg);
+// the blocked MAC of such a layer streams its weights (its ring stays for larger input chunks)
+bool mac_streams(uint32_t G, uint32_t B);
 // blocked MACs of n layers (layer i on ctxs[i]) in ceil(n / kMaxSegs) launches
 hc_status launch_mac_conv_layers(const hc_ctx *const *ctxs, const MacLayer *layers, size_t n, cudaStream_t s);
 

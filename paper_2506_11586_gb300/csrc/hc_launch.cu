@@ -124,6 +124,8 @@ static uint32_t mac_stage_channels(uint32_t G, uint32_t B, uint32_t M, int varia
     return ms;
 }
 
+bool mac_streams(uint32_t G, uint32_t B) { return mac_smem(G, B, 0, 64) <= kMacSmemCap / 4; }
+
 // fill the launch geometry of one segment: enough CTAs for about `waves` waves of
 // the layer's full work (all L limbs).  ring: through the weight ring whatever B is.
 MacSeg make_mac_seg(const hc_ctx *ctx, const uint64_t *x, const uint64_t *w, uint64_t *y, uint32_t G, uint32_t B,
@@ -143,7 +145,7 @@ MacSeg make_mac_seg(const hc_ctx *ctx, const uint64_t *x, const uint64_t *w, uin
     sg.M = M;
     // streamed: the input chunk alone, at least four CTAs per SM
     const uint32_t skc = mac_smem(G, B, 0, 128) <= kMacSmemCap / 4 ? 128 : 64;
-    const bool stream = !ring && mac_smem(G, B, 0, skc) <= kMacSmemCap / 4;
+    const bool stream = !ring && mac_streams(G, B);
     const uint32_t kc = sg.KC = stream ? skc : kMacKC;
     sg.MS = stream ? 0 : mac_stage_channels(G, B, M, v, kc);
     const size_t smem = mac_smem(G, B, sg.MS, kc);

@@ -1,5 +1,6 @@
 """The host-buffer layer's blocks of output channels: every channel count from one block to seven
-gives the bits of the device-buffer call, with several spatial blocks and a ragged last block."""
+gives the bits of the device-buffer call, with several spatial blocks and a ragged last block, in
+layers whose MAC streams its weights (blocks double to the end) and in others (up to a quarter)."""
 import numpy as np
 import pytest
 
@@ -21,12 +22,17 @@ def L():
 
 
 @pytest.mark.parametrize("M", [1, 2, 3, 4, 5, 7, 15, 16, 17, 19, 31, 33, 64, 67])
-def test_blocks(L, M):
+@pytest.mark.parametrize("streams", [True, False])
+def test_blocks(L, M, streams):
     N, moduli = 4096, CANONICAL_PRIMES[:2]
     ctx = L.hc_ctx_create(N, moduli, T_PLAIN)
     s = Stream(85, M)
-    w = L.hc_weights_preprocess(ctx, L.make_desc(5, 30, 31, M, 3, 3, pad=1, Cw=2, Hw=18, Ww=33),
-                                s.int8(M * 45).reshape(M, 5, 3, 3))
+    if streams:      # three channel groups by two spatial blocks
+        w = L.hc_weights_preprocess(ctx, L.make_desc(5, 30, 31, M, 3, 3, pad=1, Cw=2, Hw=18, Ww=33),
+                                    s.int8(M * 45).reshape(M, 5, 3, 3))
+    else:            # eleven by five
+        w = L.hc_weights_preprocess(ctx, L.make_desc(22, 5, 6, M, 1, 1, Cw=2, Hw=1, Ww=6),
+                                    s.int8(M * 22).reshape(M, 22, 1, 1))
     ct = uniform_residues(s, moduli, (w.I, 2), N)
     ref = torch.empty(w.O * 4 * N, dtype=torch.int64, device="cuda")
     L.hc_conv_ct_pt(ctx, w, to_dev(ct), ref)
