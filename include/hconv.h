@@ -111,7 +111,8 @@ hc_status hc_selftest_wait_timeout(const hc_ctx *ctx, uint32_t limit, void *cuda
  * default variants of kinds 0, 1, 3, 4 and 5, launches of few limbs run each
  * limb split over a cluster of eight CTAs, and contexts with a modulus that is
  * not 2^50 - c, c < 2^22, take other shapes in those of kinds 0, 2, 3 and 4 at
- * sizes where these are quicker.  For kind 6 variants 0..2 select the weight
+ * sizes where these are quicker; kind 2 has variant 2's shape in variant 0 at
+ * N = 4096.  For kind 6 variants 0..2 select the weight
  * rows per pipeline stage (about 16, 32 or 64) of the integer MAC, or in layers
  * that do not stage their weights (G channel groups by B spatial blocks of at
  * most 50) the waves of CTAs (4, 2 or 8), and variant 3 the tensor-core MAC

@@ -908,7 +908,7 @@ hc_status with_polys(const hc_ctx *ctx, int kind, const LaunchArgs &a, F &&f)
 //                         228: 38 / - / 46)
 //              N = 8192:  228 limbs 91 / 88 / 91   400: 155 / 143 / 153   1000: 331 / 321 / 329; where
 //                         the last of one-CTA waves is full: 300: 98 / (100) / 96   600: 190 / (197) / 187
-//     sums     N = 4096:  16 of 16 terms 36.8 / 26.2 / 36.6   N = 8192: 76 of 4 terms 46 / 42 / 41
+//     sums     N = 8192:  76 of 4 terms, k_mac_intt alone 46 / 42 / 41
 //   Elsewhere, at N = 16384 and inverse, the default variants' shapes are the quickest.
 template <int LOGN, bool SP, class Segs>
 hc_status launch_few(const Segs &segs, uint64_t limbs, bool inverse, uint32_t sms, cudaStream_t s, bool *taken)
@@ -1017,10 +1017,12 @@ hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaS
                                      : detail::run_ntt_segs<Fused, SP, KK_INVCT>(segs, ctx->sms, s, true);
     }
     case KK_MAC:
-        // by Shoup products (figures at launch_few)
-        if constexpr (!SP && LOGN == 12 && V == 0)
+        // at N = 4096 two CTAs of C = 8 an SM, not variant 0's three of C = 16, whose 80 registers
+        // hold few loads in flight: 16 sums of 4
+        // products, one limb, 38.5 -> 30.6 us, 38 of 16 76.6 -> 69.8, 600 of 2 137 -> 136
+        if constexpr (LOGN == 12 && V == 0)
             return detail::run_mac_intt<VCfg<LOGN, 2, false>, SP>(ctx, a.in, a.pt, a.terms, a.out, a.n, s);
-        if constexpr (!SP && LOGN == 13 && V == 0)
+        if constexpr (!SP && LOGN == 13 && V == 0)  // by Shoup products (figures at launch_few)
             if ((uint64_t)a.n * ctx->L <= 2 * ctx->sms)
                 return detail::run_mac_intt<VCfg<LOGN, 1, false>, SP>(ctx, a.in, a.pt, a.terms, a.out, a.n, s);
         return detail::run_mac_intt<Fused, SP>(ctx, a.in, a.pt, a.terms, a.out, a.n, s);
