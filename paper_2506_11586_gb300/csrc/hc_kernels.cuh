@@ -1018,8 +1018,8 @@ hc_status launch_variant(const hc_ctx *ctx, int kind, const LaunchArgs &a, cudaS
     }
     case KK_MAC:
         // at N = 4096 two CTAs of C = 8 an SM, not variant 0's three of C = 16, whose 80 registers
-        // hold few loads in flight: 16 sums of 4
-        // products, one limb, 38.5 -> 30.6 us, 38 of 16 76.6 -> 69.8, 600 of 2 137 -> 136
+        // hold few loads in flight: 16 sums of 4 products, one limb, 38.5 -> 30.6 us, 38 of 16
+        // 76.6 -> 69.8, 600 of 2 137 -> 136
         if constexpr (LOGN == 12 && V == 0)
             return detail::run_mac_intt<VCfg<LOGN, 2, false>, SP>(ctx, a.in, a.pt, a.terms, a.out, a.n, s);
         if constexpr (!SP && LOGN == 13 && V == 0)  // by Shoup products (figures at launch_few)
